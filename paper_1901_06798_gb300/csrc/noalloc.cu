@@ -15,6 +15,7 @@
 // and keeps the contents of the last call; each call rewrites all of it (and
 // clears the speed accumulator) before use.  Calls whose work overlaps on the
 // GPU (different streams, or different host threads) race on it.
+#include <algorithm>
 #include <cstdint>
 #include <cstring>
 #include <mutex>
@@ -64,7 +65,7 @@ cudaError_t scratch_for_current_device(void **out)
 }
 
 __global__ void noalloc_prepare_kernel(unsigned char *scratch, long long fstride, int nx, int ny, int pitch,
-                                       double dt, int W, int nsx, int nsy)
+                                       double dt, int W, int nsx, int n)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         PatchDesc d;
@@ -83,7 +84,6 @@ __global__ void noalloc_prepare_kernel(unsigned char *scratch, long long fstride
         sm[1] = 0ull;
     }
     StepItem *items = reinterpret_cast<StepItem *>(scratch + kItemsOff);
-    const int n = nsx * nsy;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         int sx = k % nsx, sy = k / nsx;
         int x0 = sx * W, y0 = sy * kSegRows;
@@ -111,16 +111,19 @@ extern "C" int tsu_grid_step_noalloc(int precision, void *block, int nx, int ny,
     if (((uintptr_t)block) % esz) return TSU_ERR_ARG;
     const int nt = precision == TSU_F64 ? step_threads_f64() : step_threads_f32p();
     const int W = precision == TSU_F64 ? step_strip_width_f64(nt, 0) : step_strip_width_f32p(nt, 0);
-    const int nsx = (nx + W - 1) / W, nsy = (ny + kSegRows - 1) / kSegRows;
-    if ((long long)nsx * nsy > kMaxItems) return TSU_ERR_ARG;
+    // FP64: work items in the scratch; FP32: tiles found from the CTA's index
+    const int rows = precision == TSU_F64 ? kSegRows : tile_cut(ny, tile_rows_f32p(1, &nx, &ny, nt));
+    const int nsx = (nx + W - 1) / W, nsy = (ny + rows - 1) / rows;
+    const int n_items = precision == TSU_F64 ? nsx * nsy : 0;
+    if (n_items > kMaxItems) return TSU_ERR_ARG;
 
     cudaStream_t st = (cudaStream_t)cuda_stream;
     void *sp = nullptr;
     if (scratch_for_current_device(&sp) != cudaSuccess) return TSU_ERR_CUDA;
     unsigned char *scratch = reinterpret_cast<unsigned char *>(sp);
 
-    int blocks = (nsx * nsy + 255) / 256;
-    noalloc_prepare_kernel<<<blocks, 256, 0, st>>>(scratch, field_stride, nx, ny, pitch, dt, W, nsx, nsy);
+    int blocks = std::max(1, (n_items + 255) / 256);
+    noalloc_prepare_kernel<<<blocks, 256, 0, st>>>(scratch, field_stride, nx, ny, pitch, dt, W, nsx, n_items);
     if (cudaGetLastError() != cudaSuccess) return TSU_ERR_CUDA;
 
     const PatchDesc *desc = reinterpret_cast<const PatchDesc *>(scratch + kDescOff);
@@ -135,7 +138,9 @@ extern "C" int tsu_grid_step_noalloc(int precision, void *block, int nx, int ny,
 
     StepArgs a{};
     a.descs = desc;
-    a.items = reinterpret_cast<const StepItem *>(scratch + kItemsOff);
+    a.items = precision == TSU_F64 ? reinterpret_cast<const StepItem *>(scratch + kItemsOff) : nullptr;
+    a.tile_rows = rows;
+    a.tile_nsx = nsx;
     a.arena = block;
     a.cur = cur;
     a.dt1 = reinterpret_cast<const double *>(scratch + kDtOff);

@@ -1,67 +1,92 @@
 // step_f32p.cu -- FP32 surface-perturbation form of the patch update: state
 // (eta' = h + B, hu, hv) and B in FP32.  The surface jump that drives the waves
 // is formed from eta' directly, so still water is exactly still and the
-// ocean-depth cancellation of h + B never enters the flux.  Levels with a Q*
-// scratch run the split step as two kernels (step_split_f32.cuh); without one
-// (the allocation-free entry point) the fused kernel (step_f32x2.cuh).
-#include "step_split_f32.cuh"
+// ocean-depth cancellation of h + B never enters the flux.
+#include <algorithm>
+#include <cmath>
+#include "step_tile_f32.cuh"
 
 namespace tsu {
 
 static constexpr int kThreadsF32 = 128;
 
 int step_threads_f32p() { return kThreadsF32; }
-int step_strip_width_f32p(int threads, int transverse) { return transverse ? threads - 4 : 2 * threads - 4; }
+int step_strip_width_f32p(int threads, int transverse) { return transverse ? threads - 4 : kTileCols; }
 
-// threads per CTA: 32, 64, 128 or 256 (two columns per thread: strip width 2 threads - 4)
+namespace {
+
+constexpr int kSMs = 152;
+int tile_smem(int rows) { return (rows + 4) * kTileRow * (int)sizeof(float); }
+
+// CTAs of `threads` that fit on an SM: 16 warps of 128 registers, 228 KiB of
+// shared memory of which each CTA takes 1 KiB beside its tile
+int tile_ctas(int rows, int threads)
+{
+    return std::max(1, std::min(512 / threads, 228 * 1024 / (tile_smem(rows) + 1024)));
+}
+
+template <int NW, bool GEO, bool BULK> int launch_tile(const StepArgs &a, int n, cudaStream_t st)
+{
+    // above 48 KiB of dynamic shared memory a kernel has to be told so, once per device
+    static unsigned long long told = 0;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return (int)e;
+    if (dev >= 64 || !(told >> dev & 1)) {
+        e = cudaFuncSetAttribute(step_tile_f32<NW, GEO, BULK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 tile_smem(kTileRowsMax));
+        if (e != cudaSuccess) return (int)e;
+        if (dev < 64) told |= 1ull << dev;
+    }
+    step_tile_f32<NW, GEO, BULK><<<n, NW * 32, tile_smem(a.tile_rows), st>>>(a);
+    return (int)cudaGetLastError();
+}
+
+template <int NW> int launch_tile_nw(const StepArgs &a, int n, cudaStream_t st)
+{
+    const bool geo = a.kap != nullptr;
+    if (a.bulk_rows) return geo ? launch_tile<NW, true, true>(a, n, st) : launch_tile<NW, false, true>(a, n, st);
+    return geo ? launch_tile<NW, true, false>(a, n, st) : launch_tile<NW, false, false>(a, n, st);
+}
+
+}  // namespace
+
+// The tile height that the model below finds fastest.  A tile of R rows takes
+// about R + kOver row times (its ghost rows, the wait for its copies, the ramp of
+// the y march); a second to fourth CTA on an SM slows the others by kShare each
+// (they share the issue slots that one leaves free); tiles come in waves of as
+// many CTAs as fit.
+int tile_rows_f32p(int n, const int *nx, const int *ny, int threads)
+{
+    static const int cand[] = {4, 6, 8, 10, 12, 16, 20, 24, 30, 36, 44, 60};
+    constexpr double kOver = 10.0, kShare = 0.2;
+    int best = 44;
+    double bc = 1e300;
+    for (int R : cand) {
+        double items = 0.0;
+        for (int k = 0; k < n; k++) items += (double)((nx[k] + kTileCols - 1) / kTileCols) * ((ny[k] + R - 1) / R);
+        const int occ = tile_ctas(R, threads);
+        const double per = items / kSMs, full = std::floor(per / occ), rest = std::ceil(per - full * occ - 1e-9);
+        const double one = R + kOver;
+        const double c = full * one * (1.0 + kShare * (occ - 1)) + (rest > 0 ? one * (1.0 + kShare * (rest - 1)) : 0.0);
+        if (c < bc) { bc = c; best = R; }
+    }
+    return best;
+}
+
+// threads per CTA: 32, 64, 128 or 256
 int launch_step_f32p(const StepArgs &a, int n_items, int threads, cudaStream_t st)
 {
     if (n_items <= 0) return 0;
     if (a.transverse) return launch_unsplit_f32p(a, n_items, threads, st);
-    if (a.scratch != nullptr) {
-        // x sweep over a.items (strips of 2 threads - 4 columns), then y sweep over a.items_y
-        const bool geo = a.kap != nullptr;
-        if (a.bulk_rows) {   // rows by bulk copies on mbarriers (Cartesian and latitude-longitude)
-            switch (threads) {
-            case 32: geo ? step_x_f32x2<32, 4, true, true><<<n_items, 32, 0, st>>>(a) : step_x_f32x2<32, 4, false, true><<<n_items, 32, 0, st>>>(a); break;
-            case 64: geo ? step_x_f32x2<64, 4, true, true><<<n_items, 64, 0, st>>>(a) : step_x_f32x2<64, 4, false, true><<<n_items, 64, 0, st>>>(a); break;
-            case 128: geo ? step_x_f32x2<128, 4, true, true><<<n_items, 128, 0, st>>>(a) : step_x_f32x2<128, 4, false, true><<<n_items, 128, 0, st>>>(a); break;
-            case 256: geo ? step_x_f32x2<256, 4, true, true><<<n_items, 256, 0, st>>>(a) : step_x_f32x2<256, 4, false, true><<<n_items, 256, 0, st>>>(a); break;
-            default: return (int)cudaErrorInvalidValue;
-            }
-        } else {
-            switch (threads) {
-            case 32: geo ? step_x_f32x2<32, 4, true><<<n_items, 32, 0, st>>>(a) : step_x_f32x2<32, 4, false><<<n_items, 32, 0, st>>>(a); break;
-            case 64: geo ? step_x_f32x2<64, 4, true><<<n_items, 64, 0, st>>>(a) : step_x_f32x2<64, 4, false><<<n_items, 64, 0, st>>>(a); break;
-            case 128: geo ? step_x_f32x2<128, 4, true><<<n_items, 128, 0, st>>>(a) : step_x_f32x2<128, 4, false><<<n_items, 128, 0, st>>>(a); break;
-            case 256: geo ? step_x_f32x2<256, 4, true><<<n_items, 256, 0, st>>>(a) : step_x_f32x2<256, 4, false><<<n_items, 256, 0, st>>>(a); break;
-            default: return (int)cudaErrorInvalidValue;
-            }
-        }
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess || a.n_items_y <= 0) return (int)e;
-        if (geo) step_y_f32x2<true><<<a.n_items_y, kSplitYThreads, 0, st>>>(a);
-        else step_y_f32x2<false><<<a.n_items_y, kSplitYThreads, 0, st>>>(a);
-        return (int)cudaGetLastError();
-    }
-    if (a.kap != nullptr) {   // latitude-longitude grid (capacity form)
-        switch (threads) {
-        case 32: step_kernel_f32x2<32, 4, true><<<n_items, 32, 0, st>>>(a); break;
-        case 64: step_kernel_f32x2<64, 4, true><<<n_items, 64, 0, st>>>(a); break;
-        case 128: step_kernel_f32x2<128, 4, true><<<n_items, 128, 0, st>>>(a); break;
-        case 256: step_kernel_f32x2<256, 4, true><<<n_items, 256, 0, st>>>(a); break;
-        default: return (int)cudaErrorInvalidValue;
-        }
-        return (int)cudaGetLastError();
-    }
+    if (a.tile_rows < 1 || a.tile_rows > kTileRowsMax) return (int)cudaErrorInvalidValue;
     switch (threads) {
-    case 32: step_kernel_f32x2<32, 4><<<n_items, 32, 0, st>>>(a); break;
-    case 64: step_kernel_f32x2<64, 4><<<n_items, 64, 0, st>>>(a); break;
-    case 128: step_kernel_f32x2<128, 4><<<n_items, 128, 0, st>>>(a); break;
-    case 256: step_kernel_f32x2<256, 4><<<n_items, 256, 0, st>>>(a); break;
+    case 32: return launch_tile_nw<1>(a, n_items, st);
+    case 64: return launch_tile_nw<2>(a, n_items, st);
+    case 128: return launch_tile_nw<4>(a, n_items, st);
+    case 256: return launch_tile_nw<8>(a, n_items, st);
     default: return (int)cudaErrorInvalidValue;
     }
-    return (int)cudaGetLastError();
 }
 
 }  // namespace tsu

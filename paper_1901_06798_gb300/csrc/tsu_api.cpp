@@ -322,19 +322,16 @@ struct BoxIndex {
     }
 };
 
-constexpr int kRetakeThreads = 256, kRetakeRows = 64;   // x-sweep shape of the level-1 retake launch
-
 struct Lvl {
     std::vector<PatchDesc> P;
     std::vector<size_t> blk, blkbytes;
-    std::vector<StepItem> items, items_y;   // patch update work items (items_y: FP32 split y kernel)
-    std::vector<StepItem> items_rt;         // level 1, FP32 split update: x-sweep items of the retake launch
+    std::vector<StepItem> items;   // patch update work items
+    int tile_rows = 0;             // FP32 split update: most rows of an item
     std::vector<int> nbrs, bclist, olds;
     std::vector<BoxIndex> idx;   // per scenario spatial index of P, rebuilt by every finish_level of the level
     std::vector<int> ccand;   // coarse patches overlapping each patch's coarse-map footprint
     DevBuf<PatchDesc> dP;
-    DevBuf<StepItem> dItems, dItemsY, dItemsRt;
-    DevBuf<float> dScratch;                 // FP32 split update: Q* of every patch (3 fields each)
+    DevBuf<StepItem> dItems;
     DevBuf<int> dNbrs, dCmap, dCcand, dBc, dOlds, dList;
     DevBuf<GhostSrc> dGmap;      // ghost-cell sources of every patch, in ghost-ring order
     DevBuf<long long> dGoff;     // first dGmap entry of each patch
@@ -401,7 +398,7 @@ struct tsu_ctx {
     long long n_patches_renewed = 0, n_patches_reused = 0;   // new patches at regrids, of which kept their block
     bool ext_state = false;           // a state came from the caller (tsu_level1_buffers, restore): check its depths
     DevBuf<int> dneg;                 // count of the depth check
-    int bulk_rows = 0;                // FP32 split update: x-sweep rows by bulk copies (tsu_set_bulk_copies)
+    int bulk_rows = 0;                // FP32 split update: tile rows by bulk copies (tsu_set_bulk_copies)
     unsigned wait_polls = 1u << 22;   // polls a kernel spends on one bulk copy before giving up
     int seg_rows = 0;  // rows per work item of the patch update (0: library default)
     int step_nt = 0;   // threads per CTA of the patch update (0: library default)
@@ -464,18 +461,18 @@ struct tsu_ctx {
     int device = 0;                            // the CUDA device current at tsu_create
 
     // ------------------------------------------------------------ helpers
-    // FP32 split scheme: the patch update runs as the x and y kernels with a Q* scratch
+    // FP32 split scheme: the patch update runs on tiles (step_tile_f32.cuh)
     bool split_f32() const { return prec != TSU_F64 && c.transverse == 0; }
     int nt() const
     {
         if (step_nt > 0) return step_nt;
-        return prec == TSU_F64 ? step_threads_f64() : (split_f32() ? 32 : step_threads_f32p());
+        return prec == TSU_F64 ? step_threads_f64() : step_threads_f32p();
     }
     // physical cell sizes of level l (of an equatorial cell on latitude-longitude grids)
     double pdx(int l) const { return c.spherical ? lv[l].dxp : lv[l].dx; }
     double pdy(int l) const { return c.spherical ? lv[l].dyp : lv[l].dy; }
     // per-level launch data of the patch update: cell sizes, latitude-longitude
-    // tables, and the FP32 split kernels' scratch and y work items
+    // tables, tile height
     void level_args(StepArgs &a, int l) const
     {
         a.dx = pdx(l);
@@ -483,27 +480,16 @@ struct tsu_ctx {
         if (c.spherical) {
             a.kap = lv[l].dKap.p; a.ced = lv[l].dCed.p; a.kapf = lv[l].dKapF.p; a.cedf = lv[l].dCedF.p;
         }
-        if (split_f32()) {
-            a.scratch = lv[l].dScratch.p;
-            a.items_y = lv[l].dItemsY.p;
-            a.n_items_y = (int)lv[l].items_y.size();
-        }
+        a.tile_rows = lv[l].tile_rows;
         a.err = derr.p;
         a.bulk_rows = bulk_rows;
         a.wait_polls = wait_polls;
     }
     const int *retake_gate() const { return retake.p; }
-    // kernels one patch-update launch of level l runs
-    int step_kernels() const { return split_f32() ? 2 : 1; }
-    int seg() const { return seg_rows > 0 ? seg_rows : (prec == TSU_F64 ? 128 : (split_f32() ? 16 : 64)); }
-    // the level-1 retake launch (a.gate set): the FP32 split update sweeps x with
-    // its own wide items, the rest as the step itself
-    int retake_launch(StepArgs a, const Lvl &L)
+    int seg() const { return seg_rows > 0 ? seg_rows : (prec == TSU_F64 ? 128 : 64); }
+    // one launch of the patch update (a.gate set: the level-1 retake)
+    int launch_step(const StepArgs &a, const Lvl &L)
     {
-        if (prec != TSU_F64 && !L.items_rt.empty() && a.scratch != nullptr && !a.transverse) {
-            a.items = L.dItemsRt.p;
-            return launch_step_f32p(a, (int)L.items_rt.size(), kRetakeThreads, st);
-        }
         return prec == TSU_F64 ? launch_step_f64(a, (int)L.items.size(), nt(), st)
                                : launch_step_f32p(a, (int)L.items.size(), nt(), st);
     }
@@ -611,14 +597,10 @@ struct tsu_ctx {
         L.bclist.clear();
         L.maxring = 0;
         L.maxcells = 0;
-        L.items_y.clear();
         const int W = prec == TSU_F64 ? step_strip_width_f64(nt(), c.transverse) : step_strip_width_f32p(nt(), c.transverse);
         const bool split = split_f32();
-        size_t soff = 0;
         for (int k = 0; k < n; k++) {
             PatchDesc &p = L.P[k];
-            p.soff = split ? (long long)soff : 0;
-            if (split) soff += 3 * (size_t)p.fs;
             L.maxring = std::max(L.maxring, (p.nx + 4) * (p.ny + 4) - p.nx * p.ny);
             L.maxcells = std::max(L.maxcells, (p.nx + 4) * (p.ny + 4));
             if (p.bcmask) L.bclist.push_back(k);
@@ -626,52 +608,32 @@ struct tsu_ctx {
         // work items of the patch update in patch order, built in patch ranges on
         // host threads and joined in range order
         {
+            // FP32 split update: tiles of equal heights within a patch
+            if (split) {
+                if (seg_rows > 0) {
+                    L.tile_rows = std::min(seg_rows, kTileRowsMax);
+                } else {
+                    std::vector<int> px(n), py(n);
+                    for (int k = 0; k < n; k++) { px[k] = L.P[k].nx; py[k] = L.P[k].ny; }
+                    L.tile_rows = tile_rows_f32p(n, px.data(), py.data(), nt());
+                }
+            }
             const int sg = seg();
-            std::vector<std::vector<StepItem>> xi(16), yi(16);
-            std::array<std::array<int, 2>, 16> rr{};
+            std::vector<std::vector<StepItem>> xi(16);
             parallel_ranges(n, [&](int q, int b, int e) {
-                rr[q] = {b, e};
-                std::vector<StepItem> &ox = xi[q], &oy = yi[q];
+                std::vector<StepItem> &ox = xi[q];
                 for (int k = b; k < e; k++) {
                     const PatchDesc &p = L.P[k];
-                    if (split) {
-                        // x kernel: every row including the ghost rows, no halo rows; y kernel:
-                        // strips of 64 columns and segments of 64 interior rows
-                        for (int x0 = 0; x0 < p.nx; x0 += W)
-                            for (int y0 = -2; y0 < p.ny + 2; y0 += sg)
-                                ox.push_back(StepItem{k, x0, y0, std::min(W, p.nx - x0), std::min(sg, p.ny + 2 - y0)});
-                        constexpr int WY = 64, SY = 64;
-                        for (int x0 = 0; x0 < p.nx; x0 += WY)
-                            for (int y0 = 0; y0 < p.ny; y0 += SY)
-                                oy.push_back(StepItem{k, x0, y0, std::min(WY, p.nx - x0), std::min(SY, p.ny - y0)});
-                    } else {
-                        for (int x0 = 0; x0 < p.nx; x0 += W)
-                            for (int y0 = 0; y0 < p.ny; y0 += sg)
-                                ox.push_back(StepItem{k, x0, y0, std::min(W, p.nx - x0), std::min(sg, p.ny - y0)});
-                    }
+                    const int sk = split ? tile_cut(p.ny, L.tile_rows) : sg;
+                    for (int x0 = 0; x0 < p.nx; x0 += W)
+                        for (int y0 = 0; y0 < p.ny; y0 += sk)
+                            ox.push_back(StepItem{k, x0, y0, std::min(W, p.nx - x0), std::min(sk, p.ny - y0)});
                 }
             });
-            size_t nxi = 0, nyi = 0;
-            for (int q = 0; q < 16; q++) { nxi += xi[q].size(); nyi += yi[q].size(); }
+            size_t nxi = 0;
+            for (int q = 0; q < 16; q++) nxi += xi[q].size();
             L.items.reserve(nxi);
-            L.items_y.reserve(nyi);
-            for (int q = 0; q < 16; q++) {
-                L.items.insert(L.items.end(), xi[q].begin(), xi[q].end());
-                L.items_y.insert(L.items_y.end(), yi[q].begin(), yi[q].end());
-            }
-        }
-        // the level-1 retake launch of the FP32 split update: its CTAs exit unless
-        // their scenario is retaken, so its x sweep runs the widest CTAs (every
-        // launch shape gives the same bits), about 30 times fewer than the default
-        L.items_rt.clear();
-        if (split && l == 0 && c.cfl_retake) {
-            const int Wr = step_strip_width_f32p(kRetakeThreads, 0);
-            for (int k = 0; k < n; k++) {
-                const PatchDesc &p = L.P[k];
-                for (int x0 = 0; x0 < p.nx; x0 += Wr)
-                    for (int y0 = -2; y0 < p.ny + 2; y0 += kRetakeRows)
-                        L.items_rt.push_back(StepItem{k, x0, y0, std::min(Wr, p.nx - x0), std::min(kRetakeRows, p.ny + 2 - y0)});
-            }
+            for (int q = 0; q < 16; q++) L.items.insert(L.items.end(), xi[q].begin(), xi[q].end());
         }
         // per scenario spatial indices of this level and the coarser one
         std::vector<std::vector<int>> ids(nscen);
@@ -748,11 +710,8 @@ struct tsu_ctx {
                     L.P[order[o]].ccand_off += cshift[q];
                 }
         }
-        if (split) L.dScratch.ensure(std::max<size_t>(soff, 64), st);
         L.dP.upload(L.P, st, uring);
         L.dItems.upload(L.items, st, uring);
-        L.dItemsY.upload(L.items_y, st, uring);
-        if (!L.items_rt.empty()) L.dItemsRt.upload(L.items_rt, st, uring);
         L.dNbrs.upload(L.nbrs, st, uring);
         if (l > 0) {
             // the coarse table's device copy is current: its finish_level ran first
@@ -1225,13 +1184,10 @@ struct tsu_ctx {
                 ps.e0 = prof_event();
                 ps.e1 = prof_event();
                 for (int sc = 0; sc < nscen; sc++) ps.cells += cells_h[(size_t)sc * kMaxLevels + l];
-                ps.kernels = step_kernels();
+                ps.kernels = 1;
                 CK(cudaEventRecord(ps.e0, st));
             }
-            int e = prec == TSU_F64 ? launch_step_f64(a, (int)L.items.size(), nt(), st)
-                                    : launch_step_f32p(a, (int)L.items.size(), nt(), st);
-            kl(e, "patch step");
-            launches += step_kernels() - 1;
+            kl(launch_step(a, L), "patch step");
             // Sec. 2.2 CFL condition: a level-1 step with nu > cfl_max is taken
             // again with dt^1 = cfl_desired / rate before any finer level moves.
             // The decision stays on the device: the step's input buffer is
@@ -1245,12 +1201,10 @@ struct tsu_ctx {
                "post step");
             if (retake) {
                 a.gate = retake_gate();
-                e = retake_launch(a, L);
-                kl(e, "patch step (retake)");
-                launches += step_kernels() - 1;
+                kl(launch_step(a, L), "patch step (retake)");
                 kl(k_post_level(ctrl(), l, nscen, L.R, pdx(l), pdy(l), c.cfl_max, c.cfl_desired, 3, st, ends ? 1 : 0),
                    "post step (retake)");
-                ps.kernels += step_kernels() + 1;
+                ps.kernels += 2;
             }
             if (ends) end_done_ = true;
             if (prof) {
@@ -1817,8 +1771,7 @@ struct tsu_ctx {
             L.dP.release(); L.dItems.release(); L.dNbrs.release(); L.dCmap.release(); L.dCcand.release(); L.dBc.release();
             L.dOlds.release(); L.dList.release();
             L.dKap.release(); L.dCed.release(); L.dKapF.release(); L.dCedF.release();
-            L.dItemsY.release(); L.dScratch.release();
-            L.dGmap.release(); L.dGoff.release(); L.dGinterp.release(); L.dGcount.release(); L.dItemsRt.release();
+            L.dGmap.release(); L.dGoff.release(); L.dGinterp.release(); L.dGcount.release();
         }
         for (auto &g : grids) if (g.dev) cudaFreeAsync(g.dev, st);
         dGrids.release(); dGridScen.release(); dEtaIdx.release();
@@ -2334,11 +2287,11 @@ int tsu_autotune(tsu_ctx *ctx, int reps, int *best_threads, int *best_seg_rows, 
         ctx->zero_dtf.ensure(ctx->nscen, ctx->st);
         CK(cudaMemsetAsync(ctx->zero_dt.p, 0, ctx->nscen * sizeof(double), ctx->st));
         CK(cudaMemsetAsync(ctx->zero_dtf.p, 0, ctx->nscen * sizeof(float), ctx->st));
-        // threads x rows per work item; the FP32 split update's x kernel also takes
-        // 32 threads and needs no halo rows, so it gets shorter segments
+        // threads x rows per work item; the FP32 split update also takes 32 threads,
+        // and its items are tiles held in shared memory: shorter ones
         const bool split = ctx->split_f32();
         const int nts[4] = {64, 128, 256, 32};
-        const int segs[4] = {split ? 16 : 32, split ? 32 : 64, split ? 64 : 128, split ? 128 : 256};
+        const int segs[4] = {split ? 16 : 32, split ? 30 : 64, split ? 44 : 128, split ? 60 : 256};
         const int n_nt = split ? 4 : 3;
         cudaEvent_t e0, e1;
         CK(cudaEventCreate(&e0));
@@ -2363,10 +2316,7 @@ int tsu_autotune(tsu_ctx *ctx, int reps, int *best_threads, int *best_seg_rows, 
                         sa.manning = (ctx->c.manning_n * ctx->c.manning_n) * ctx->c.g;
                         ctx->level_args(sa, l);
                         set_f32_constants(sa);
-                        int e = ctx->prec == TSU_F64 ? launch_step_f64(sa, (int)L.items.size(), ctx->nt(), ctx->st)
-                                                     : launch_step_f32p(sa, (int)L.items.size(), ctx->nt(), ctx->st);
-                        ctx->kl(e, "autotune step");
-                        ctx->launches += ctx->step_kernels() - 1;
+                        ctx->kl(ctx->launch_step(sa, L), "autotune step");
                     }
                 };
                 run();
@@ -2530,10 +2480,7 @@ int tsu_time_level1_steps(tsu_ctx *ctx, int warmup, int n, double *kernel_ms_out
             ctx->level_args(a, 0);
             set_f32_constants(a);
             CK(cudaEventRecord(ev[2 * k], ctx->st));
-            int e = ctx->prec == TSU_F64 ? launch_step_f64(a, (int)L.items.size(), ctx->nt(), ctx->st)
-                                         : launch_step_f32p(a, (int)L.items.size(), ctx->nt(), ctx->st);
-            ctx->kl(e, "patch step");
-            ctx->launches += ctx->step_kernels() - 1;
+            ctx->kl(ctx->launch_step(a, L), "patch step");
             CK(cudaEventRecord(ev[2 * k + 1], ctx->st));
             // the rest of the step exactly as level_step and coarse_step run it: with
             // the CFL retake on, the post-level check, the retake launch (its CTAs
@@ -2546,9 +2493,7 @@ int tsu_time_level1_steps(tsu_ctx *ctx, int warmup, int n, double *kernel_ms_out
                     "post step");
             if (retake) {
                 a.gate = ctx->retake_gate();
-                e = ctx->retake_launch(a, L);
-                ctx->kl(e, "patch step (retake)");
-                ctx->launches += ctx->step_kernels() - 1;
+                ctx->kl(ctx->launch_step(a, L), "patch step (retake)");
                 ctx->kl(k_post_level(ctx->ctrl(), 0, ctx->nscen, L.R, ctx->pdx(0), ctx->pdy(0), ctx->c.cfl_max,
                                      ctx->c.cfl_desired, 3, ctx->st, 1),
                         "post step (retake)");

@@ -21,7 +21,6 @@ struct PatchDesc {
     int cmap_off, cmap_i0, cmap_j0, cmap_w, cmap_h;  // coarse-level patch index per coarse cell (levels >= 2)
     int ccand_off, ccand_cnt;  // coarse patches overlapping the coarse map's footprint (the map's painters)
     int old_off, old_cnt;      // old same-level patches overlapping (regrid initialisation)
-    long long soff;            // FP32 split update: element offset of the patch's Q* (3 fields of fs) in the scratch
 };
 
 // One work item of the patch update: a strip of columns [x0, x0+w) and a row
@@ -53,17 +52,15 @@ struct StepArgs {
     // length of the latitude edge below row J at ced[J + 2]; null on Cartesian grids
     const double *kap, *ced;
     const float *kapf, *cedf;
-    // FP32 split update (two kernels): the level's Q* scratch and the y kernel's
-    // work items (strips of 64 columns x row segments); null scratch: fused kernel
-    float *scratch;
-    const StepItem *items_y;
-    int n_items_y;
+    // FP32 split update (step_tile_f32.cuh): the most rows of a work item, and,
+    // with null items, the tile columns of the one patch the launch covers
+    int tile_rows, tile_nsx;
     // CFL retake of a level-1 step: when set, a work item of scenario s runs
     // only if gate[s] != 0 (null: every item runs)
     const int *gate;
     // device error flag (TSU_DEV_ERR_* bits; null: not reported); FP32 split
-    // update: bulk row copies in the x-sweep kernel (0: per-thread cp.async) and
-    // the polls it spends waiting for one before it gives up
+    // update: bulk copies of the tile's rows (0: per-thread cp.async) and the
+    // polls a thread spends waiting for them before it gives up
     int *err;
     int bulk_rows;
     unsigned wait_polls;
@@ -97,5 +94,15 @@ int step_threads_f32p();
 // per CTA (the unsplit kernels take one column per thread in both precisions)
 int step_strip_width_f64(int threads, int transverse);
 int step_strip_width_f32p(int threads, int transverse);
+// FP32 split update: rows of a tile for n patches of nx[k] x ny[k] cells
+// advanced together by CTAs of `threads`, and rows of a patch's tiles (of at most
+// `cap` rows): equal and even
+int tile_rows_f32p(int n, const int *nx, const int *ny, int threads);
+inline int tile_cut(int ny, int cap)
+{
+    const int nt = (ny + cap - 1) / cap, r = (ny + nt - 1) / nt;
+    return r + (r & 1) <= cap ? r + (r & 1) : r;
+}
+constexpr int kTileRowsMax = 124;   // a tile row takes 1 KiB of shared memory
 
 }  // namespace tsu
