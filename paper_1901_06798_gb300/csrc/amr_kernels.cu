@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 #include <type_traits>
 #include "amr_kernels.h"
+#include "step_tail.cuh"
 
 namespace tsu {
 
@@ -297,9 +298,28 @@ __device__ __forceinline__ bool bc_source(const PatchDesc &P, int nxl, int nyl, 
     return out;
 }
 
-template <typename T>
-__global__ void bc_kernel(LevelView L, int cur, BcArgs bcs, int do_state, int do_B)
+// Start of a coarse step: dt^1 = min(dt_max, nu_d / max_l(rate_l / R_l)).
+__device__ __forceinline__ void begin_step(const CtrlView &cv, const BeginArgs &b)
 {
+    for (int s = threadIdx.x; s < b.nscen; s += blockDim.x) {
+        double m = 0.0;
+        for (int l = 0; l < b.nlev; l++) m = fmax(m, cv.rate[(long long)s * cv.max_levels + l] / b.Rl[l]);
+        const double dt = m > 0.0 ? b.cfl_desired / m : b.dt_max;
+        cv.dt1[s] = fmin(dt, b.dt_max);
+        cv.dt1f[s] = (float)cv.dt1[s];
+        for (int l = 0; l < cv.max_levels; l++) cv.rate[(long long)s * cv.max_levels + l] = 0.0;
+    }
+}
+
+// (with bg.nscen > 0, on level 1, one more CTA row starts the coarse step: the
+// boundaries need no dt)
+template <typename T>
+__global__ void bc_kernel(LevelView L, int cur, BcArgs bcs, int do_state, int do_B, CtrlView cv, BeginArgs bg)
+{
+    if (bg.nscen > 0 && blockIdx.x + 1 == gridDim.x) {
+        if (blockIdx.y == 0) begin_step(cv, bg);
+        return;
+    }
     const PatchDesc P = L.descs[bcs.list[blockIdx.x]];
     const int n = ring_count(P);
     Acc<T> a = acc<T>(L.arena, P);
@@ -912,115 +932,46 @@ __global__ void __launch_bounds__(256) cell_speed_kernel(LevelView L, const int 
     }
 }
 
-// After a level step (mode 0) or a cell-speed scan (mode 1): fold the level's
-// max speeds into its rate max(sx/dx, sy/dy), check the CFL number of the step
-// just taken and count cell updates (mode 0).
-// After a level's step: the level's rate max(sx/dx, sy/dy) from the speeds
-// the step kernels reduced (smax is cleared for the next step).
-//   mode 0: a kept step -- count its cells, a violation if dt rate > cfl_max,
-//           and fold the rate into the level's maximum;
-//   mode 1: cell speeds of new patches -- the rate only;
-//   mode 2: a level-1 step that may be retaken (Sec. 2.2 CFL condition): if
-//           dt rate > cfl_max, mark the scenario for a retake and set
-//           dt^1 = cfl_desired / rate (the state is still in the untouched
-//           buffer); otherwise keep it as in mode 0;
-//   mode 3: after the retake launch -- keep the retaken steps as in mode 0.
-// A rate that is not a finite number (a NaN or infinite speed) sets the error
-// flag to TSU_DEV_ERR_NAN.  end_step (modes 0 and 3, every scenario): then
-// t += dt^1, as end_step_kernel.
-__global__ void post_level_kernel(CtrlView cv, int level, int nscen, double R, double dx, double dy, double cfl_max,
-                                  double cfl_desired, int mode, int end_step)
+// Cell speeds of new patches folded into the level's rate (mode 1 of post_level;
+// the speed accumulators are cleared for the next step).
+__global__ void post_rate_kernel(CtrlView cv, int level, int nscen, double R, double dx, double dy)
 {
     for (int s = threadIdx.x; s < nscen; s += blockDim.x) {
-        do {
-            unsigned long long *sm = cv.smax + 2 * s;
-            double sx = __longlong_as_double((long long)sm[0]);
-            double sy = __longlong_as_double((long long)sm[1]);
-            sm[0] = 0ull;
-            sm[1] = 0ull;
-            if (mode == 3 && cv.retake[s] == 0) break;
-            double rate = fmax(sx / dx, sy / dy);
-            if (!(sx <= 1.0e300 && sy <= 1.0e300)) atomicOr(cv.err, TSU_DEV_ERR_NAN);
-            double *ra = cv.rate + (long long)s * cv.max_levels + level;
-            if (mode != 1) {
-                double dt = cv.dt1[s] / R;
-                if (dt * rate > cfl_max) {
-                    if (mode == 2) {
-                        cv.retake[s] = 1;
-                        cv.retakes[s] += 1;
-                        cv.dt1[s] = cfl_desired / rate;
-                        cv.dt1f[s] = (float)cv.dt1[s];
-                        break;
-                    }
-                    cv.cfl_viol[s] += 1;
-                }
-                if (mode == 2 || mode == 3) cv.retake[s] = 0;
-                cv.cell_updates[s] += cv.cells[(long long)s * cv.max_levels + level];
-            }
-            *ra = fmax(*ra, rate);
-        } while (false);
-        if (end_step) cv.t[s] = cv.t[s] + cv.dt1[s];
+        unsigned long long *sm = cv.smax + 2 * s;
+        const double sx = __longlong_as_double((long long)sm[0]), sy = __longlong_as_double((long long)sm[1]);
+        sm[0] = 0ull;
+        sm[1] = 0ull;
+        post_level(cv, s, level, sx, sy, R, dx, dy, 0.0, 0.0, 1);
     }
 }
 
-// Start of a coarse step: dt^1 = min(dt_max, nu_d / max_l(rate_l / R_l)).
-__global__ void begin_step_kernel(CtrlView cv, int nscen, int nlev, const double *Rl, double cfl_desired,
-                                  double dt_max)
-{
-    for (int s = threadIdx.x; s < nscen; s += blockDim.x) {
-        double m = 0.0;
-        for (int l = 0; l < nlev; l++) m = fmax(m, cv.rate[(long long)s * cv.max_levels + l] / Rl[l]);
-        double dt = m > 0.0 ? cfl_desired / m : dt_max;
-        cv.dt1[s] = fmin(dt, dt_max);
-        cv.dt1f[s] = (float)cv.dt1[s];
-        for (int l = 0; l < cv.max_levels; l++) cv.rate[(long long)s * cv.max_levels + l] = 0.0;
-    }
-}
-
-__global__ void end_step_kernel(CtrlView cv, int nscen)
-{
-    for (int s = threadIdx.x; s < nscen; s += blockDim.x) cv.t[s] = cv.t[s] + cv.dt1[s];
-}
+// the end of a level step whose update launch does not count its CTAs
+template <typename T, bool PERT> __global__ void tail_kernel(StepArgs a) { end_level<T, PERT>(a); }
 
 // ---------------------------------------------------------------- gauges, fields
 
+// The end of a coarse step of a refined run: t += dt^1, then the gauge samples
+// from the finest patches (a one-level grid does both in step_tail)
 template <typename T, bool PERT>
-__global__ void gauge_kernel(GaugeArgs ga, CtrlView cv)
+__global__ void end_step_kernel(GaugeArgs ga, CtrlView cv)
 {
+    for (int s = threadIdx.x; s < ga.nscen; s += blockDim.x) cv.t[s] = cv.t[s] + cv.dt1[s];
+    if (ga.ngauges <= 0) return;
+    __syncthreads();
     const int total = ga.nscen * ga.ngauges;
     const long long sidx = *ga.nsamp;
     for (int c = threadIdx.x; c < total; c += blockDim.x) {
-        int s = c / ga.ngauges;
+        const int s = c / ga.ngauges, q = c - s * ga.ngauges;
         const GaugeLoc gl = ga.loc[c];
         double eta = __longlong_as_double(0x7ff8000000000000LL);
         if (gl.patch >= 0) {
             const LevelView &L = ga.levels[gl.level];
             const PatchDesc P = L.descs[gl.patch];
-            Acc<T> a = acc<T>(L.arena, P);
-            int cur = ga.curs[gl.level];
-            double dxl = ga.dxl[gl.level], dyl = ga.dyl[gl.level];
-            double x = ga.xy[2 * (c % ga.ngauges)], y = ga.xy[2 * (c % ga.ngauges) + 1];
-            double fx = (x - ga.x0) / dxl - 0.5, fy = (y - ga.y0) / dyl - 0.5;
-            int ia = (int)floor(fx), ja = (int)floor(fy);
-            double tx = fx - (double)ia, ty = fy - (double)ja;
-            if (ia < P.i0) { ia = P.i0; tx = 0.0; }
-            if (ia > P.i0 + P.nx - 2) { ia = P.i0 + P.nx - 2; tx = 1.0; }
-            if (ja < P.j0) { ja = P.j0; ty = 0.0; }
-            if (ja > P.j0 + P.ny - 2) { ja = P.j0 + P.ny - 2; ty = 1.0; }
-            int i = ia - P.i0, j = ja - P.j0;
-            const T *q0 = a.f(cur, 0), *B = a.Bp();
-            double e[4];
-            int di[4] = {0, 1, 0, 1}, dj[4] = {0, 0, 1, 1};
-            for (int m = 0; m < 4; m++) {
-                long long k = a.idx(i + di[m], j + dj[m]);
-                e[m] = PERT ? (double)q0[k] : (double)q0[k] + (double)B[k];
-            }
-            double aa = e[0] + tx * (e[1] - e[0]);
-            double bb = e[2] + tx * (e[3] - e[2]);
-            eta = aa + ty * (bb - aa);
+            eta = gauge_eta<T, PERT>(P, reinterpret_cast<const T *>(L.arena) + P.off, ga.curs[gl.level], ga.xy[2 * q],
+                                     ga.xy[2 * q + 1], ga.x0, ga.y0, ga.dxl[gl.level], ga.dyl[gl.level]);
         }
-        ga.eta[(sidx * ga.nscen + s) * ga.ngauges + (c % ga.ngauges)] = eta;
-        if (c % ga.ngauges == 0) ga.t[sidx * ga.nscen + s] = cv.t[s];
+        ga.eta[(sidx * ga.nscen + s) * ga.ngauges + q] = eta;
+        if (q == 0) ga.t[sidx * ga.nscen + s] = cv.t[s];
     }
     __syncthreads();
     if (threadIdx.x == 0) *ga.nsamp = sidx + 1;
@@ -1207,12 +1158,15 @@ int k_ghost_fill(int prec, const LevelView &L, const LevelView &C, int npatch, i
 }
 
 int k_bc(int prec, const LevelView &L, const BcArgs &b, int nlist, int maxring, int cur, int do_state, int do_B,
-         cudaStream_t st)
+         cudaStream_t st, const CtrlView *cv, const BeginArgs *bg)
 {
     if (nlist <= 0) return 0;
     dim3 g = grid_for(maxring, nlist, 128);
-    if (prec == 0) bc_kernel<double><<<g, 128, 0, st>>>(L, cur, b, do_state, do_B);
-    else bc_kernel<float><<<g, 128, 0, st>>>(L, cur, b, do_state, do_B);
+    if (bg) g.x++;
+    const CtrlView c = cv ? *cv : CtrlView{};
+    const BeginArgs a = bg ? *bg : BeginArgs{};
+    if (prec == 0) bc_kernel<double><<<g, 128, 0, st>>>(L, cur, b, do_state, do_B, c, a);
+    else bc_kernel<float><<<g, 128, 0, st>>>(L, cur, b, do_state, do_B, c, a);
     return (int)cudaGetLastError();
 }
 
@@ -1447,31 +1401,21 @@ int k_cell_speed(int prec, const LevelView &L, const int *list, int nlist, int m
     return (int)cudaGetLastError();
 }
 
-int k_post_level(const CtrlView &cv, int level, int nscen, double R, double dx, double dy, double cfl_max,
-                 double cfl_desired, int mode,
-                 cudaStream_t st, int end_step)
+int k_tail(int prec, const StepArgs &a, cudaStream_t st)
 {
-    post_level_kernel<<<1, 128, 0, st>>>(cv, level, nscen, R, dx, dy, cfl_max, cfl_desired, mode,
-                                         (mode == 0 || mode == 3) ? end_step : 0);
+    TSU_DISPATCH(prec, tail_kernel, <<<1, 128, 0, st>>>(a));
     return (int)cudaGetLastError();
 }
 
-int k_begin_step(const CtrlView &cv, int nscen, int nlev, const double *Rl, double cfl_desired, double dt_max,
-                 cudaStream_t st)
+int k_post_rate(const CtrlView &cv, int level, int nscen, double R, double dx, double dy, cudaStream_t st)
 {
-    begin_step_kernel<<<1, 128, 0, st>>>(cv, nscen, nlev, Rl, cfl_desired, dt_max);
+    post_rate_kernel<<<1, 128, 0, st>>>(cv, level, nscen, R, dx, dy);
     return (int)cudaGetLastError();
 }
 
-int k_end_step(const CtrlView &cv, int nscen, cudaStream_t st)
+int k_end_step(int prec, const GaugeArgs &ga, const CtrlView &cv, cudaStream_t st)
 {
-    end_step_kernel<<<1, 128, 0, st>>>(cv, nscen);
-    return (int)cudaGetLastError();
-}
-
-int k_gauges(int prec, const GaugeArgs &ga, const CtrlView &cv, cudaStream_t st)
-{
-    TSU_DISPATCH(prec, gauge_kernel, <<<1, 256, 0, st>>>(ga, cv));
+    TSU_DISPATCH(prec, end_step_kernel, <<<1, 256, 0, st>>>(ga, cv));
     return (int)cudaGetLastError();
 }
 

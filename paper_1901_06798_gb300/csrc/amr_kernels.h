@@ -37,22 +37,6 @@ struct LevelView {
     const int *icount;      // entries of ilist
 };
 
-// Device control block of a context: per scenario dt, time, rates, counters.
-struct CtrlView {
-    double *dt1, *t;
-    float *dt1f;                 // FP32 copy of dt1 for the perturbation-form kernel
-    double *rate;                // [scen][max_levels]
-    double *cell_updates;        // [scen]
-    const double *cells;         // [scen][max_levels] interior cells per level
-    long long *cfl_viol;         // [scen]
-    unsigned long long *smax;    // [scen][2]
-    int *retake;                 // [scen] 1: the level-1 step is being retaken (the step kernels' gate)
-    long long *retakes;          // [scen] level-1 steps retaken
-    int *err;                    // device error flag (TSU_DEV_ERR_*)
-    int max_levels;
-};
-
-
 struct TopoDev {
     int nx, ny;
     double x0, y0, dx, dy;
@@ -106,8 +90,11 @@ struct BcArgs {
     int bc[4];
 };
 
-struct GaugeLoc {
-    int level, patch;            // finest patch containing the gauge, or patch = -1
+// start of a coarse step; nscen = 0: none
+struct BeginArgs {
+    int nscen, nlev;
+    const double *Rl;
+    double cfl_desired, dt_max;
 };
 
 struct GaugeArgs {
@@ -129,8 +116,9 @@ int k_ghost_map(const LevelView &L, GhostSrc *gmap, int2 *ilist, int *icount, in
                 cudaStream_t st);
 int k_ghost_fill(int prec, const LevelView &L, const LevelView &C, int npatch, int maxring, int cur, int cur_c,
                  int ratio, double alpha, double drytol, int *err, cudaStream_t st);
+// bg (level 1): the same launch starts the coarse step (dt^1 from the rates)
 int k_bc(int prec, const LevelView &L, const BcArgs &b, int nlist, int maxring, int cur, int do_state, int do_B,
-         cudaStream_t st);
+         cudaStream_t st, const CtrlView *cv = nullptr, const BeginArgs *bg = nullptr);
 int k_average(int prec, const LevelView &F, const LevelView &C, int npatch, int maxcells, int cur_f, int cur_c, int r,
               double drytol, int *err, cudaStream_t st);
 // Old: the level's previous patch table at a regrid (B copied where an old patch held the cell), or a view
@@ -174,15 +162,12 @@ struct HaloMsg {
 // pack (unpack = 0: patch buffers -> buf) or unpack (buf -> patch buffers) n boxes
 int k_halo(int prec, const LevelView &L, const HaloMsg *msgs, int n, int cur, void *buf, int unpack, cudaStream_t st);
 
-// end_step 1 (modes 0 and 3): the step was a one-level grid's whole coarse step (mode 3: after its
-// retake launch), and the kernel also advances t by dt^1 (the work of k_end_step, saving its launch)
-int k_post_level(const CtrlView &cv, int level, int nscen, double R, double dx, double dy, double cfl_max,
-                 double cfl_desired, int mode,
-                 cudaStream_t st, int end_step = 0);
-int k_begin_step(const CtrlView &cv, int nscen, int nlev, const double *Rl, double cfl_desired, double dt_max,
-                 cudaStream_t st);
-int k_end_step(const CtrlView &cv, int nscen, cudaStream_t st);
-int k_gauges(int prec, const GaugeArgs &ga, const CtrlView &cv, cudaStream_t st);
+// rate of a level from the cell speeds of new patches (smax, cleared)
+int k_post_rate(const CtrlView &cv, int level, int nscen, double R, double dx, double dy, cudaStream_t st);
+// what ends a level step (a.tail), as a launch of its own
+int k_tail(int prec, const StepArgs &a, cudaStream_t st);
+// end of a coarse step of a refined run: t += dt^1, gauge samples
+int k_end_step(int prec, const GaugeArgs &ga, const CtrlView &cv, cudaStream_t st);
 // maxpts: an upper bound on the output points one patch covers (sizes the grid)
 int k_read_field(int prec, const LevelView &L, int npatch, int maxpts, int cur, int scen, int field, double *dst, int nx,
                  int ny, double x0, double y0, double dx, double dy, double X0, double Y0, double dxl, double dyl,

@@ -25,20 +25,35 @@ int tile_ctas(int rows, int threads)
     return std::max(1, std::min(512 / threads, 228 * 1024 / (tile_smem(rows) + 1024)));
 }
 
-template <int NW, bool GEO, bool BULK> int launch_tile(const StepArgs &a, int n, cudaStream_t st)
+// above 48 KiB of dynamic shared memory a kernel has to be told so, once per device
+template <typename K> int allow_smem(K kernel, unsigned long long &told)
 {
-    // above 48 KiB of dynamic shared memory a kernel has to be told so, once per device
-    static unsigned long long told = 0;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return (int)e;
-    if (dev >= 64 || !(told >> dev & 1)) {
-        e = cudaFuncSetAttribute(step_tile_f32<NW, GEO, BULK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 tile_smem(kTileRowsMax));
-        if (e != cudaSuccess) return (int)e;
-        if (dev < 64) told |= 1ull << dev;
-    }
+    if (dev < 64 && (told >> dev & 1)) return 0;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_smem(kTileRowsMax));
+    if (e == cudaSuccess && dev < 64) told |= 1ull << dev;
+    return (int)e;
+}
+
+template <int NW, bool GEO, bool BULK> int launch_tile(const StepArgs &a, int n, cudaStream_t st)
+{
+    static unsigned long long told = 0;
+    const int e = allow_smem(step_tile_f32<NW, GEO, BULK>, told);
+    if (e) return e;
     step_tile_f32<NW, GEO, BULK><<<n, NW * 32, tile_smem(a.tile_rows), st>>>(a);
+    return (int)cudaGetLastError();
+}
+
+template <bool GEO> int launch_retake(const StepArgs &a, int n, cudaStream_t st)
+{
+    static unsigned long long told = 0;
+    const int e = allow_smem(retake_tile_f32<GEO>, told);
+    if (e) return e;
+    StepArgs b = a;
+    b.n_items = n;
+    retake_tile_f32<GEO><<<std::min(n, kSMs * tile_ctas(a.tile_rows, 128)), 128, tile_smem(a.tile_rows), st>>>(b);
     return (int)cudaGetLastError();
 }
 
@@ -80,6 +95,8 @@ int launch_step_f32p(const StepArgs &a, int n_items, int threads, cudaStream_t s
     if (n_items <= 0) return 0;
     if (a.transverse) return launch_unsplit_f32p(a, n_items, threads, st);
     if (a.tile_rows < 1 || a.tile_rows > kTileRowsMax) return (int)cudaErrorInvalidValue;
+    // (every launch shape and way of copying gives the same bits)
+    if (a.gate != nullptr) return a.kap != nullptr ? launch_retake<true>(a, n_items, st) : launch_retake<false>(a, n_items, st);
     switch (threads) {
     case 32: return launch_tile_nw<1>(a, n_items, st);
     case 64: return launch_tile_nw<2>(a, n_items, st);

@@ -33,6 +33,7 @@
 // two agree to the last bit.
 #pragma once
 #include <cuda_runtime.h>
+#include "step_tail.cuh"
 #include "tsu_device.h"
 
 namespace tsu {
@@ -315,8 +316,7 @@ template <typename T> __device__ __forceinline__ const T *geo_table(const double
 template <> __device__ __forceinline__ const double *geo_table<double>(const double *d, const float *) { return d; }
 template <> __device__ __forceinline__ const float *geo_table<float>(const double *, const float *f) { return f; }
 
-template <typename T, bool PERT, int NT, int RING, bool GEO = false>
-__global__ void __launch_bounds__(NT) step_kernel(StepArgs a)
+template <typename T, bool PERT, int NT, int RING, bool GEO> __device__ __forceinline__ void step_item(const StepArgs &a)
 {
     static_assert(RING >= 3, "the derived values of row k+1 need its copy complete at iteration k");
     __shared__ T ring[RING][4][NT];
@@ -534,6 +534,14 @@ __global__ void __launch_bounds__(NT) step_kernel(StepArgs a)
         atomic_max_speed(a.smax + 2 * P.scen + 0, (double)mx);
         atomic_max_speed(a.smax + 2 * P.scen + 1, (double)my);
     }
+}
+
+template <typename T, bool PERT, int NT, int RING, bool GEO = false>
+__global__ void __launch_bounds__(NT) step_kernel(StepArgs a)
+{
+    if (!launch_live(a)) return;
+    step_item<T, PERT, NT, RING, GEO>(a);
+    step_tail<T, PERT>(a);
 }
 
 }  // namespace tsu

@@ -52,8 +52,7 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem));
 }
 
-template <int NW, bool GEO, bool BULK>
-__global__ void __launch_bounds__(NW * 32, 16 / NW) step_tile_f32(StepArgs a)
+template <int NW, bool GEO, bool BULK> __device__ __forceinline__ void tile_item(const StepArgs &a, int item)
 {
     using namespace x2;
     constexpr unsigned ALL = 0xffffffffu;
@@ -65,9 +64,9 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) step_tile_f32(StepArgs a)
     __shared__ unsigned dry_rows[(kTileRowsMax + 4 + 31) / 32];   // bit k: tile row k has a dry cell
 
     StepItem it;
-    if (a.items) it = a.items[blockIdx.x];
+    if (a.items) it = a.items[item];
     else {   // one patch cut into tiles of a.tile_rows rows
-        const int nsx = a.tile_nsx, sy = blockIdx.x / nsx, sx = blockIdx.x - sy * nsx;
+        const int nsx = a.tile_nsx, sy = item / nsx, sx = item - sy * nsx;
         const PatchDesc &P0 = a.descs[0];
         it.patch = 0;
         it.x0 = sx * kTileCols; it.y0 = sy * a.tile_rows;
@@ -491,6 +490,27 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) step_tile_f32(StepArgs a)
         atomic_max_speed(a.smax + 2 * P.scen + 0, (double)mx);
         atomic_max_speed(a.smax + 2 * P.scen + 1, (double)my);
     }
+}
+
+template <int NW, bool GEO, bool BULK>
+__global__ void __launch_bounds__(NW * 32, 16 / NW) step_tile_f32(StepArgs a)
+{
+    if (!launch_live(a)) return;
+    tile_item<NW, GEO, BULK>(a, blockIdx.x);
+    step_tail<float, true>(a);
+}
+
+// The retake launch (a.gate set): a CTA slot's worth of CTAs, which leave at once
+// unless a scenario is to be retaken and otherwise stride over the items.  With as
+// many CTAs as items it cost 12 us on the 4096^2 grid to find nothing to do.
+template <bool GEO> __global__ void __launch_bounds__(128, 4) retake_tile_f32(StepArgs a)
+{
+    if (!launch_live(a)) return;
+    for (int item = blockIdx.x; item < a.n_items; item += gridDim.x) {
+        tile_item<4, GEO, false>(a, item);
+        __syncthreads();   // before the next tile overwrites this one
+    }
+    step_tail<float, true>(a);
 }
 
 }  // namespace tsu

@@ -155,8 +155,7 @@ template <typename T> __device__ __forceinline__ T dt_level(const StepArgs &a, i
 template <> __device__ __forceinline__ double dt_level<double>(const StepArgs &a, int scen) { return a.dt1[scen] / a.R; }
 template <> __device__ __forceinline__ float dt_level<float>(const StepArgs &a, int scen) { return a.dt1f[scen] * a.rR; }
 
-template <typename T, bool PERT, int NT, int RING>
-__global__ void __launch_bounds__(NT) step_unsplit_kernel(StepArgs a)
+template <typename T, bool PERT, int NT, int RING> __device__ __forceinline__ void unsplit_item(const StepArgs &a)
 {
     static_assert(RING >= 5, "rows r-2 .. r are read while rows r+1, r+2 are in flight");
     using S = UnsplitSmem<NT, RING>;
@@ -423,6 +422,14 @@ __global__ void __launch_bounds__(NT) step_unsplit_kernel(StepArgs a)
         atomic_max_speed(a.smax + 2 * P.scen + 0, (double)mx);
         atomic_max_speed(a.smax + 2 * P.scen + 1, (double)my);
     }
+}
+
+template <typename T, bool PERT, int NT, int RING>
+__global__ void __launch_bounds__(NT) step_unsplit_kernel(StepArgs a)
+{
+    if (!launch_live(a)) return;
+    unsplit_item<T, PERT, NT, RING>(a);
+    step_tail<T, PERT>(a);
 }
 
 template <typename T, bool PERT, int NT>

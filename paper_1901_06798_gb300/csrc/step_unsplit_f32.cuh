@@ -52,8 +52,7 @@ template <int NT, int RING> struct UnsplitF32Smem {
     static constexpr int total = red + 2 * (NT / 32);
 };
 
-template <int NT, int RING>
-__global__ void __launch_bounds__(NT) step_unsplit_f32_kernel(StepArgs a)
+template <int NT, int RING> __device__ __forceinline__ void unsplit_f32_item(const StepArgs &a)
 {
     static_assert(RING >= 5, "rows r-2 .. r are read while rows r+1, r+2 are in flight");
     using T = float;
@@ -330,6 +329,13 @@ __global__ void __launch_bounds__(NT) step_unsplit_f32_kernel(StepArgs a)
         atomic_max_speed(a.smax + 2 * P.scen + 0, (double)mx);
         atomic_max_speed(a.smax + 2 * P.scen + 1, (double)my);
     }
+}
+
+template <int NT, int RING> __global__ void __launch_bounds__(NT) step_unsplit_f32_kernel(StepArgs a)
+{
+    if (!launch_live(a)) return;
+    unsplit_f32_item<NT, RING>(a);
+    step_tail<float, true>(a);
 }
 
 template <int NT>

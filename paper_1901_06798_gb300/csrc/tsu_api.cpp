@@ -373,7 +373,8 @@ struct tsu_ctx {
     DevBuf<float> dt1f;
     DevBuf<long long> viol, retakes;
     DevBuf<unsigned long long> smax;
-    DevBuf<int> derr, retake;
+    DevBuf<int> derr, retake, any_retake;
+    DevBuf<unsigned> tail_count;   // CTAs of a patch-update launch that are done (step_tail.cuh)
     std::vector<double> cells_h;
     std::vector<std::array<long long, kMaxLevels>> nsteps;
     bool initialized = false;
@@ -485,7 +486,6 @@ struct tsu_ctx {
         a.bulk_rows = bulk_rows;
         a.wait_polls = wait_polls;
     }
-    const int *retake_gate() const { return retake.p; }
     int seg() const { return seg_rows > 0 ? seg_rows : (prec == TSU_F64 ? 128 : 64); }
     // one launch of the patch update (a.gate set: the level-1 retake)
     int launch_step(const StepArgs &a, const Lvl &L)
@@ -789,10 +789,11 @@ struct tsu_ctx {
         hier_version++;   // the gauge kernel's pointers changed
     }
 
-    void sample_gauges()
+    // the end of a coarse step of a refined run (or of one driven level by level):
+    // t += dt^1 and the gauge samples
+    void end_step()
     {
-        int ng = (int)gxy.size() / 2;
-        if (!ng) return;
+        const int ng = (int)gxy.size() / 2;
         // room for this sample (a no-op inside a captured step: tsu_step made
         // room for all of its steps before capturing)
         ensure_samples(nsamp + 1);
@@ -805,8 +806,8 @@ struct tsu_ctx {
             ga.dxl[l] = lv[l].dx;
             ga.dyl[l] = lv[l].dy;
         }
-        kl(k_gauges(prec, ga, ctrl(), st), "gauges");
-        nsamp++;
+        kl(k_end_step(prec, ga, ctrl(), st), "end step");
+        if (ng) nsamp++;
     }
 
     // ------------------------------------------------------------ regrid
@@ -1134,7 +1135,7 @@ struct tsu_ctx {
             L.dList.upload(renewed, st, uring);
             kl(k_cell_speed(prec, view(lf), L.dList.p, (int)renewed.size(), L.maxcells, L.cur, c.g, c.drytol, smax.p, st),
                "cell speed");
-            kl(k_post_level(ctrl(), lf, nscen, L.R, pdx(lf), pdy(lf), c.cfl_max, c.cfl_desired, 1, st), "post rate");
+            kl(k_post_rate(ctrl(), lf, nscen, L.R, pdx(lf), pdy(lf), st), "post rate");
         }
         // release the replaced patches of the regridded scenarios
         for (size_t k = 0; k < oldP.size(); k++)
@@ -1151,68 +1152,95 @@ struct tsu_ctx {
     }
 
     // ------------------------------------------------------------ stepping
+    // launch arguments of the patch update of level l
+    StepArgs step_args(int l)
+    {
+        const Lvl &L = lv[l];
+        StepArgs a{};
+        a.descs = L.dP.p; a.items = L.dItems.p; a.arena = arena.base; a.cur = L.cur; a.dt1 = dt1.p;
+        a.smax = smax.p; a.R = L.R; a.g = c.g; a.drytol = c.drytol;
+        a.dt1f = dt1f.p;
+        a.transverse = c.transverse;
+        a.manning = (c.manning_n * c.manning_n) * c.g;
+        level_args(a, l);
+        set_f32_constants(a);
+        return a;
+    }
+    // The patch update of level l with what ends it (step_tail.cuh): the
+    // level's rate and CFL check and, with `ends` (one-level grids), the end of the
+    // coarse step.  Sec. 2.2 CFL condition: a level-1 step with nu > cfl_max is
+    // taken again with dt^1 = cfl_desired / rate before any finer level moves.  The
+    // decision stays on the device: the step's input buffer is untouched, and the
+    // retake launch runs only the work items of the scenarios that the check
+    // marked.  Returns the kernels launched.
+    int update_level(int l, bool ends)
+    {
+        Lvl &L = lv[l];
+        const bool retake_on = l == 0 && c.cfl_retake;
+        StepArgs a = step_args(l);
+        TailArgs &t_ = a.tail;
+        t_.cv = ctrl();
+        // (a finer level saves one launch by it, level 1 two)
+        const bool counted = (int)L.items.size() <= (l == 0 ? kTailMaxCtas : kTailMaxCtas / 4);
+        t_.count = counted ? tail_count.p : nullptr;
+        t_.any_retake = retake_on ? any_retake.p : nullptr;
+        t_.level = l; t_.nscen = nscen; t_.mode = retake_on ? 2 : 0; t_.end_step = ends ? 1 : 0;
+        t_.R = L.R; t_.dx = pdx(l); t_.dy = pdy(l); t_.cfl_max = c.cfl_max; t_.cfl_desired = c.cfl_desired;
+        const int ng = (int)gxy.size() / 2;
+        if (ends && ng) {
+            ensure_samples(nsamp + 1);   // (a no-op inside a captured step, as in end_step)
+            t_.ngauges = ng;
+            t_.gloc = dgloc.p; t_.gxy = dgxy.p; t_.geta = dgeta.p; t_.gt = dgt.p; t_.nsamp = dnsamp.p;
+            t_.x0 = c.x0; t_.y0 = c.y0; t_.gdx = L.dx; t_.gdy = L.dy;
+            nsamp++;
+        }
+        kl(launch_step(a, L), "patch step");
+        if (!counted) kl(k_tail(prec, a, st), "step tail");
+        if (!retake_on) return counted ? 1 : 2;
+        a.gate = retake.p;
+        t_.mode = 3;
+        t_.count = tail_count.p;   // (its CTAs reach the count only when there is something to retake)
+        kl(launch_step(a, L), "patch step (retake)");
+        return counted ? 2 : 3;
+    }
+
     // One step of level l alone (Sec. 3.1 step 1): ghost fill (time fraction
-    // k / r_{l-1} of the coarser level's step), physical boundaries, the patch
-    // update with the CFL check (and, on level 1, the retake), bookkeeping.
-    void level_step(int l, int k)
+    // k / r_{l-1} of the coarser level's step), physical boundaries (on level 1 with
+    // the start of the coarse step), the patch update with the CFL check and the
+    // retake.
+    void level_step(int l, int k, bool ends = false)
     {
         Lvl &L = lv[l];
         const int n = (int)L.P.size();
-        if (n > 0) {
-            if (l > 0 || n > 1) {
-                double alpha = l > 0 ? (double)k / (double)ratio[l - 1] : 0.0;
-                LevelView Cv = l > 0 ? view(l - 1) : view(l);
-                kl(k_ghost_fill(prec, view(l), Cv, n, L.maxring, L.cur, l > 0 ? lv[l - 1].cur : 0,
-                                l > 0 ? ratio[l - 1] : 0, alpha, c.drytol, derr.p, st), "ghost fill");
-                if (l > 0) launches++;   // the interpolated cells' kernel
-            }
-            if (!L.bclist.empty()) {
-                BcArgs ba{L.dBc.p, {c.bc[0], c.bc[1], c.bc[2], c.bc[3]}};
-                kl(k_bc(prec, view(l), ba, (int)L.bclist.size(), L.maxring, L.cur, 1, 0, st), "bc");
-            }
-            StepArgs a{};
-            a.descs = L.dP.p; a.items = L.dItems.p; a.arena = arena.base; a.cur = L.cur; a.dt1 = dt1.p;
-            a.smax = smax.p; a.R = L.R; a.g = c.g; a.drytol = c.drytol;
-            a.dt1f = dt1f.p;
-            a.transverse = c.transverse;
-            a.manning = (c.manning_n * c.manning_n) * c.g;
-            level_args(a, l);
-            set_f32_constants(a);
-            ProfStep ps{};
-            if (prof) {
-                ps.level = l;
-                ps.e0 = prof_event();
-                ps.e1 = prof_event();
-                for (int sc = 0; sc < nscen; sc++) ps.cells += cells_h[(size_t)sc * kMaxLevels + l];
-                ps.kernels = 1;
-                CK(cudaEventRecord(ps.e0, st));
-            }
-            kl(launch_step(a, L), "patch step");
-            // Sec. 2.2 CFL condition: a level-1 step with nu > cfl_max is taken
-            // again with dt^1 = cfl_desired / rate before any finer level moves.
-            // The decision stays on the device: the step's input buffer is
-            // untouched, and the retake launch runs only the work items of the
-            // scenarios whose post-level kernel set their gate.
-            const bool retake = l == 0 && c.cfl_retake;
-            // on a one-level grid the last post-level kernel also ends the coarse step
-            const bool ends = l == 0 && end_in_post_;
-            kl(k_post_level(ctrl(), l, nscen, L.R, pdx(l), pdy(l), c.cfl_max, c.cfl_desired, retake ? 2 : 0, st,
-                            ends && !retake ? 1 : 0),
-               "post step");
-            if (retake) {
-                a.gate = retake_gate();
-                kl(launch_step(a, L), "patch step (retake)");
-                kl(k_post_level(ctrl(), l, nscen, L.R, pdx(l), pdy(l), c.cfl_max, c.cfl_desired, 3, st, ends ? 1 : 0),
-                   "post step (retake)");
-                ps.kernels += 2;
-            }
-            if (ends) end_done_ = true;
-            if (prof) {
-                CK(cudaEventRecord(ps.e1, st));
-                prof_steps.push_back(ps);
-            }
-            L.cur ^= 1;
+        if (n == 0) return;
+        if (l > 0 || n > 1) {
+            double alpha = l > 0 ? (double)k / (double)ratio[l - 1] : 0.0;
+            LevelView Cv = l > 0 ? view(l - 1) : view(l);
+            kl(k_ghost_fill(prec, view(l), Cv, n, L.maxring, L.cur, l > 0 ? lv[l - 1].cur : 0,
+                            l > 0 ? ratio[l - 1] : 0, alpha, c.drytol, derr.p, st), "ghost fill");
+            if (l > 0) launches++;   // the interpolated cells' kernel
         }
+        if (!L.bclist.empty()) {   // never empty on level 1, which covers the domain
+            BcArgs ba{L.dBc.p, {c.bc[0], c.bc[1], c.bc[2], c.bc[3]}};
+            const CtrlView cv = ctrl();
+            const BeginArgs bg{nscen, nlev, Rl.p, c.cfl_desired, c.dt_max};
+            kl(k_bc(prec, view(l), ba, (int)L.bclist.size(), L.maxring, L.cur, 1, 0, st, l == 0 ? &cv : nullptr,
+                    l == 0 ? &bg : nullptr), "bc");
+        }
+        ProfStep ps{};
+        if (prof) {
+            ps.level = l;
+            ps.e0 = prof_event();
+            ps.e1 = prof_event();
+            for (int sc = 0; sc < nscen; sc++) ps.cells += cells_h[(size_t)sc * kMaxLevels + l];
+            CK(cudaEventRecord(ps.e0, st));
+        }
+        ps.kernels = update_level(l, ends);
+        if (prof) {
+            CK(cudaEventRecord(ps.e1, st));
+            prof_steps.push_back(ps);
+        }
+        L.cur ^= 1;
     }
 
     // What follows the r_l substeps of level l + 1 (or level l's own step when
@@ -1240,7 +1268,7 @@ struct tsu_ctx {
     // l + 1 (each with its own recursion), then the finish of level l.
     void advance(int l, int k)
     {
-        level_step(l, k);
+        level_step(l, k, nlev == 1);
         if (l + 1 < nlev && !lv[l + 1].P.empty())
             for (int kk = 0; kk < ratio[l]; kk++) advance(l + 1, kk);
         level_finish(l);
@@ -1264,18 +1292,11 @@ struct tsu_ctx {
         return false;
     }
 
-    // On a one-level grid the level-1 step's post-level kernel also ends the
-    // coarse step (t += dt), which saves a launch per step.
-    bool end_in_post_ = false, end_done_ = false;
+    // on a one-level grid the level-1 update also ends the coarse step
     void coarse_step()
     {
-        kl(k_begin_step(ctrl(), nscen, nlev, Rl.p, c.cfl_desired, c.dt_max, st), "begin step");
-        end_in_post_ = nlev == 1;
-        end_done_ = false;
         advance(0, 0);
-        end_in_post_ = false;
-        if (!end_done_) kl(k_end_step(ctrl(), nscen, st), "end step");
-        sample_gauges();
+        if (nlev > 1) end_step();
     }
 
     void step(int n)
@@ -1379,7 +1400,6 @@ struct tsu_ctx {
         if (l == 0) {
             if (!synchronised()) throw Err(TSU_ERR_ARG, "level 1 steps only between coarse steps");
             ensure_samples(nsamp + 2);
-            kl(k_begin_step(ctrl(), nscen, nlev, Rl.p, c.cfl_desired, c.dt_max, st), "begin step");
         } else {
             if (pend[l - 1] == 0) throw Err(TSU_ERR_ARG, "the coarser level has no substep of this level pending");
             if (pend[l] != 0) throw Err(TSU_ERR_ARG, "the finer level's substeps are still pending");
@@ -1393,8 +1413,7 @@ struct tsu_ctx {
         for (;;) {   // finish this level, and every coarser one whose last substep this was
             level_finish(l);
             if (l == 0) {
-                kl(k_end_step(ctrl(), nscen, st), "end step");
-                sample_gauges();
+                end_step();
                 return;
             }
             if (--pend[l - 1] > 0) return;
@@ -1555,7 +1574,7 @@ struct tsu_ctx {
         }
         kl(k_cell_speed(prec, view(0), L.dList.p, (int)all.size(), L.maxcells, L.cur, c.g, c.drytol, smax.p, st),
            "cell speed");
-        kl(k_post_level(ctrl(), 0, nscen, L.R, pdx(0), pdy(0), c.cfl_max, c.cfl_desired, 1, st), "post rate");
+        kl(k_post_rate(ctrl(), 0, nscen, L.R, pdx(0), pdy(0), st), "post rate");
         initialized = true;
         std::vector<int> everyone(nscen);
         for (int s = 0; s < nscen; s++) everyone[s] = s;
@@ -1776,7 +1795,7 @@ struct tsu_ctx {
         for (auto &g : grids) if (g.dev) cudaFreeAsync(g.dev, st);
         dGrids.release(); dGridScen.release(); dEtaIdx.release();
         dt1.release(); dt1f.release(); t.release(); rate.release(); cellupd.release(); cells.release(); Rl.release(); mass.release();
-        viol.release(); smax.release(); derr.release(); retake.release(); retakes.release(); dneg.release();
+        viol.release(); smax.release(); derr.release(); retake.release(); retakes.release(); any_retake.release(); tail_count.release(); dneg.release();
         tabI.release(); tabT.release(); tabIn.release();
         dgxy.release(); dgeta.release(); dgt.release(); dnsamp.release(); dgloc.release();
         fraw.release(); fcov.release(); ftmp.release(); fF.release(); fN.release(); fpack.release(); fslot.release(); fbox.release();
@@ -1892,7 +1911,9 @@ int tsu_create(const tsu_config *cfg, void *cuda_stream, tsu_ctx **out)
         x->dt1.ensure(S, st); x->dt1f.ensure(S, st); x->t.ensure(S, st); x->rate.ensure((size_t)S * kMaxLevels, st);
         x->cellupd.ensure(S, st); x->viol.ensure(S, st); x->smax.ensure(2 * (size_t)S, st);
         x->derr.ensure(1, st); x->mass.ensure(S, st); x->dnsamp.ensure(1, st);
-        x->retake.ensure(S, st); x->retakes.ensure(S, st);
+        x->retake.ensure(S, st); x->retakes.ensure(S, st); x->any_retake.ensure(1, st); x->tail_count.ensure(1, st);
+        CK(cudaMemsetAsync(x->any_retake.p, 0, sizeof(int), st));
+        CK(cudaMemsetAsync(x->tail_count.p, 0, sizeof(unsigned), st));
         CK(cudaMemsetAsync(x->retake.p, 0, S * sizeof(int), st));
         CK(cudaMemsetAsync(x->retakes.p, 0, S * sizeof(long long), st));
         CK(cudaMemsetAsync(x->dt1.p, 0, S * sizeof(double), st));
@@ -2308,14 +2329,9 @@ int tsu_autotune(tsu_ctx *ctx, int reps, int *best_threads, int *best_seg_rows, 
                     for (int l = 0; l < ctx->nlev; l++) {
                         Lvl &L = ctx->lv[l];
                         if (L.P.empty()) continue;
-                        StepArgs sa{};
-                        sa.descs = L.dP.p; sa.items = L.dItems.p; sa.arena = ctx->arena.base; sa.cur = L.cur;
-                        sa.dt1 = ctx->zero_dt.p; sa.dt1f = ctx->zero_dtf.p; sa.smax = ctx->smax.p; sa.R = L.R;
-                        sa.g = ctx->c.g; sa.drytol = ctx->c.drytol;
-                        sa.transverse = ctx->c.transverse;
-                        sa.manning = (ctx->c.manning_n * ctx->c.manning_n) * ctx->c.g;
-                        ctx->level_args(sa, l);
-                        set_f32_constants(sa);
+                        StepArgs sa = ctx->step_args(l);
+                        sa.dt1 = ctx->zero_dt.p;
+                        sa.dt1f = ctx->zero_dtf.p;
                         ctx->kl(ctx->launch_step(sa, L), "autotune step");
                     }
                 };
@@ -2461,46 +2477,21 @@ int tsu_time_level1_steps(tsu_ctx *ctx, int warmup, int n, double *kernel_ms_out
         Lvl &L = ctx->lv[0];
         CK(cudaEventRecord(ev[2 * n], ctx->st));
         for (int k = 0; k < n; k++) {
-            ctx->kl(k_begin_step(ctx->ctrl(), ctx->nscen, ctx->nlev, ctx->Rl.p, ctx->c.cfl_desired, ctx->c.dt_max, ctx->st),
-                    "begin step");
+            // the kernels of level_step and coarse_step, with an event on either side of
+            // the update (its retake launch included)
             if (L.P.size() > 1) {
                 ctx->kl(k_ghost_fill(ctx->prec, ctx->view(0), ctx->view(0), (int)L.P.size(), L.maxring, L.cur, 0, 0, 0.0,
                                      ctx->c.drytol, ctx->derr.p, ctx->st), "ghost fill");
             }
-            if (!L.bclist.empty()) {
-                BcArgs ba{L.dBc.p, {ctx->c.bc[0], ctx->c.bc[1], ctx->c.bc[2], ctx->c.bc[3]}};
-                ctx->kl(k_bc(ctx->prec, ctx->view(0), ba, (int)L.bclist.size(), L.maxring, L.cur, 1, 0, ctx->st), "bc");
-            }
-            StepArgs a{};
-            a.descs = L.dP.p; a.items = L.dItems.p; a.arena = ctx->arena.base; a.cur = L.cur; a.dt1 = ctx->dt1.p;
-            a.smax = ctx->smax.p; a.R = L.R; a.g = ctx->c.g; a.drytol = ctx->c.drytol;
-            a.dt1f = ctx->dt1f.p;
-            a.transverse = ctx->c.transverse;
-            a.manning = (ctx->c.manning_n * ctx->c.manning_n) * ctx->c.g;
-            ctx->level_args(a, 0);
-            set_f32_constants(a);
+            BcArgs ba{L.dBc.p, {ctx->c.bc[0], ctx->c.bc[1], ctx->c.bc[2], ctx->c.bc[3]}};
+            const CtrlView cv = ctx->ctrl();
+            const BeginArgs bg{ctx->nscen, ctx->nlev, ctx->Rl.p, ctx->c.cfl_desired, ctx->c.dt_max};
+            ctx->kl(k_bc(ctx->prec, ctx->view(0), ba, (int)L.bclist.size(), L.maxring, L.cur, 1, 0, ctx->st, &cv, &bg), "bc");
             CK(cudaEventRecord(ev[2 * k], ctx->st));
-            ctx->kl(ctx->launch_step(a, L), "patch step");
+            ctx->update_level(0, true);
             CK(cudaEventRecord(ev[2 * k + 1], ctx->st));
-            // the rest of the step exactly as level_step and coarse_step run it: with
-            // the CFL retake on, the post-level check, the retake launch (its CTAs
-            // exit unless their scenario is retaken) and the check after it, then
-            // the end of the coarse step; without it, the post-level kernel also ends
-            // the coarse step
-            const bool retake = ctx->c.cfl_retake != 0;
-            ctx->kl(k_post_level(ctx->ctrl(), 0, ctx->nscen, L.R, ctx->pdx(0), ctx->pdy(0), ctx->c.cfl_max,
-                                 ctx->c.cfl_desired, retake ? 2 : 0, ctx->st, retake ? 0 : 1),
-                    "post step");
-            if (retake) {
-                a.gate = ctx->retake_gate();
-                ctx->kl(ctx->launch_step(a, L), "patch step (retake)");
-                ctx->kl(k_post_level(ctx->ctrl(), 0, ctx->nscen, L.R, ctx->pdx(0), ctx->pdy(0), ctx->c.cfl_max,
-                                     ctx->c.cfl_desired, 3, ctx->st, 1),
-                        "post step (retake)");
-            }
             L.cur ^= 1;
             for (int s = 0; s < ctx->nscen; s++) ctx->nsteps[s][0]++;
-            ctx->sample_gauges();
         }
         CK(cudaEventRecord(ev[2 * n + 1], ctx->st));
         ctx->sync();

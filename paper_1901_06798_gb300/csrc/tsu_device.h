@@ -30,6 +30,46 @@ struct StepItem {
     int x0, y0, w, h;
 };
 
+// Device control block of a context: per scenario dt, time, rates, counters.
+struct CtrlView {
+    double *dt1, *t;
+    float *dt1f;                 // FP32 copy of dt1 for the perturbation-form kernel
+    double *rate;                // [scen][max_levels]
+    double *cell_updates;        // [scen]
+    const double *cells;         // [scen][max_levels] interior cells per level
+    long long *cfl_viol;         // [scen]
+    unsigned long long *smax;    // [scen][2]
+    int *retake;                 // [scen] 1: the level-1 step is being retaken (the step kernels' gate)
+    long long *retakes;          // [scen] level-1 steps retaken
+    int *err;                    // device error flag (TSU_DEV_ERR_*)
+    int max_levels;
+};
+
+struct GaugeLoc {
+    int level, patch;            // finest patch containing the gauge, or patch = -1
+};
+
+// What ends a level step (step_tail.cuh), done by the last CTA of the patch-update
+// launch unless count is null.  mode as post_level's; end_step: then t += dt^1 and the gauge samples
+// (one-level grids), unless a scenario is to be retaken.
+struct TailArgs {
+    CtrlView cv;
+    unsigned *count;             // CTAs done, zero between launches
+    int *any_retake;             // a scenario is marked for a retake (null: the step is never retaken)
+    int level, nscen, mode, end_step;
+    double R, dx, dy, cfl_max, cfl_desired;
+    int ngauges;
+    const GaugeLoc *gloc;        // [scen][gauge]
+    const double *gxy;
+    double *geta, *gt;
+    long long *nsamp;
+    double x0, y0, gdx, gdy;     // the level's origin and cell size in the gauges' coordinates
+};
+
+// the most CTAs of a launch that are counted: two waves of the FP32 split
+// update's (the launch saved, against the wait at the end of each wave)
+constexpr int kTailMaxCtas = 1216;
+
 struct StepArgs {
     const PatchDesc *descs;
     const StepItem *items;
@@ -64,6 +104,8 @@ struct StepArgs {
     int *err;
     int bulk_rows;
     unsigned wait_polls;
+    int n_items;                // work items (the FP32 split update's retake launch strides over them)
+    TailArgs tail;
 };
 
 // device error flag bits: 1, 2, 4 a ghost, coarse or parent cell without a
