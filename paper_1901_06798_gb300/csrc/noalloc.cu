@@ -8,14 +8,13 @@
 // behind its back, and latency-critical loops cannot afford a cudaMalloc that
 // may block or fail.  The context-based entry points allocate (the patch
 // arena, tables, flags); this one keeps its few bytes of scratch -- patch
-// descriptor, work items, boundary list, dt and the wave-speed accumulator --
+// descriptor, boundary list, dt and the wave-speed accumulator --
 // in one file-scope __device__ array instead.
 //
 // The scratch array is shared by every call in the process on a given GPU
 // and keeps the contents of the last call; each call rewrites all of it (and
 // clears the speed accumulator) before use.  Calls whose work overlaps on the
 // GPU (different streams, or different host threads) race on it.
-#include <algorithm>
 #include <cstdint>
 #include <cstring>
 #include <mutex>
@@ -29,15 +28,13 @@ namespace tsu {
 
 namespace {
 
-constexpr size_t kScratchBytes = 1u << 20;          // 1 MiB per GPU
+constexpr size_t kScratchBytes = 512;               // per GPU
 constexpr size_t kDescOff = 0;                      // PatchDesc
 constexpr size_t kListOff = 256;                    // int bclist[1]
 constexpr size_t kDtOff = 272;                      // double dt
 constexpr size_t kDtfOff = 280;                     // float dt
 constexpr size_t kSmaxOff = 288;                    // unsigned long long smax[2]
-constexpr size_t kItemsOff = 512;                   // StepItem items[]
-constexpr int kMaxItems = (int)((kScratchBytes - kItemsOff) / sizeof(StepItem));
-constexpr int kSegRows = 128;
+static_assert(sizeof(PatchDesc) <= kListOff, "the descriptor fits its slot");
 constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -64,31 +61,23 @@ cudaError_t scratch_for_current_device(void **out)
     return cudaSuccess;
 }
 
-__global__ void noalloc_prepare_kernel(unsigned char *scratch, long long fstride, int nx, int ny, int pitch,
-                                       double dt, int W, int nsx, int n)
+__global__ void noalloc_prepare_kernel(unsigned char *scratch, long long fstride, int nx, int ny, int pitch, double dt)
 {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        PatchDesc d;
-        memset(&d, 0, sizeof d);
-        d.off = 0;
-        d.fs = fstride;
-        d.i0 = 0; d.j0 = 0; d.nx = nx; d.ny = ny; d.pitch = pitch;
-        d.scen = 0;
-        d.bcmask = 15;
-        *reinterpret_cast<PatchDesc *>(scratch + kDescOff) = d;
-        *reinterpret_cast<int *>(scratch + kListOff) = 0;
-        *reinterpret_cast<double *>(scratch + kDtOff) = dt;
-        *reinterpret_cast<float *>(scratch + kDtfOff) = (float)dt;
-        unsigned long long *sm = reinterpret_cast<unsigned long long *>(scratch + kSmaxOff);
-        sm[0] = 0ull;
-        sm[1] = 0ull;
-    }
-    StepItem *items = reinterpret_cast<StepItem *>(scratch + kItemsOff);
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        int sx = k % nsx, sy = k / nsx;
-        int x0 = sx * W, y0 = sy * kSegRows;
-        items[k] = StepItem{0, x0, y0, min(W, nx - x0), min(kSegRows, ny - y0)};
-    }
+    if (threadIdx.x != 0) return;
+    PatchDesc d;
+    memset(&d, 0, sizeof d);
+    d.off = 0;
+    d.fs = fstride;
+    d.i0 = 0; d.j0 = 0; d.nx = nx; d.ny = ny; d.pitch = pitch;
+    d.scen = 0;
+    d.bcmask = 15;
+    *reinterpret_cast<PatchDesc *>(scratch + kDescOff) = d;
+    *reinterpret_cast<int *>(scratch + kListOff) = 0;
+    *reinterpret_cast<double *>(scratch + kDtOff) = dt;
+    *reinterpret_cast<float *>(scratch + kDtfOff) = (float)dt;
+    unsigned long long *sm = reinterpret_cast<unsigned long long *>(scratch + kSmaxOff);
+    sm[0] = 0ull;
+    sm[1] = 0ull;
 }
 
 }  // namespace
@@ -109,21 +98,18 @@ extern "C" int tsu_grid_step_noalloc(int precision, void *block, int nx, int ny,
         if (bc[k] != TSU_BC_WALL && bc[k] != TSU_BC_EXTRAP) return TSU_ERR_ARG;
     const size_t esz = precision == TSU_F64 ? 8 : 4;
     if (((uintptr_t)block) % esz) return TSU_ERR_ARG;
-    const int nt = precision == TSU_F64 ? step_threads_f64() : step_threads_f32p();
+    // tiles found from the CTA's index
+    const int nt = precision == TSU_F64 ? step_threads_f64(0) : step_threads_f32p();
     const int W = precision == TSU_F64 ? step_strip_width_f64(nt, 0) : step_strip_width_f32p(nt, 0);
-    // FP64: work items in the scratch; FP32: tiles found from the CTA's index
-    const int rows = precision == TSU_F64 ? kSegRows : tile_cut(ny, tile_rows_f32p(1, &nx, &ny, nt));
+    const int rows = tile_cut(ny, precision == TSU_F64 ? tile_rows_f64(1, &nx, &ny) : tile_rows_f32p(1, &nx, &ny, nt));
     const int nsx = (nx + W - 1) / W, nsy = (ny + rows - 1) / rows;
-    const int n_items = precision == TSU_F64 ? nsx * nsy : 0;
-    if (n_items > kMaxItems) return TSU_ERR_ARG;
 
     cudaStream_t st = (cudaStream_t)cuda_stream;
     void *sp = nullptr;
     if (scratch_for_current_device(&sp) != cudaSuccess) return TSU_ERR_CUDA;
     unsigned char *scratch = reinterpret_cast<unsigned char *>(sp);
 
-    int blocks = std::max(1, (n_items + 255) / 256);
-    noalloc_prepare_kernel<<<blocks, 256, 0, st>>>(scratch, field_stride, nx, ny, pitch, dt, W, nsx, n_items);
+    noalloc_prepare_kernel<<<1, 32, 0, st>>>(scratch, field_stride, nx, ny, pitch, dt);
     if (cudaGetLastError() != cudaSuccess) return TSU_ERR_CUDA;
 
     const PatchDesc *desc = reinterpret_cast<const PatchDesc *>(scratch + kDescOff);
@@ -138,7 +124,6 @@ extern "C" int tsu_grid_step_noalloc(int precision, void *block, int nx, int ny,
 
     StepArgs a{};
     a.descs = desc;
-    a.items = precision == TSU_F64 ? reinterpret_cast<const StepItem *>(scratch + kItemsOff) : nullptr;
     a.tile_rows = rows;
     a.tile_nsx = nsx;
     a.arena = block;

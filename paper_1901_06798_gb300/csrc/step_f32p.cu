@@ -89,6 +89,29 @@ int tile_rows_f32p(int n, const int *nx, const int *ny, int threads)
     return best;
 }
 
+// Rows of the unsplit kernels' row segments (strips of threads - 4 columns), each
+// of which sweeps 4 more and fills its pipeline.  FP32: about 16 warps run on an
+// SM, which share its issue slots as the tiles' do.  FP64: an SM's CTAs share its
+// FP64 pipe, so their times add up.
+int unsplit_rows(int n, const int *nx, const int *ny, int threads, int precision)
+{
+    static const int cand[] = {8, 12, 16, 24, 32, 48, 64};
+    const bool f64 = precision == 0;
+    const int W = threads - 4, occ = std::max(1, 512 / threads);
+    int best = f64 ? 128 : 64;
+    double bc = 1e300;
+    for (int R : cand) {
+        double items = 0.0;
+        for (int k = 0; k < n; k++) items += (double)((nx[k] + W - 1) / W) * ((ny[k] + R - 1) / R);
+        const double per = items / kSMs, full = std::floor(per / occ), rest = std::ceil(per - full * occ - 1e-9);
+        const double one = R + 6;
+        const double c = f64 ? std::ceil(per) * one
+                             : full * one * (1.0 + 0.4 * (occ - 1)) + (rest > 0 ? one * (1.0 + 0.4 * (rest - 1)) : 0.0);
+        if (c < bc) { bc = c; best = R; }
+    }
+    return best;
+}
+
 // threads per CTA: 32, 64, 128 or 256
 int launch_step_f32p(const StepArgs &a, int n_items, int threads, cudaStream_t st)
 {

@@ -1,36 +1,72 @@
-// step_f64.cu -- FP64 instantiation of the fused patch update.  Built with
-// --fmad=false so every multiply and add rounds exactly as the FP64 oracle's.
-#include "step_kernel.cuh"
+// step_f64.cu -- FP64 split update (step_tile_f64.cuh).  Built with --fmad=false so
+// every multiply and add rounds exactly as the FP64 oracle's.
+#include <algorithm>
+#include <cmath>
+#include "step_tile_f64.cuh"
 
 namespace tsu {
 
-static constexpr int kThreadsF64 = 64;
+namespace {
 
-int step_threads_f64() { return kThreadsF64; }
-int step_strip_width_f64(int threads, int) { return threads - 4; }
+constexpr int kThreadsF64 = 128, kThreadsUnsplitF64 = 64;
+constexpr int kSMs = 152;
+int tile_smem(int rows) { return (rows + 4) * d1::kRow * (int)sizeof(double); }
 
-// threads per CTA: 64, 128 or 256 (strip width threads - 4 columns)
+template <int NW, bool GEO> int launch_tile(const StepArgs &a, int n, cudaStream_t st)
+{
+    // above 48 KiB of dynamic shared memory a kernel has to be told so, once per device
+    static unsigned long long told = 0;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return (int)e;
+    if (dev >= 64 || !(told >> dev & 1)) {
+        e = cudaFuncSetAttribute(step_tile_f64<NW, GEO>, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_smem(kTileRowsMaxF64));
+        if (e != cudaSuccess) return (int)e;
+        if (dev < 64) told |= 1ull << dev;
+    }
+    step_tile_f64<NW, GEO><<<n, NW * 32, tile_smem(a.tile_rows), st>>>(a);
+    return (int)cudaGetLastError();
+}
+
+template <int NW> int launch_geo(const StepArgs &a, int n, cudaStream_t st)
+{
+    return a.kap != nullptr ? launch_tile<NW, true>(a, n, st) : launch_tile<NW, false>(a, n, st);
+}
+
+}  // namespace
+
+int step_threads_f64(int transverse) { return transverse ? kThreadsUnsplitF64 : kThreadsF64; }
+int step_strip_width_f64(int threads, int transverse) { return transverse ? threads - 4 : d1::kCols; }
+
+// The tile height with the least FP64 work on the busiest SM.  A tile of R rows
+// costs about 2 (R + 4) warp rows of x sweep and 2 (R / 2 + 3) of y march on each
+// half of its columns (two segments); an SM's tiles share its FP64 pipe, so they
+// add up however many run at once.  At most 32 rows: three CTAs then fit on an SM.
+int tile_rows_f64(int n, const int *nx, const int *ny)
+{
+    int best = 32;
+    double bc = 1e300;
+    for (int R = 32; R >= 4; R -= 2) {
+        double items = 0.0;
+        for (int k = 0; k < n; k++) items += (double)((nx[k] + d1::kCols - 1) / d1::kCols) * ((ny[k] + R - 1) / R);
+        const double c = std::ceil(items / kSMs) * (2.0 * (R + 4) + 4.0 * (R / 2 + 3));
+        if (c < bc) { bc = c; best = R; }
+    }
+    return best;
+}
+
+// threads per CTA: 64, 128 or 256
 int launch_step_f64(const StepArgs &a, int n_items, int threads, cudaStream_t st)
 {
     if (n_items <= 0) return 0;
     if (a.transverse) return launch_unsplit_f64(a, n_items, threads, st);
-    const bool geo = a.kap != nullptr;   // latitude-longitude grid (capacity form)
+    if (a.tile_rows < 1 || a.tile_rows > kTileRowsMaxF64) return (int)cudaErrorInvalidValue;
     switch (threads) {
-    case 64:
-        if (geo) step_kernel<double, false, 64, 4, true><<<n_items, 64, 0, st>>>(a);
-        else step_kernel<double, false, 64, 4><<<n_items, 64, 0, st>>>(a);
-        break;
-    case 128:
-        if (geo) step_kernel<double, false, 128, 4, true><<<n_items, 128, 0, st>>>(a);
-        else step_kernel<double, false, 128, 4><<<n_items, 128, 0, st>>>(a);
-        break;
-    case 256:
-        if (geo) step_kernel<double, false, 256, 4, true><<<n_items, 256, 0, st>>>(a);
-        else step_kernel<double, false, 256, 4><<<n_items, 256, 0, st>>>(a);
-        break;
+    case 64: return launch_geo<2>(a, n_items, st);
+    case 128: return launch_geo<4>(a, n_items, st);
+    case 256: return launch_geo<8>(a, n_items, st);
     default: return (int)cudaErrorInvalidValue;
     }
-    return (int)cudaGetLastError();
 }
 
 }  // namespace tsu

@@ -1,33 +1,8 @@
-// step_kernel.cuh -- one dimensionally split wave-propagation step of every
-// patch of a level in one launch (Sec. 2.2 Eqs. wave_propagation_2nd_order_x
-// then _y), with the per-patch CFL wave-speed reduction fused in.
-//
-// Per CTA: a strip of W = NT - 4 columns of one patch and a segment of rows.
-// The CTA streams down the rows:
-//   * row r (W + 4 cells of q0, q1, q2, B) is prefetched into a ring of
-//     shared-memory slots with cp.async, RING - 1 rows ahead, so every
-//     state value is read from HBM once (plus the 4-row / 4-column halo);
-//   * x sweep of row r: thread t solves the Riemann problem of x-edge t
-//     (between ring cells t and t+1) and publishes its f-waves; after a
-//     barrier it limits them with the upwind neighbour's waves (Eq. theta,
-//     MC limiter), publishes A+dQ and the correction flux, and after a second
-//     barrier updates cell t from its own A-dQ / correction (registers) and
-//     its left neighbour's A+dQ / correction (shared memory) -- the
-//     edge-then-cell thread mapping of Sec. 4.3.3, no redundant solves;
-//   * the same thread owns column t for the y sweep: Q* of rows r-2 .. r and
-//     the y-edge waves of rows r-2 .. r stay in its registers, so the y sweep
-//     needs neither shared memory nor barriers and Q* never goes to HBM --
-//     the x and y sweeps are fused in one kernel;
-//   * the max |s| of the edges touching interior cells is reduced with warp
-//     shuffles, then one atomicMax per CTA (Sec. 4.3 reduction).
-// GEO: latitude-longitude grid in capacity form (Sec. 2.1 spherical
-// coordinates; LeVeque's capacity-form wave propagation): row j has capacity
-// kap_j, the latitude edge below it the relative length ced_j.  The x sweep of
-// row j runs with dt / (kap_j dx) and reports speeds / kap_j; each y-edge's
-// fluctuations and correction flux are weighted by ced_e, its Courant number
-// uses dt ced_e / (kbar_e dy) (kbar_e the mean capacity of its two cells), the
-// cell update divides by kap_j, and the mass gets the term
-// (ced_{j+1} - ced_j) hv_j of the varying edge length.
+// step_kernel.cuh -- device functions of the patch update shared by its kernels:
+// the normal Riemann solver with bed steps, dry states and walls, the MC-limited
+// fluctuations and correction fluxes (Sec. 2.2 Eqs. wave_propagation_2nd_order,
+// theta), wet/dry post-processing, Manning friction, and the copies into shared
+// memory.
 // The arithmetic of riemann()/limit() follows the FP64 oracle operation by
 // operation; the FP64 instantiation is compiled without contraction so the
 // two agree to the last bit.
@@ -310,238 +285,6 @@ constexpr unsigned kDrainPolls = 1u << 26;
 __device__ __forceinline__ void atomic_max_speed(unsigned long long *dst, double v)
 {
     atomicMax(dst, (unsigned long long)__double_as_longlong(v));
-}
-
-template <typename T> __device__ __forceinline__ const T *geo_table(const double *d, const float *f);
-template <> __device__ __forceinline__ const double *geo_table<double>(const double *d, const float *) { return d; }
-template <> __device__ __forceinline__ const float *geo_table<float>(const double *, const float *f) { return f; }
-
-template <typename T, bool PERT, int NT, int RING, bool GEO> __device__ __forceinline__ void step_item(const StepArgs &a)
-{
-    static_assert(RING >= 3, "the derived values of row k+1 need its copy complete at iteration k");
-    __shared__ T ring[RING][4][NT];
-    __shared__ T sZ[9][NT];
-    __shared__ T sAp[3][NT];
-    __shared__ T sF[3][NT];
-    __shared__ T sD[2][4][NT];     // derived u, v, c, sqrt(h) of the ring cells, by row parity
-    __shared__ T red[2][NT / 32];
-
-    const StepItem it = a.items[blockIdx.x];
-    if (it.w > NT - 4 || it.w < 1 || it.h < 1) return;   // not a work item of this launch shape
-    const PatchDesc P = a.descs[it.patch];
-    if (a.gate != nullptr && a.gate[P.scen] == 0) return;   // not retaken (uniform over the CTA)
-    const int t = threadIdx.x;
-    const int cur = a.cur;
-    T *base = reinterpret_cast<T *>(a.arena) + P.off;
-    const T *qin0 = base + (long long)(cur * 3 + 0) * P.fs;
-    const T *qin1 = base + (long long)(cur * 3 + 1) * P.fs;
-    const T *qin2 = base + (long long)(cur * 3 + 2) * P.fs;
-    const T *Bg = base + 6LL * P.fs;
-    T *qo0 = base + (long long)((1 - cur) * 3 + 0) * P.fs;
-    T *qo1 = base + (long long)((1 - cur) * 3 + 1) * P.fs;
-    T *qo2 = base + (long long)((1 - cur) * 3 + 2) * P.fs;
-
-    const double dt = a.dt1[P.scen] / a.R;
-    const T dtdx = (T)(dt / a.dx), dtdy = (T)(dt / a.dy);
-    const T g = (T)a.g, drytol = (T)a.drytol;
-    const int x0 = it.x0, y0 = it.y0, w = it.w, h = it.h;
-    const int pitch = P.pitch;
-    const int nrows = h + 4;
-    // capacity of patch row j at kapP[j], relative length of the y-edge below it at cedP[j]
-    const T *kapP = GEO ? geo_table<T>(a.kap, a.kapf) + (P.j0 + 2) : nullptr;
-    const T *cedP = GEO ? geo_table<T>(a.ced, a.cedf) + (P.j0 + 2) : nullptr;
-    // ring cell t <-> patch column x0 - 2 + t (storage column x0 + t)
-    const bool loader = t < w + 4;
-    const long long colofs = (long long)(x0 + t);
-
-    auto prefetch = [&](int k) {
-        if (k < nrows && loader) {
-            int slot = k % RING;
-            long long gi = (long long)(y0 + k) * pitch + colofs;  // storage row (y0 - 2 + k) + 2
-            cp_async_elem(&ring[slot][0][t], qin0 + gi, sizeof(T));
-            cp_async_elem(&ring[slot][1][t], qin1 + gi, sizeof(T));
-            cp_async_elem(&ring[slot][2][t], qin2 + gi, sizeof(T));
-            cp_async_elem(&ring[slot][3][t], Bg + gi, sizeof(T));
-        }
-        cp_async_commit();
-    };
-    // own ring cell of row k (x-sweep roles: normal hu, transverse hv), derived
-    // and published for the left neighbour's edge
-    auto own_cell = [&](int k, Cell<T> &z) {
-        const int slot = k % RING;
-        z.q0 = ring[slot][0][t]; z.hn = ring[slot][1][t]; z.ht = ring[slot][2][t]; z.B = ring[slot][3][t];
-        derive<T, PERT>(z, g, drytol);
-        sD[k & 1][0][t] = z.u; sD[k & 1][1][t] = z.v; sD[k & 1][2][t] = z.c; sD[k & 1][3][t] = z.sq;
-    };
-
-#pragma unroll
-    for (int k = 0; k < RING - 1; k++) prefetch(k);
-    Cell<T> xc;   // this thread's ring cell of the current row
-    cp_async_wait<RING - 2>();
-    if (loader) own_cell(0, xc);
-
-    // y-sweep state of column t (valid for update threads 2 <= t < w + 2)
-    Cell<T> ym1;                 // Q* of row r-1 with derived values (y roles)
-    T qm2[3], Bm2 = T(0);
-    Wave<T> yold, ymid;
-    T yap[3] = {T(0), T(0), T(0)}, yF[3] = {T(0), T(0), T(0)};
-    T smx = T(0), smy = T(0);
-    const bool upd = t >= 2 && t < w + 2;
-    const bool rsolve = t < w + 3;
-    const bool lim = t >= 1 && t < w + 2;
-
-    for (int k = 0; k < nrows; k++) {
-        prefetch(k + RING - 1);
-        cp_async_wait<RING - 2>();   // rows <= k+1 of this thread have landed
-        __syncthreads();
-        const int slot = k % RING;
-        const int r = y0 - 2 + k;            // patch-local row of this iteration
-        const bool rowint = r >= y0 && r < y0 + h;
-        const T kr = GEO ? kapP[r] : T(1);
-        const T dtdxr = GEO ? (T)(dt / (kr * a.dx)) : dtdx;
-
-        // ---- x sweep: Riemann problem at edge t (ring cells t, t+1)
-        Wave<T> xw;
-        if (rsolve) {
-            Cell<T> xr;
-            xr.q0 = ring[slot][0][t + 1]; xr.hn = ring[slot][1][t + 1]; xr.ht = ring[slot][2][t + 1];
-            xr.B = ring[slot][3][t + 1];
-            xr.h = PERT ? xr.q0 - xr.B : xr.q0;
-            xr.wet = xr.h >= drytol;
-            xr.u = sD[k & 1][0][t + 1]; xr.v = sD[k & 1][1][t + 1]; xr.c = sD[k & 1][2][t + 1];
-            xr.sq = sD[k & 1][3][t + 1];
-            riemann<T, PERT>(g, xc, xr, xw);
-#pragma unroll
-            for (int p = 0; p < 3; p++)
-#pragma unroll
-                for (int m = 0; m < 3; m++) sZ[p * 3 + m][t] = xw.Z[p][m];
-        }
-        __syncthreads();
-
-        T xam[3], xap[3], xF[3];
-        if (lim) {
-            T ZI[3][3];
-#pragma unroll
-            for (int p = 0; p < 3; p++) {
-                int nb = xw.s[p] >= T(0) ? t - 1 : t + 1;
-#pragma unroll
-                for (int m = 0; m < 3; m++) ZI[p][m] = sZ[p * 3 + m][nb];
-            }
-            limit<T>(xw, ZI, dtdxr, xam, xap, xF);
-#pragma unroll
-            for (int m = 0; m < 3; m++) { sAp[m][t] = xap[m]; sF[m][t] = xF[m]; }
-            if (rowint) {
-                const T se = dmax<T>(-xw.s[0], xw.s[2]);
-                smx = dmax<T>(smx, GEO ? se / kr : se);
-            }
-        }
-        __syncthreads();
-
-        if (upd) {
-            // cell t: left edge t-1 (shared memory), right edge t (registers)
-            T qs[3] = {xc.q0, xc.hn, xc.ht};
-#pragma unroll
-            for (int m = 0; m < 3; m++) {
-                T u = (sAp[m][t - 1] + xam[m]) + (xF[m] - sF[m][t - 1]);
-                qs[m] = qs[m] - dtdxr * u;
-            }
-            postprocess<T, PERT>(qs[0], qs[1], qs[2], xc.B, drytol);
-
-            // ---- y sweep of column t: y-edge between rows r-1 and r
-            Cell<T> yc;
-            yc.q0 = qs[0]; yc.hn = qs[2]; yc.ht = qs[1]; yc.B = xc.B;
-            derive<T, PERT>(yc, g, drytol);
-            if (k >= 1) {
-                Wave<T> ynew;
-                riemann<T, PERT>(g, ym1, yc, ynew);
-                if (k >= 3) {
-                    // limit y-edge r-1 (ymid) with neighbours r-2 (yold) and r (ynew)
-                    const int e = r - 1;
-                    if (e >= y0 && e <= y0 + h) {
-                        T ZI[3][3];
-#pragma unroll
-                        for (int p = 0; p < 3; p++)
-#pragma unroll
-                            for (int m = 0; m < 3; m++) ZI[p][m] = ymid.s[p] >= T(0) ? yold.Z[p][m] : ynew.Z[p][m];
-                        T yam[3], yapn[3], yFn[3];
-                        T dtdye = dtdy, cratio = T(1);
-                        if (GEO) {
-                            const T kbar = T(0.5) * (kapP[e - 1] + kapP[e]);
-                            dtdye = ((T)dt * cedP[e]) / (kbar * (T)a.dy);
-                            cratio = cedP[e] / kbar;
-                        }
-                        limit<T>(ymid, ZI, dtdye, yam, yapn, yFn);
-                        const T se = dmax<T>(-ymid.s[0], ymid.s[2]);
-                        smy = dmax<T>(smy, GEO ? se * cratio : se);
-                        const int rc = r - 2;   // cell between y-edges r-2 and r-1
-                        if (rc >= y0 && rc < y0 + h) {
-                            T qn[3] = {qm2[0], qm2[2], qm2[1]};   // (mass, normal = hv, transverse = hu)
-                            if (GEO) {
-                                const T clo = cedP[rc], chi = cedP[e];
-                                const T dtk = (T)dt / (kapP[rc] * (T)a.dy);
-                                const T hv = qm2[2];
-#pragma unroll
-                                for (int m = 0; m < 3; m++) {
-                                    T u = (clo * yap[m] + chi * yam[m]) + (chi * yFn[m] - clo * yF[m]);
-                                    if (m == 0) u = u + (chi - clo) * hv;
-                                    qn[m] = qn[m] - dtk * u;
-                                }
-                            } else {
-#pragma unroll
-                                for (int m = 0; m < 3; m++) {
-                                    T u = (yap[m] + yam[m]) + (yFn[m] - yF[m]);
-                                    qn[m] = qn[m] - dtdy * u;
-                                }
-                            }
-                            postprocess<T, PERT>(qn[0], qn[1], qn[2], Bm2, drytol);
-                            if (a.manning > 0.0)   // y frame: qn[2] = hu, qn[1] = hv
-                                friction<T, PERT>(qn[0], qn[2], qn[1], Bm2, drytol, (T)a.manning, (T)dt);
-                            // a depth that is not a finite number reaches the host as an infinite speed
-                            if (!(dabs<T>(qn[0]) < T(1e30))) smy = T(INFINITY);
-                            long long gi = (long long)(rc + 2) * pitch + (x0 + t);
-                            qo0[gi] = qn[0];
-                            qo2[gi] = qn[1];
-                            qo1[gi] = qn[2];
-                        }
-#pragma unroll
-                        for (int m = 0; m < 3; m++) { yap[m] = yapn[m]; yF[m] = yFn[m]; }
-                    }
-                }
-                yold = ymid;
-                ymid = ynew;
-            }
-            qm2[0] = ym1.q0; qm2[1] = ym1.ht; qm2[2] = ym1.hn;
-            Bm2 = ym1.B;
-            ym1 = yc;
-        }
-        // derived values of this thread's cell in the next row (its own copy has landed)
-        if (loader && k + 1 < nrows) own_cell(k + 1, xc);
-    }
-
-    // CTA max of the wave speeds: warp shuffles, then one atomic per CTA
-    if (!(smx > T(0))) smx = T(0);
-    if (!(smy > T(0))) smy = T(0);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        smx = dmax<T>(smx, __shfl_xor_sync(0xffffffffu, smx, o));
-        smy = dmax<T>(smy, __shfl_xor_sync(0xffffffffu, smy, o));
-    }
-    if ((t & 31) == 0) { red[0][t >> 5] = smx; red[1][t >> 5] = smy; }
-    __syncthreads();
-    if (t == 0) {
-        T mx = T(0), my = T(0);
-        for (int k = 0; k < NT / 32; k++) { mx = dmax<T>(mx, red[0][k]); my = dmax<T>(my, red[1][k]); }
-        atomic_max_speed(a.smax + 2 * P.scen + 0, (double)mx);
-        atomic_max_speed(a.smax + 2 * P.scen + 1, (double)my);
-    }
-}
-
-template <typename T, bool PERT, int NT, int RING, bool GEO = false>
-__global__ void __launch_bounds__(NT) step_kernel(StepArgs a)
-{
-    if (!launch_live(a)) return;
-    step_item<T, PERT, NT, RING, GEO>(a);
-    step_tail<T, PERT>(a);
 }
 
 }  // namespace tsu

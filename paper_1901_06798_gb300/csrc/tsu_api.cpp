@@ -326,7 +326,7 @@ struct Lvl {
     std::vector<PatchDesc> P;
     std::vector<size_t> blk, blkbytes;
     std::vector<StepItem> items;   // patch update work items
-    int tile_rows = 0;             // FP32 split update: most rows of an item
+    int tile_rows = 0;             // most rows of an item
     std::vector<int> nbrs, bclist, olds;
     std::vector<BoxIndex> idx;   // per scenario spatial index of P, rebuilt by every finish_level of the level
     std::vector<int> ccand;   // coarse patches overlapping each patch's coarse-map footprint
@@ -462,12 +462,11 @@ struct tsu_ctx {
     int device = 0;                            // the CUDA device current at tsu_create
 
     // ------------------------------------------------------------ helpers
-    // FP32 split scheme: the patch update runs on tiles (step_tile_f32.cuh)
     bool split_f32() const { return prec != TSU_F64 && c.transverse == 0; }
     int nt() const
     {
         if (step_nt > 0) return step_nt;
-        return prec == TSU_F64 ? step_threads_f64() : step_threads_f32p();
+        return prec == TSU_F64 ? step_threads_f64(c.transverse) : step_threads_f32p();
     }
     // physical cell sizes of level l (of an equatorial cell on latitude-longitude grids)
     double pdx(int l) const { return c.spherical ? lv[l].dxp : lv[l].dx; }
@@ -486,7 +485,6 @@ struct tsu_ctx {
         a.bulk_rows = bulk_rows;
         a.wait_polls = wait_polls;
     }
-    int seg() const { return seg_rows > 0 ? seg_rows : (prec == TSU_F64 ? 128 : 64); }
     // one launch of the patch update (a.gate set: the level-1 retake)
     int launch_step(const StepArgs &a, const Lvl &L)
     {
@@ -598,7 +596,7 @@ struct tsu_ctx {
         L.maxring = 0;
         L.maxcells = 0;
         const int W = prec == TSU_F64 ? step_strip_width_f64(nt(), c.transverse) : step_strip_width_f32p(nt(), c.transverse);
-        const bool split = split_f32();
+        const bool split = c.transverse == 0;
         for (int k = 0; k < n; k++) {
             PatchDesc &p = L.P[k];
             L.maxring = std::max(L.maxring, (p.nx + 4) * (p.ny + 4) - p.nx * p.ny);
@@ -608,23 +606,25 @@ struct tsu_ctx {
         // work items of the patch update in patch order, built in patch ranges on
         // host threads and joined in range order
         {
-            // FP32 split update: tiles of equal heights within a patch
-            if (split) {
-                if (seg_rows > 0) {
-                    L.tile_rows = std::min(seg_rows, kTileRowsMax);
-                } else {
-                    std::vector<int> px(n), py(n);
-                    for (int k = 0; k < n; k++) { px[k] = L.P[k].nx; py[k] = L.P[k].ny; }
-                    L.tile_rows = tile_rows_f32p(n, px.data(), py.data(), nt());
-                }
+            // split update: tiles of equal heights within a patch; unsplit: row segments
+            // (seg_rows caps them; it sets them in the FP32 split update, whose issue-bound
+            // tiles can be worth other heights than the rule's)
+            if (seg_rows > 0 && split_f32()) {
+                L.tile_rows = std::min(seg_rows, kTileRowsMax);
+            } else {
+                std::vector<int> px(n), py(n);
+                for (int k = 0; k < n; k++) { px[k] = L.P[k].nx; py[k] = L.P[k].ny; }
+                L.tile_rows = !split ? unsplit_rows(n, px.data(), py.data(), nt(), prec)
+                                     : (prec == TSU_F64 ? tile_rows_f64(n, px.data(), py.data())
+                                                        : tile_rows_f32p(n, px.data(), py.data(), nt()));
+                if (seg_rows > 0) L.tile_rows = std::min(L.tile_rows, seg_rows);
             }
-            const int sg = seg();
             std::vector<std::vector<StepItem>> xi(16);
             parallel_ranges(n, [&](int q, int b, int e) {
                 std::vector<StepItem> &ox = xi[q];
                 for (int k = b; k < e; k++) {
                     const PatchDesc &p = L.P[k];
-                    const int sk = split ? tile_cut(p.ny, L.tile_rows) : sg;
+                    const int sk = split ? tile_cut(p.ny, L.tile_rows) : L.tile_rows;
                     for (int x0 = 0; x0 < p.nx; x0 += W)
                         for (int y0 = 0; y0 < p.ny; y0 += sk)
                             ox.push_back(StepItem{k, x0, y0, std::min(W, p.nx - x0), std::min(sk, p.ny - y0)});
@@ -2308,42 +2308,43 @@ int tsu_autotune(tsu_ctx *ctx, int reps, int *best_threads, int *best_seg_rows, 
         ctx->zero_dtf.ensure(ctx->nscen, ctx->st);
         CK(cudaMemsetAsync(ctx->zero_dt.p, 0, ctx->nscen * sizeof(double), ctx->st));
         CK(cudaMemsetAsync(ctx->zero_dtf.p, 0, ctx->nscen * sizeof(float), ctx->st));
-        // threads x rows per work item; the FP32 split update also takes 32 threads,
-        // and its items are tiles held in shared memory: shorter ones
+        // threads x rows per work item; the FP32 split update's items are tiles held
+        // in shared memory: shorter ones, and also by 32 threads
         const bool split = ctx->split_f32();
         const int nts[4] = {64, 128, 256, 32};
-        const int segs[4] = {split ? 16 : 32, split ? 30 : 64, split ? 44 : 128, split ? 60 : 256};
+        const int segs[4] = {split ? 16 : 32, split ? 32 : 64, split ? 64 : 128, split ? 128 : 256};
         const int n_nt = split ? 4 : 3;
         cudaEvent_t e0, e1;
         CK(cudaEventCreate(&e0));
         CK(cudaEventCreate(&e1));
         double best = 1e30;
         int bt = 0, bs = 0;
-        for (int a = 0; a < n_nt; a++)
-            for (int b = 0; b < 4; b++) {
-                ctx->step_nt = nts[a];
-                ctx->seg_rows = segs[b];
-                for (int l = 0; l < ctx->nlev; l++)
-                    if (!ctx->lv[l].P.empty()) ctx->finish_level(l);
-                auto run = [&] {
-                    for (int l = 0; l < ctx->nlev; l++) {
-                        Lvl &L = ctx->lv[l];
-                        if (L.P.empty()) continue;
-                        StepArgs sa = ctx->step_args(l);
-                        sa.dt1 = ctx->zero_dt.p;
-                        sa.dt1f = ctx->zero_dtf.p;
-                        ctx->kl(ctx->launch_step(sa, L), "autotune step");
-                    }
-                };
-                run();
-                CK(cudaEventRecord(e0, ctx->st));
-                for (int k = 0; k < reps; k++) run();
-                CK(cudaEventRecord(e1, ctx->st));
-                CK(cudaEventSynchronize(e1));
-                float ms = 0;
-                CK(cudaEventElapsedTime(&ms, e0, e1));
-                if (ms / reps < best) { best = ms / reps; bt = nts[a]; bs = segs[b]; }
-            }
+        // (the FP32 split update's own choice, 0 x 0, comes last)
+        const int n_shapes = 4 * n_nt + (split ? 1 : 0);
+        for (int q = 0; q < n_shapes; q++) {
+            ctx->step_nt = q < 4 * n_nt ? nts[q / 4] : 0;
+            ctx->seg_rows = q < 4 * n_nt ? segs[q % 4] : 0;
+            for (int l = 0; l < ctx->nlev; l++)
+                if (!ctx->lv[l].P.empty()) ctx->finish_level(l);
+            auto run = [&] {
+                for (int l = 0; l < ctx->nlev; l++) {
+                    Lvl &L = ctx->lv[l];
+                    if (L.P.empty()) continue;
+                    StepArgs sa = ctx->step_args(l);
+                    sa.dt1 = ctx->zero_dt.p;
+                    sa.dt1f = ctx->zero_dtf.p;
+                    ctx->kl(ctx->launch_step(sa, L), "autotune step");
+                }
+            };
+            run();
+            CK(cudaEventRecord(e0, ctx->st));
+            for (int k = 0; k < reps; k++) run();
+            CK(cudaEventRecord(e1, ctx->st));
+            CK(cudaEventSynchronize(e1));
+            float ms = 0;
+            CK(cudaEventElapsedTime(&ms, e0, e1));
+            if (ms / reps < best) { best = ms / reps; bt = ctx->step_nt; bs = ctx->seg_rows; }
+        }
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         CK(cudaMemsetAsync(ctx->smax.p, 0, 2 * ctx->nscen * sizeof(unsigned long long), ctx->st));
@@ -2352,8 +2353,8 @@ int tsu_autotune(tsu_ctx *ctx, int reps, int *best_threads, int *best_seg_rows, 
         for (int l = 0; l < ctx->nlev; l++)
             if (!ctx->lv[l].P.empty()) ctx->finish_level(l);
         ctx->sync();
-        if (best_threads) *best_threads = bt;
-        if (best_seg_rows) *best_seg_rows = bs;
+        if (best_threads) *best_threads = ctx->nt();
+        if (best_seg_rows) *best_seg_rows = bs > 0 ? bs : ctx->lv[0].tile_rows;
         if (best_ms) *best_ms = best;
     });
 }

@@ -92,7 +92,7 @@ struct StepArgs {
     // length of the latitude edge below row J at ced[J + 2]; null on Cartesian grids
     const double *kap, *ced;
     const float *kapf, *cedf;
-    // FP32 split update (step_tile_f32.cuh): the most rows of a work item, and,
+    // split update (step_tile_f32.cuh, step_tile_f64.cuh): the most rows of a work item, and,
     // with null items, the tile columns of the one patch the launch covers
     int tile_rows, tile_nsx;
     // CFL retake of a level-1 step: when set, a work item of scenario s runs
@@ -130,21 +130,24 @@ int launch_step_f64(const StepArgs &a, int n_items, int threads, cudaStream_t st
 int launch_step_f32p(const StepArgs &a, int n_items, int threads, cudaStream_t st);
 int launch_unsplit_f64(const StepArgs &a, int n_items, int threads, cudaStream_t st);
 int launch_unsplit_f32p(const StepArgs &a, int n_items, int threads, cudaStream_t st);
-int step_threads_f64();
+int step_threads_f64(int transverse);
 int step_threads_f32p();
 // columns one work item of the patch update covers, for a launch of `threads`
 // per CTA (the unsplit kernels take one column per thread in both precisions)
 int step_strip_width_f64(int threads, int transverse);
 int step_strip_width_f32p(int threads, int transverse);
-// FP32 split update: rows of a tile for n patches of nx[k] x ny[k] cells
-// advanced together by CTAs of `threads`, and rows of a patch's tiles (of at most
+// Split update: rows of a tile for n patches of nx[k] x ny[k] cells advanced
+// together (FP32: by CTAs of `threads`), and rows of a patch's tiles (of at most
 // `cap` rows): equal and even
 int tile_rows_f32p(int n, const int *nx, const int *ny, int threads);
+int tile_rows_f64(int n, const int *nx, const int *ny);
 inline int tile_cut(int ny, int cap)
 {
     const int nt = (ny + cap - 1) / cap, r = (ny + nt - 1) / nt;
     return r + (r & 1) <= cap ? r + (r & 1) : r;
 }
-constexpr int kTileRowsMax = 124;   // a tile row takes 1 KiB of shared memory
+constexpr int kTileRowsMax = 124, kTileRowsMaxF64 = 104;   // a tile row takes 1 KiB (FP64: 2 KiB) of shared memory
+// unsplit update: rows of its row segments, by the same reasoning
+int unsplit_rows(int n, const int *nx, const int *ny, int threads, int precision);
 
 }  // namespace tsu
