@@ -9,6 +9,7 @@
 //
 // Flat parameter vector: for each layer, W (C_out, C_in, k, k) then b (C_out);
 // layers (5->16, 3x3), (16->16, 3x3), (16->16, 3x3), (16->1, 1x1).
+#include <algorithm>
 #include <cstdint>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -33,147 +34,262 @@ __host__ __device__ inline LayerSpec layer_spec(int l)
     return s;
 }
 
-// y[n, o, i, j] = b[o] + sum_c sum_taps w[o, c, di, dj] x[n, c, i+di-1, j+dj-1]; one thread per output
-// pixel computes all C_out channels.  TIN: float or __half storage.
-template <typename TIN, typename TOUT, int CIN, int COUT, int K, bool RELU>
-__global__ void conv_fwd_kernel(const TIN *__restrict__ x, const float *__restrict__ theta, int off_w, int off_b,
-                                TOUT *__restrict__ y, int n, int H, int W, bool half_weights)
+// ---------------------------------------------------------------- FP32 layers
+// The 3x3 layers forward, and backward to their inputs, are the same product: a
+// sum over the channels and taps of a plane set, in that order.  Each output used
+// to re-read its 9 CI inputs from L1 and one weight per multiply (39 us for 16 ->
+// 16 on 4 x 128^2 cells); now a CTA of 128 threads stages an 8 x 32 tile of every
+// input channel (and the layer's weights, output channel fastest) in shared
+// memory, and a thread carries two neighbouring cells' CO sums, so a 16-byte
+// weight read serves eight multiplies, paired (__ffma2_rn) over output channels.
+// The order of every sum is the one before, so the values are too.  Tiles of 256
+// cells: 4 x 128^2 cells are 256 CTAs, enough for every SM.
+constexpr int kTy = 8, kTx = 32;                       // tile of a CTA
+constexpr int kIy = kTy + 2, kIx = kTx + 2;            // its inputs
+
+// a tile of CI planes with its margin, zero outside the plane; plane stride ps floats
+template <int CI>
+__device__ __forceinline__ void stage_tile(const float *__restrict__ x, float *s, int ps, int H, int W, int ty, int tx)
 {
-    __shared__ float sw[COUT * CIN * K * K];
-    __shared__ float sb[COUT];
-    for (int k = threadIdx.x; k < COUT * CIN * K * K; k += blockDim.x) {
-        float v = theta[off_w + k];
-        sw[k] = half_weights ? __half2float(__float2half_rn(v)) : v;
-    }
-    for (int k = threadIdx.x; k < COUT; k += blockDim.x) sb[k] = theta[off_b + k];
-    __syncthreads();
     const long long plane = (long long)H * W;
-    const long long total = (long long)n * plane;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < total; p += (long long)gridDim.x * blockDim.x) {
-        const int img = (int)(p / plane);
-        const int rem = (int)(p - (long long)img * plane);
-        const int i = rem / W, j = rem % W;
-        float acc[COUT];
+    for (int e = threadIdx.x; e < CI * kIy * kIx; e += blockDim.x) {
+        const int c = e / (kIy * kIx), r = e - c * (kIy * kIx), i = r / kIx, j = r - i * kIx;
+        const int yy = ty - 1 + i, xx = tx - 1 + j;
+        s[c * ps + r] = yy >= 0 && yy < H && xx >= 0 && xx < W ? x[c * plane + (long long)yy * W + xx] : 0.0f;
+    }
+}
+
+// BACK = false: y[o] = relu(b[o] + sum_c sum_tap w[o, c, tap] x[c, cell + tap]);
+// BACK = true: y[c] = relu'(act[c]) sum_o sum_tap w[o, c, tap] x[o, cell - tap].
+// CI planes in, CO planes out; wn, wi: the layer's own output and input channels.
+template <int CI, int CO, bool BACK>
+__global__ void __launch_bounds__(128) conv3_kernel(const float *__restrict__ x, const float *__restrict__ theta, int off_w,
+                                                    int off_b, const float *__restrict__ act, float *__restrict__ y, int H,
+                                                    int W, int tiles_x, int tiles_y)
+{
+    constexpr int PS = kIy * kIx;
+    __shared__ __align__(16) float sx[CI * PS];
+    __shared__ __align__(16) float sw[CI * 9 * CO];
+    const int img = blockIdx.x / (tiles_x * tiles_y), tq = blockIdx.x - img * (tiles_x * tiles_y);
+    const int ty = (tq / tiles_x) * kTy, tx = (tq % tiles_x) * kTx;
+    const long long plane = (long long)H * W;
+    x += (long long)img * CI * plane;
+    y += (long long)img * CO * plane;
+    for (int e = threadIdx.x; e < CI * 9 * CO; e += 128) {
+        const int o = e % CO, q = e / CO, tap = q % 9, c = q / 9;   // into [c][tap][o]
+        sw[e] = theta[off_w + (BACK ? (c * CO + o) : (o * CI + c)) * 9 + tap];
+    }
+    stage_tile<CI>(x, sx, PS, H, W, ty, tx);
+    __syncthreads();
+    const int r = threadIdx.x >> 4, c0 = 2 * (threadIdx.x & 15);   // cells (ty + r, tx + c0) and the next
+    float2 acc[2][CO / 2];
 #pragma unroll
-        for (int o = 0; o < COUT; o++) acc[o] = sb[o];
-        const TIN *xi = x + (long long)img * CIN * plane;
-        for (int c = 0; c < CIN; c++) {
+    for (int o = 0; o < CO / 2; o++) {
+        const float2 b = BACK ? make_float2(0.0f, 0.0f) : make_float2(theta[off_b + 2 * o], theta[off_b + 2 * o + 1]);
+        acc[0][o] = b;
+        acc[1][o] = b;
+    }
+#pragma unroll 1
+    for (int c = 0; c < CI; c++) {
+        float v[3][4];
 #pragma unroll
-            for (int di = 0; di < K; di++) {
-                const int ii = i + di - K / 2;
-                if (ii < 0 || ii >= H) continue;
+        for (int i = 0; i < 3; i++) {
+            const float2 *p = reinterpret_cast<const float2 *>(sx + c * PS + (r + i) * kIx + c0);
+            const float2 a = p[0], b = p[1];
+            v[i][0] = a.x; v[i][1] = a.y; v[i][2] = b.x; v[i][3] = b.y;
+        }
 #pragma unroll
-                for (int dj = 0; dj < K; dj++) {
-                    const int jj = j + dj - K / 2;
-                    if (jj < 0 || jj >= W) continue;
-                    const float v = (float)xi[(long long)c * plane + (long long)ii * W + jj];
+        for (int tap = 0; tap < 9; tap++) {
+            const int i = BACK ? 2 - tap / 3 : tap / 3, j = BACK ? 2 - tap % 3 : tap % 3;
+            const float4 *w4 = reinterpret_cast<const float4 *>(sw + (c * 9 + tap) * CO);
+            const float2 v0 = make_float2(v[i][j], v[i][j]), v1 = make_float2(v[i][j + 1], v[i][j + 1]);
 #pragma unroll
-                    for (int o = 0; o < COUT; o++) acc[o] = fmaf(sw[((o * CIN + c) * K + di) * K + dj], v, acc[o]);
-                }
+            for (int o = 0; o < CO / 4; o++) {
+                const float4 w = w4[o];
+                const float2 wa = make_float2(w.x, w.y), wb = make_float2(w.z, w.w);
+                acc[0][2 * o] = __ffma2_rn(wa, v0, acc[0][2 * o]);
+                acc[1][2 * o] = __ffma2_rn(wa, v1, acc[1][2 * o]);
+                acc[0][2 * o + 1] = __ffma2_rn(wb, v0, acc[0][2 * o + 1]);
+                acc[1][2 * o + 1] = __ffma2_rn(wb, v1, acc[1][2 * o + 1]);
             }
         }
-        TOUT *yo = y + (long long)img * COUT * plane + rem;
+    }
+    const int yy = ty + r;
+    if (yy >= H) return;
 #pragma unroll
-        for (int o = 0; o < COUT; o++) {
-            float v = RELU ? fmaxf(acc[o], 0.0f) : acc[o];
-            yo[(long long)o * plane] = (TOUT)v;
+    for (int q = 0; q < 2; q++) {
+        const int xx = tx + c0 + q;
+        if (xx >= W) continue;
+        const long long k = (long long)yy * W + xx;
+#pragma unroll
+        for (int o = 0; o < CO; o++) {
+            float v = o & 1 ? acc[q][o / 2].y : acc[q][o / 2].x;
+            if (BACK) v = act[(long long)img * CO * plane + o * plane + k] > 0.0f ? v : 0.0f;
+            else v = fmaxf(v, 0.0f);
+            y[o * plane + k] = v;
         }
     }
 }
 
-// dL/dz of the head and the loss: g = (sigmoid(z) - t) m / M
-__global__ void bce_grad_kernel(const float *z, const float *t, const float *m, long long total, float inv_count,
-                                float *g, double *loss)
+// The 1x1 head on its own (inference in FP32)
+__global__ void head_kernel(const float *__restrict__ a3, const float *__restrict__ theta, int off_w, int off_b,
+                            float *__restrict__ z, int n, long long plane)
 {
+    const long long total = (long long)n * plane;
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < total; p += (long long)gridDim.x * blockDim.x) {
+        const long long img = p / plane, k = p - img * plane;
+        float v = theta[off_b];
+#pragma unroll
+        for (int c = 0; c < HID; c++) v = fmaf(theta[off_w + c], a3[(img * HID + c) * plane + k], v);
+        z[p] = v;
+    }
+}
+
+// The head, its loss and its backward pass in one pass over the last activations:
+// the logit z, g = dL/dz = (sigmoid(z) - t) m / M and the loss, the head's weight
+// and bias gradients, and dL/d(a3) times ReLU'.  As four kernels they read a3 three
+// times, and the weight gradient alone took 381 us.
+__global__ void __launch_bounds__(128) head_loss_kernel(const float *__restrict__ a3, const float *__restrict__ theta, int off_w,
+                                                        int off_b, const float *__restrict__ t, const float *__restrict__ m,
+                                                        long long total, long long plane, float inv_count, float *ga, float *gw,
+                                                        float *gb, double *loss)
+{
+    float w[HID], dw[HID], db = 0.0f;
     double part = 0.0;
+#pragma unroll
+    for (int c = 0; c < HID; c++) { w[c] = theta[off_w + c]; dw[c] = 0.0f; }
+    const float b = theta[off_b];
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < total; p += (long long)gridDim.x * blockDim.x) {
-        float zz = z[p], tt = t[p], mm = m[p];
-        float s = 1.0f / (1.0f + __expf(-zz));
-        g[p] = (s - tt) * mm * inv_count;
-        float l = fmaxf(zz, 0.0f) - zz * tt + log1pf(__expf(-fabsf(zz)));
+        const long long img = p / plane, k = p - img * plane, q = img * HID * plane + k;
+        float a[HID], zz = b;
+#pragma unroll
+        for (int c = 0; c < HID; c++) { a[c] = a3[q + c * plane]; }
+#pragma unroll
+        for (int c = 0; c < HID; c++) zz = fmaf(w[c], a[c], zz);
+        const float tt = t[p], mm = m[p];
+        const float sg = 1.0f / (1.0f + __expf(-zz));
+        const float g = (sg - tt) * mm * inv_count;
+        const float l = fmaxf(zz, 0.0f) - zz * tt + log1pf(__expf(-fabsf(zz)));
         part += (double)(l * mm);
-    }
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, part * (double)inv_count);
-}
-
-// weight and bias gradients of one layer: dW[o,c,di,dj] = sum g[n,o,i,j] a[n,c,i+di-1,j+dj-1].
-// Each block reduces a slice of the pixels for every weight entry (threads over entries) and adds its
-// partial sums with one atomic per entry.
-template <int CIN, int COUT, int K>
-__global__ void conv_wgrad_kernel(const float *__restrict__ g, const float *__restrict__ a, int n, int H, int W,
-                                  float *gw, float *gb, int pix_per_block)
-{
-    constexpr int NW = COUT * CIN * K * K;
-    const long long plane = (long long)H * W;
-    const long long total = (long long)n * plane;
-    const long long p0 = (long long)blockIdx.x * pix_per_block;
-    const long long p1 = p0 + pix_per_block < total ? p0 + pix_per_block : total;
-    for (int e = threadIdx.x; e < NW + COUT; e += blockDim.x) {
-        float acc = 0.0f;
-        if (e < NW) {
-            const int dj = e % K, di = (e / K) % K, c = (e / (K * K)) % CIN, o = e / (K * K * CIN);
-            for (long long p = p0; p < p1; p++) {
-                const int img = (int)(p / plane);
-                const int rem = (int)(p - (long long)img * plane);
-                const int i = rem / W, j = rem % W;
-                const int ii = i + di - K / 2, jj = j + dj - K / 2;
-                if (ii < 0 || ii >= H || jj < 0 || jj >= W) continue;
-                acc = fmaf(g[((long long)img * COUT + o) * plane + rem],
-                           a[((long long)img * CIN + c) * plane + (long long)ii * W + jj], acc);
-            }
-            atomicAdd(gw + e, acc);
-        } else {
-            const int o = e - NW;
-            for (long long p = p0; p < p1; p++) {
-                const int img = (int)(p / plane);
-                const int rem = (int)(p - (long long)img * plane);
-                acc += g[((long long)img * COUT + o) * plane + rem];
-            }
-            atomicAdd(gb + o, acc);
+        db += g;
+#pragma unroll
+        for (int c = 0; c < HID; c++) {
+            dw[c] = fmaf(g, a[c], dw[c]);
+            ga[q + c * plane] = a[c] > 0.0f ? w[c] * g : 0.0f;
         }
     }
+    __shared__ float red[4][HID + 1];
+    __shared__ double redl[4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        part += __shfl_xor_sync(0xffffffffu, part, o);
+        db += __shfl_xor_sync(0xffffffffu, db, o);
+#pragma unroll
+        for (int c = 0; c < HID; c++) dw[c] += __shfl_xor_sync(0xffffffffu, dw[c], o);
+    }
+    if (lane == 0) {
+#pragma unroll
+        for (int c = 0; c < HID; c++) red[warp][c] = dw[c];
+        red[warp][HID] = db;
+        redl[warp] = part;
+    }
+    __syncthreads();
+    if (threadIdx.x <= HID) {
+        const float v = (red[0][threadIdx.x] + red[1][threadIdx.x]) + (red[2][threadIdx.x] + red[3][threadIdx.x]);
+        atomicAdd(threadIdx.x < HID ? gw + threadIdx.x : gb, v);
+    }
+    if (threadIdx.x == 32) atomicAdd(loss, ((redl[0] + redl[1]) + (redl[2] + redl[3])) * (double)inv_count);
 }
 
-// gradient with respect to the layer input, times ReLU' of that input:
-// ga[n,c,i,j] = relu'(a) * sum_o sum_taps w[o,c,di,dj] g[n,o,i-di+1,j-dj+1]
-template <int CIN, int COUT, int K>
-__global__ void conv_dgrad_kernel(const float *__restrict__ g, const float *__restrict__ theta, int off_w,
-                                  const float *__restrict__ a, int n, int H, int W, float *ga)
+// Weight and bias gradients of a 3x3 layer: dW[o, c, tap] = sum over cells of g[o,
+// cell] a[c, cell + tap], db[o] = sum of g[o].  One thread used to walk 1024 cells
+// for each weight, dividing for every index (2.6 ms a 16 -> 16 layer on 4 x 128^2
+// cells).  Now a CTA of 256 threads keeps a tile of both operands in shared memory
+// (g with the channels together), and a thread owns one input channel and four
+// output channels: their 36 sums stay in registers while a 3 x 3 window slides along
+// units of 16 cells, 18 paired multiply-adds for one 16-byte and three 4-byte reads.
+// The threads that are left over split the units.  A CTA adds up several tiles
+// before it adds its sums to the result, one atomic per weight.
+template <int CI>
+__global__ void __launch_bounds__(256) wgrad3_kernel(const float *__restrict__ g, const float *__restrict__ a, int n, int H,
+                                                     int W, int tiles_x, int tiles_y, float *gw, float *gb)
 {
-    __shared__ float sw[COUT * CIN * K * K];
-    for (int k = threadIdx.x; k < COUT * CIN * K * K; k += blockDim.x) sw[k] = theta[off_w + k];
-    __syncthreads();
+    constexpr int PS = kIy * kIx + 1;          // odd: channels fall on different banks
+    constexpr int NC = 4 * CI;                 // (channel, four outputs) pairs
+    constexpr int SUB = 256 / NC;              // threads per pair
+    constexpr int UNITS = kTy * kTx / 16;      // units of 16 cells of a row
+    __shared__ float sa[CI * PS];
+    __shared__ __align__(16) float sg[kTy * kTx * HID];
     const long long plane = (long long)H * W;
-    const long long total = (long long)n * plane;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < total; p += (long long)gridDim.x * blockDim.x) {
-        const int img = (int)(p / plane);
-        const int rem = (int)(p - (long long)img * plane);
-        const int i = rem / W, j = rem % W;
-        float acc[CIN];
+    const int pair = threadIdx.x % NC, sub = threadIdx.x / NC;
+    const int c = pair % CI, og = pair / CI;
+    float2 acc[9][2], bs[2];
 #pragma unroll
-        for (int c = 0; c < CIN; c++) acc[c] = 0.0f;
-        for (int o = 0; o < COUT; o++) {
+    for (int q = 0; q < 9; q++) { acc[q][0] = make_float2(0.0f, 0.0f); acc[q][1] = make_float2(0.0f, 0.0f); }
+    bs[0] = make_float2(0.0f, 0.0f); bs[1] = make_float2(0.0f, 0.0f);
+    const int ntile = n * tiles_x * tiles_y;
+    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+        const int img = tile / (tiles_x * tiles_y), q = tile - img * (tiles_x * tiles_y);
+        const int ty = (q / tiles_x) * kTy, tx = (q % tiles_x) * kTx;
+        __syncthreads();   // the last tile has been used
+        stage_tile<CI>(a + (long long)img * CI * plane, sa, PS, H, W, ty, tx);
+        for (int e = threadIdx.x; e < kTy * kTx * HID; e += 256) {
+            const int o = e / (kTy * kTx), r = e - o * (kTy * kTx), i = r / kTx, j = r - i * kTx;
+            const int yy = ty + i, xx = tx + j;
+            sg[r * HID + o] = yy < H && xx < W ? g[((long long)img * HID + o) * plane + (long long)yy * W + xx] : 0.0f;
+        }
+        __syncthreads();
+        if (sub < SUB)
+            for (int u = sub; u < UNITS; u += SUB) {
+                const int i = u / (kTx / 16), j0 = (u % (kTx / 16)) * 16;
+                const float *w0 = sa + c * PS + i * kIx + j0;
+                const float4 *gp = reinterpret_cast<const float4 *>(sg + (i * kTx + j0) * HID) + og;
+                float v[3][3];
 #pragma unroll
-            for (int di = 0; di < K; di++) {
-                const int ii = i - di + K / 2;
-                if (ii < 0 || ii >= H) continue;
+                for (int d = 0; d < 3; d++) { v[d][1] = w0[d * kIx]; v[d][2] = w0[d * kIx + 1]; }
+#pragma unroll 4
+                for (int j = 0; j < 16; j++) {
 #pragma unroll
-                for (int dj = 0; dj < K; dj++) {
-                    const int jj = j - dj + K / 2;
-                    if (jj < 0 || jj >= W) continue;
-                    const float gv = g[((long long)img * COUT + o) * plane + (long long)ii * W + jj];
+                    for (int d = 0; d < 3; d++) { v[d][0] = v[d][1]; v[d][1] = v[d][2]; v[d][2] = w0[d * kIx + j + 2]; }
+                    const float4 gg = gp[j * (HID / 4)];
+                    const float2 g0 = make_float2(gg.x, gg.y), g1 = make_float2(gg.z, gg.w);
+                    bs[0] = __fadd2_rn(bs[0], g0);
+                    bs[1] = __fadd2_rn(bs[1], g1);
 #pragma unroll
-                    for (int c = 0; c < CIN; c++) acc[c] = fmaf(sw[((o * CIN + c) * K + di) * K + dj], gv, acc[c]);
+                    for (int t = 0; t < 9; t++) {
+                        const float2 x = make_float2(v[t / 3][t % 3], v[t / 3][t % 3]);
+                        acc[t][0] = __ffma2_rn(g0, x, acc[t][0]);
+                        acc[t][1] = __ffma2_rn(g1, x, acc[t][1]);
+                    }
                 }
             }
-        }
+    }
+    // the sums of the threads of a pair, through the shared arrays
+    __syncthreads();
+    float *red = sg;   // [HID][CI][9] and the bias sums: fits in the g tile
+    static_assert(HID * CI * 9 + HID <= kTy * kTx * HID, "the sums fit");
+    for (int e = threadIdx.x; e < HID * CI * 9 + HID; e += 256) red[e] = 0.0f;
+    for (int s = 0; s < SUB; s++) {
+        __syncthreads();
+        if (sub == s) {
 #pragma unroll
-        for (int c = 0; c < CIN; c++) {
-            const long long q = ((long long)img * CIN + c) * plane + rem;
-            ga[q] = a[q] > 0.0f ? acc[c] : 0.0f;
+            for (int t = 0; t < 9; t++) {
+                float *d = red + ((4 * og) * CI + c) * 9 + t;
+                d[0] += acc[t][0].x;
+                d[CI * 9] += acc[t][0].y;
+                d[2 * CI * 9] += acc[t][1].x;
+                d[3 * CI * 9] += acc[t][1].y;
+            }
+            if (c == 0) {
+                float *d = red + HID * CI * 9 + 4 * og;
+                d[0] += bs[0].x; d[1] += bs[0].y; d[2] += bs[1].x; d[3] += bs[1].y;
+            }
         }
     }
+    __syncthreads();
+    for (int e = threadIdx.x; e < HID * CI * 9; e += 256) atomicAdd(gw + e, red[e]);
+    if (threadIdx.x < HID) atomicAdd(gb + threadIdx.x, red[HID * CI * 9 + threadIdx.x]);
 }
 
 __global__ void adam_kernel(float *theta, const float *grad, float *m, float *v, int np, float lr, float b1, float b2,
@@ -220,9 +336,10 @@ constexpr int N0 = H0 * W0, N1 = H1 * W1, N2 = H2 * W2;
 constexpr int NWARP = 4;
 // per layer: 9 taps x 2 n-blocks x 32 lanes x 2 registers of packed FP16 weights
 constexpr int WFRAG = 9 * 2 * 32 * 2;
+constexpr int PACK = 3 * WFRAG + 3 * 16 + 32;   // words of the packed weights: fragments, biases, head and its bias
 constexpr size_t smem_bytes()
 {
-    return (size_t)(N0 > N2 ? N0 : N2) * PS * 2 + (size_t)N1 * PS * 2 + 3 * WFRAG * 4 + 3 * 16 * 4 + 16 * 4 + 16;
+    return (size_t)(N0 > N2 ? N0 : N2) * PS * 2 + (size_t)N1 * PS * 2 + (size_t)PACK * 4;
 }
 }  // namespace tc
 
@@ -332,22 +449,14 @@ __device__ __forceinline__ void tc_layer(const __half *in, int wi, __half *out, 
     }
 }
 
-__global__ void __launch_bounds__(tc::NWARP * 32) cnn_infer_tc_kernel(const float *__restrict__ theta,
-                                                                      const float *__restrict__ x, int H, int W,
-                                                                      float *__restrict__ logits)
+// The weights as the inference kernel's CTAs hold them: MMA fragments b0 =
+// (W[o][2t][tap], W[o][2t+1][tap]), b1 = channels 2t+8, 2t+9, o = nb*8 + lane/4;
+// biases; the head rounded to FP16 and its bias.  Packed once per call: every CTA
+// gathering them from theta itself took longer than its three layers.
+__global__ void cnn_pack_kernel(const float *__restrict__ theta, uint32_t *out)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __half *s0 = reinterpret_cast<__half *>(smem);                               // inputs, then layer 2
-    __half *s1 = s0 + (size_t)(tc::N0 > tc::N2 ? tc::N0 : tc::N2) * tc::PS;      // layer 1
-    uint32_t *wf = reinterpret_cast<uint32_t *>(s1 + (size_t)tc::N1 * tc::PS);    // weight fragments, 3 layers
-    float *bias = reinterpret_cast<float *>(wf + 3 * tc::WFRAG);                 // 3 x 16
-    float *whead = bias + 48;                                                     // 16, then its bias
-    const int img = blockIdx.z;
-    const int ty0 = blockIdx.y * tc::TH, tx0 = blockIdx.x * tc::TW;
-    const long long plane = (long long)H * W;
-    const float *xi = x + (long long)img * kCnnIn * plane;
-    // weight fragments: b0 = (W[o][2t][tap], W[o][2t+1][tap]), b1 = channels 2t+8, 2t+9; o = nb*8 + lane/4
-    for (int e = threadIdx.x; e < 3 * 9 * 2 * 32; e += blockDim.x) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < 3 * 9 * 2 * 32) {
         const int l = e / (9 * 2 * 32), rem = e % (9 * 2 * 32);
         const int tap = rem / 64, nb = (rem / 32) % 2, ln = rem % 32;
         const LayerSpec S = layer_spec(l);
@@ -358,24 +467,47 @@ __global__ void __launch_bounds__(tc::NWARP * 32) cnn_infer_tc_kernel(const floa
             const int cch = k0 + (q & 1) + (q >> 1) * 8;
             w[q] = cch < S.cin ? theta[S.woff + (o * S.cin + cch) * 9 + tap] : 0.0f;
         }
-        uint32_t *f = wf + l * tc::WFRAG + ((tap * 2 + nb) * 32 + ln) * 2;
+        uint32_t *f = out + l * tc::WFRAG + ((tap * 2 + nb) * 32 + ln) * 2;
         f[0] = pack_half2(w[0], w[1]);
         f[1] = pack_half2(w[2], w[3]);
     }
-    for (int e = threadIdx.x; e < 48; e += blockDim.x) bias[e] = theta[layer_spec(e / 16).boff + e % 16];
-    if (threadIdx.x < 16) {
+    float *tail = reinterpret_cast<float *>(out + 3 * tc::WFRAG);
+    if (e < 48) tail[e] = theta[layer_spec(e / 16).boff + e % 16];
+    if (e < 32) {
         const LayerSpec S = layer_spec(3);
-        whead[threadIdx.x] = __half2float(__float2half_rn(theta[S.woff + threadIdx.x]));
-        if (threadIdx.x == 0) whead[16] = theta[S.boff];
+        tail[48 + e] = e < 16 ? __half2float(__float2half_rn(theta[S.woff + e])) : (e == 16 ? theta[S.boff] : 0.0f);
     }
-    // inputs of the 3-cell grown tile, FP16, zero outside the plane and in channels 5..15
-    for (int e = threadIdx.x; e < tc::N0 * 16; e += blockDim.x) {
-        const int p = e / 16, ch = e % 16;
+}
+
+__global__ void __launch_bounds__(tc::NWARP * 32) cnn_infer_tc_kernel(const uint32_t *__restrict__ packed,
+                                                                      const float *__restrict__ x, int H, int W,
+                                                                      float *__restrict__ logits)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __half *s0 = reinterpret_cast<__half *>(smem);                               // inputs, then layer 2
+    __half *s1 = s0 + (size_t)(tc::N0 > tc::N2 ? tc::N0 : tc::N2) * tc::PS;      // layer 1
+    uint32_t *wf = reinterpret_cast<uint32_t *>(s1 + (size_t)tc::N1 * tc::PS);    // packed weights
+    const float *bias = reinterpret_cast<const float *>(wf + 3 * tc::WFRAG);     // 3 x 16
+    const float *whead = bias + 48;                                               // 16, then its bias
+    const int img = blockIdx.z;
+    const int ty0 = blockIdx.y * tc::TH, tx0 = blockIdx.x * tc::TW;
+    const long long plane = (long long)H * W;
+    const float *xi = x + (long long)img * kCnnIn * plane;
+    static_assert(tc::PACK % 4 == 0 && ((tc::N0 > tc::N2 ? tc::N0 : tc::N2) + tc::N1) * tc::PS % 8 == 0, "16-byte copies");
+    for (int e = threadIdx.x; e < tc::PACK / 4; e += blockDim.x)
+        reinterpret_cast<uint4 *>(wf)[e] = reinterpret_cast<const uint4 *>(packed)[e];
+    // inputs of the 3-cell grown tile, FP16, zero outside the plane and in channels
+    // 5..15; a cell's 16 channels are two 16-byte stores
+    for (int p = threadIdx.x; p < tc::N0; p += blockDim.x) {
         const int r = p / tc::W0, c = p - r * tc::W0;
         const int yy = ty0 - 3 + r, xx = tx0 - 3 + c;
-        float v = 0.0f;
-        if (ch < kCnnIn && yy >= 0 && yy < H && xx >= 0 && xx < W) v = xi[(long long)ch * plane + (long long)yy * W + xx];
-        s0[p * tc::PS + ch] = __float2half_rn(v);
+        float v[kCnnIn];
+        const bool in = yy >= 0 && yy < H && xx >= 0 && xx < W;
+#pragma unroll
+        for (int ch = 0; ch < kCnnIn; ch++) v[ch] = in ? xi[(long long)ch * plane + (long long)yy * W + xx] : 0.0f;
+        uint4 *d = reinterpret_cast<uint4 *>(s0 + p * tc::PS);
+        d[0] = make_uint4(pack_half2(v[0], v[1]), pack_half2(v[2], v[3]), pack_half2(v[4], 0.0f), 0u);
+        d[1] = make_uint4(0u, 0u, 0u, 0u);
     }
     __syncthreads();
     tc_layer<false>(s0, tc::W0, s1, tc::H1, tc::W1, ty0 - 2, tx0 - 2, H, W, wf, bias, nullptr, 0.0f, nullptr);
@@ -399,25 +531,36 @@ int cnn_n_params()
 size_t cnn_workspace_floats(int n, int H, int W)
 {
     const size_t px = (size_t)n * H * W;
-    return px * (size_t)(3 * HID + 1) /* activations a1..a3, logits */ + px * (size_t)(2 * HID) /* two grad planes */ +
-           px /* head grad */;
+    return px * (size_t)(3 * HID) /* activations a1..a3 */ + px * (size_t)(2 * HID) /* two gradient plane sets */;
+}
+
+// the three hidden layers in FP32, activations a1, a2, a3 to act
+static int hidden_forward(const float *theta, const float *x, int n, int H, int W, float *act, cudaStream_t st)
+{
+    const long long px = (long long)n * H * W;
+    const LayerSpec L0 = layer_spec(0), L1 = layer_spec(1), L2 = layer_spec(2);
+    const int txs = (W + kTx - 1) / kTx, tys = (H + kTy - 1) / kTy;
+    const long long tiles = (long long)n * txs * tys;
+    if (tiles > 0x7fffffffLL) return (int)cudaErrorInvalidValue;
+    const unsigned grid = (unsigned)tiles;
+    float *a1 = act, *a2 = act + px * HID, *a3 = act + 2 * px * HID;
+    conv3_kernel<kCnnIn, HID, false><<<grid, 128, 0, st>>>(x, theta, L0.woff, L0.boff, nullptr, a1, H, W, txs, tys);
+    conv3_kernel<HID, HID, false><<<grid, 128, 0, st>>>(a1, theta, L1.woff, L1.boff, nullptr, a2, H, W, txs, tys);
+    conv3_kernel<HID, HID, false><<<grid, 128, 0, st>>>(a2, theta, L2.woff, L2.boff, nullptr, a3, H, W, txs, tys);
+    return (int)cudaGetLastError();
 }
 
 int cnn_forward(const float *theta, const float *x, int n, int H, int W, bool fp16, float *act, float *logits,
                 void *half_ws, cudaStream_t st)
 {
     const long long px = (long long)n * H * W;
-    const int th = 128, bl = blocks_for(px, th);
-    float *a1 = act, *a2 = act + px * HID, *a3 = act + 2 * px * HID;
-    LayerSpec L0 = layer_spec(0), L1 = layer_spec(1), L2 = layer_spec(2), L3 = layer_spec(3);
     if (!fp16) {
-        conv_fwd_kernel<float, float, kCnnIn, HID, 3, true><<<bl, th, 0, st>>>(x, theta, L0.woff, L0.boff, a1, n, H, W, false);
-        conv_fwd_kernel<float, float, HID, HID, 3, true><<<bl, th, 0, st>>>(a1, theta, L1.woff, L1.boff, a2, n, H, W, false);
-        conv_fwd_kernel<float, float, HID, HID, 3, true><<<bl, th, 0, st>>>(a2, theta, L2.woff, L2.boff, a3, n, H, W, false);
-        conv_fwd_kernel<float, float, HID, 1, 1, false><<<bl, th, 0, st>>>(a3, theta, L3.woff, L3.boff, logits, n, H, W, false);
+        const LayerSpec L3 = layer_spec(3);
+        const int e = hidden_forward(theta, x, n, H, W, act, st);
+        if (e) return e;
+        head_kernel<<<blocks_for(px, 128), 128, 0, st>>>(act + 2 * px * HID, theta, L3.woff, L3.boff, logits, n, (long long)H * W);
     } else {
         // FP16 activations and weights, FP32 accumulation: one fused tensor-core kernel
-        (void)half_ws;
         static bool configured = false;
         const size_t sm = tc::smem_bytes();
         if (!configured) {
@@ -426,43 +569,43 @@ int cnn_forward(const float *theta, const float *x, int n, int H, int W, bool fp
             configured = true;
         }
         dim3 grid((W + tc::TW - 1) / tc::TW, (H + tc::TH - 1) / tc::TH, n);
-        cnn_infer_tc_kernel<<<grid, tc::NWARP * 32, sm, st>>>(theta, x, H, W, logits);
+        uint32_t *packed = reinterpret_cast<uint32_t *>(half_ws);
+        cnn_pack_kernel<<<(3 * 9 * 2 * 32 + 127) / 128, 128, 0, st>>>(theta, packed);
+        cnn_infer_tc_kernel<<<grid, tc::NWARP * 32, sm, st>>>(packed, x, H, W, logits);
     }
     return (int)cudaGetLastError();
 }
 
 size_t cnn_half_workspace_bytes(int, int, int)
 {
-    return 16;   // the fused inference kernel keeps its activations in shared memory
+    return (size_t)tc::PACK * 4;   // the packed weights (activations stay in shared memory)
 }
 
 int cnn_loss_grad(const float *theta, const float *x, const float *t, const float *m, int n, int H, int W, float mcount,
                   float *ws, float *grad, double *loss, cudaStream_t st)
 {
     const long long px = (long long)n * H * W;
-    float *act = ws, *logits = ws + px * 3 * HID;
-    float *ga = logits + px, *gb = ga + px * HID, *gz = gb + px * HID;
-    int e = cnn_forward(theta, x, n, H, W, false, act, logits, nullptr, st);
-    if (e) return e;
-    const int th = 128, bl = blocks_for(px, th);
-    float *a1 = act, *a2 = act + px * HID, *a3 = act + 2 * px * HID;
-    LayerSpec L0 = layer_spec(0), L1 = layer_spec(1), L2 = layer_spec(2), L3 = layer_spec(3);
+    const long long plane = (long long)H * W;
+    float *act = ws, *ga = ws + px * 3 * HID, *gb = ga + px * HID;
+    const float *a1 = act, *a2 = act + px * HID, *a3 = act + 2 * px * HID;
+    const LayerSpec L0 = layer_spec(0), L1 = layer_spec(1), L2 = layer_spec(2), L3 = layer_spec(3);
     cudaMemsetAsync(grad, 0, cnn_n_params() * sizeof(float), st);
     cudaMemsetAsync(loss, 0, sizeof(double), st);
-    bce_grad_kernel<<<bl, th, 0, st>>>(logits, t, m, px, mcount > 0 ? 1.0f / mcount : 0.0f, gz, loss);
-    const int ppb = 1024;
-    const int wb = (int)((px + ppb - 1) / ppb);
+    const int e = hidden_forward(theta, x, n, H, W, act, st);
+    if (e) return e;
     // head (1x1, 16 -> 1)
-    conv_wgrad_kernel<HID, 1, 1><<<wb, 128, 0, st>>>(gz, a3, n, H, W, grad + L3.woff, grad + L3.boff, ppb);
-    conv_dgrad_kernel<HID, 1, 1><<<bl, th, 0, st>>>(gz, theta, L3.woff, a3, n, H, W, ga);
+    head_loss_kernel<<<(int)std::min<long long>((px + 127) / 128, 152 * 8), 128, 0, st>>>(
+        a3, theta, L3.woff, L3.boff, t, m, px, plane, mcount > 0 ? 1.0f / mcount : 0.0f, ga, grad + L3.woff, grad + L3.boff, loss);
+    const int txs = (W + kTx - 1) / kTx, tys = (H + kTy - 1) / kTy;
+    const int grid = n * txs * tys, wb = std::min(grid, 152 * 2);
     // layer 3 (3x3, 16 -> 16): input a2
-    conv_wgrad_kernel<HID, HID, 3><<<wb, 256, 0, st>>>(ga, a2, n, H, W, grad + L2.woff, grad + L2.boff, ppb);
-    conv_dgrad_kernel<HID, HID, 3><<<bl, th, 0, st>>>(ga, theta, L2.woff, a2, n, H, W, gb);
+    wgrad3_kernel<HID><<<wb, 256, 0, st>>>(ga, a2, n, H, W, txs, tys, grad + L2.woff, grad + L2.boff);
+    conv3_kernel<HID, HID, true><<<grid, 128, 0, st>>>(ga, theta, L2.woff, 0, a2, gb, H, W, txs, tys);
     // layer 2: input a1
-    conv_wgrad_kernel<HID, HID, 3><<<wb, 256, 0, st>>>(gb, a1, n, H, W, grad + L1.woff, grad + L1.boff, ppb);
-    conv_dgrad_kernel<HID, HID, 3><<<bl, th, 0, st>>>(gb, theta, L1.woff, a1, n, H, W, ga);
+    wgrad3_kernel<HID><<<wb, 256, 0, st>>>(gb, a1, n, H, W, txs, tys, grad + L1.woff, grad + L1.boff);
+    conv3_kernel<HID, HID, true><<<grid, 128, 0, st>>>(gb, theta, L1.woff, 0, a1, ga, H, W, txs, tys);
     // layer 1: input x (no ReLU before it, no input gradient needed)
-    conv_wgrad_kernel<kCnnIn, HID, 3><<<wb, 256, 0, st>>>(ga, x, n, H, W, grad + L0.woff, grad + L0.boff, ppb);
+    wgrad3_kernel<kCnnIn><<<wb, 256, 0, st>>>(ga, x, n, H, W, txs, tys, grad + L0.woff, grad + L0.boff);
     return (int)cudaGetLastError();
 }
 

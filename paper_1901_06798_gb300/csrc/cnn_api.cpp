@@ -16,11 +16,20 @@ using namespace tsu;
 
 namespace {
 
-struct Buf {
-    void *p = nullptr;
-    ~Buf() { if (p) cudaFree(p); }
-    cudaError_t alloc(size_t bytes) { return cudaMalloc(&p, bytes < 16 ? 16 : bytes); }
-    template <typename T> T *as() { return reinterpret_cast<T *>(p); }
+// The device buffers of one call, cut out of one allocation (each cudaMalloc and
+// cudaFree takes tens of microseconds, and the calls used up to twelve)
+struct Bufs {
+    char *p = nullptr;
+    size_t used = 0;
+    ~Bufs() { if (p) cudaFree(p); }
+    size_t want(size_t bytes)   // offset of a buffer; all are asked for before alloc()
+    {
+        const size_t o = used;
+        used += (bytes + 255) & ~(size_t)255;
+        return o;
+    }
+    cudaError_t alloc() { return cudaMalloc((void **)&p, used < 256 ? 256 : used); }
+    template <typename T> T *at(size_t off) const { return reinterpret_cast<T *>(p + off); }
 };
 
 #define CKR(x) do { if ((x) != cudaSuccess) return TSU_ERR_CUDA; } while (0)
@@ -34,17 +43,17 @@ extern "C" int tsu_cnn_forward(const float *theta, const float *x, int n, int h,
     if (!theta || !x || !logits || n < 1 || h < 1 || w < 1) return TSU_ERR_ARG;
     const size_t px = (size_t)n * h * w;
     const int np = cnn_n_params();
-    Buf dth, dx, dact, dlog, dhalf;
-    CKR(dth.alloc(np * sizeof(float)));
-    CKR(dx.alloc(px * kCnnIn * sizeof(float)));
-    CKR(dact.alloc(px * 3 * kCnnHidden * sizeof(float)));
-    CKR(dlog.alloc(px * sizeof(float)));
-    CKR(dhalf.alloc(cnn_half_workspace_bytes(n, h, w)));
-    CKR(cudaMemcpy(dth.p, theta, np * sizeof(float), cudaMemcpyHostToDevice));
-    CKR(cudaMemcpy(dx.p, x, px * kCnnIn * sizeof(float), cudaMemcpyHostToDevice));
-    if (cnn_forward(dth.as<float>(), dx.as<float>(), n, h, w, fp16 != 0, dact.as<float>(), dlog.as<float>(), dhalf.p, 0))
+    Bufs b;
+    const size_t oth = b.want(np * sizeof(float)), ox = b.want(px * kCnnIn * sizeof(float)), olog = b.want(px * sizeof(float));
+    const size_t oact = b.want(fp16 ? 0 : px * 3 * kCnnHidden * sizeof(float));   // FP32 only
+    const size_t ohalf = b.want(fp16 ? cnn_half_workspace_bytes(n, h, w) : 0);
+    CKR(b.alloc());
+    CKR(cudaMemcpy(b.at<float>(oth), theta, np * sizeof(float), cudaMemcpyHostToDevice));
+    CKR(cudaMemcpy(b.at<float>(ox), x, px * kCnnIn * sizeof(float), cudaMemcpyHostToDevice));
+    if (cnn_forward(b.at<float>(oth), b.at<float>(ox), n, h, w, fp16 != 0, b.at<float>(oact), b.at<float>(olog),
+                    b.at<char>(ohalf), 0))
         return TSU_ERR_CUDA;
-    CKR(cudaMemcpy(logits, dlog.p, px * sizeof(float), cudaMemcpyDeviceToHost));
+    CKR(cudaMemcpy(logits, b.at<float>(olog), px * sizeof(float), cudaMemcpyDeviceToHost));
     return TSU_OK;
 }
 
@@ -56,23 +65,20 @@ extern "C" int tsu_cnn_loss_grad(const float *theta, const float *x, const float
     const int np = cnn_n_params();
     double cnt = 0.0;
     for (size_t k = 0; k < px; k++) cnt += m[k];
-    Buf dth, dx, dt, dm, dws, dg, dl;
-    CKR(dth.alloc(np * sizeof(float)));
-    CKR(dx.alloc(px * kCnnIn * sizeof(float)));
-    CKR(dt.alloc(px * sizeof(float)));
-    CKR(dm.alloc(px * sizeof(float)));
-    CKR(dws.alloc(cnn_workspace_floats(n, h, w) * sizeof(float)));
-    CKR(dg.alloc(np * sizeof(float)));
-    CKR(dl.alloc(sizeof(double)));
-    CKR(cudaMemcpy(dth.p, theta, np * sizeof(float), cudaMemcpyHostToDevice));
-    CKR(cudaMemcpy(dx.p, x, px * kCnnIn * sizeof(float), cudaMemcpyHostToDevice));
-    CKR(cudaMemcpy(dt.p, t, px * sizeof(float), cudaMemcpyHostToDevice));
-    CKR(cudaMemcpy(dm.p, m, px * sizeof(float), cudaMemcpyHostToDevice));
-    if (cnn_loss_grad(dth.as<float>(), dx.as<float>(), dt.as<float>(), dm.as<float>(), n, h, w, (float)cnt,
-                      dws.as<float>(), dg.as<float>(), dl.as<double>(), 0))
+    Bufs b;
+    const size_t oth = b.want(np * sizeof(float)), ox = b.want(px * kCnnIn * sizeof(float)), ot = b.want(px * sizeof(float)),
+                 om = b.want(px * sizeof(float)), ows = b.want(cnn_workspace_floats(n, h, w) * sizeof(float)),
+                 og = b.want(np * sizeof(float)), ol = b.want(sizeof(double));
+    CKR(b.alloc());
+    CKR(cudaMemcpy(b.at<float>(oth), theta, np * sizeof(float), cudaMemcpyHostToDevice));
+    CKR(cudaMemcpy(b.at<float>(ox), x, px * kCnnIn * sizeof(float), cudaMemcpyHostToDevice));
+    CKR(cudaMemcpy(b.at<float>(ot), t, px * sizeof(float), cudaMemcpyHostToDevice));
+    CKR(cudaMemcpy(b.at<float>(om), m, px * sizeof(float), cudaMemcpyHostToDevice));
+    if (cnn_loss_grad(b.at<float>(oth), b.at<float>(ox), b.at<float>(ot), b.at<float>(om), n, h, w, (float)cnt,
+                      b.at<float>(ows), b.at<float>(og), b.at<double>(ol), 0))
         return TSU_ERR_CUDA;
-    CKR(cudaMemcpy(grad, dg.p, np * sizeof(float), cudaMemcpyDeviceToHost));
-    CKR(cudaMemcpy(loss, dl.p, sizeof(double), cudaMemcpyDeviceToHost));
+    CKR(cudaMemcpy(grad, b.at<float>(og), np * sizeof(float), cudaMemcpyDeviceToHost));
+    CKR(cudaMemcpy(loss, b.at<double>(ol), sizeof(double), cudaMemcpyDeviceToHost));
     return TSU_OK;
 }
 
@@ -85,25 +91,23 @@ extern "C" int tsu_cnn_train(float *theta, const float *x, const float *t, const
     if (batch > n) batch = n;
     const size_t plane = (size_t)h * w;
     const int np = cnn_n_params();
-    Buf dth, dx, dt, dm, dws, dg, dl, dmo, dv, bx, bt, bm;
-    CKR(dth.alloc(np * sizeof(float)));
-    CKR(dx.alloc((size_t)n * plane * kCnnIn * sizeof(float)));
-    CKR(dt.alloc((size_t)n * plane * sizeof(float)));
-    CKR(dm.alloc((size_t)n * plane * sizeof(float)));
-    CKR(dws.alloc(cnn_workspace_floats(batch, h, w) * sizeof(float)));
-    CKR(dg.alloc(np * sizeof(float)));
-    CKR(dl.alloc(sizeof(double)));
-    CKR(dmo.alloc(np * sizeof(float)));
-    CKR(dv.alloc(np * sizeof(float)));
-    CKR(bx.alloc((size_t)batch * plane * kCnnIn * sizeof(float)));
-    CKR(bt.alloc((size_t)batch * plane * sizeof(float)));
-    CKR(bm.alloc((size_t)batch * plane * sizeof(float)));
-    CKR(cudaMemcpy(dth.p, theta, np * sizeof(float), cudaMemcpyHostToDevice));
-    CKR(cudaMemcpy(dx.p, x, (size_t)n * plane * kCnnIn * sizeof(float), cudaMemcpyHostToDevice));
-    CKR(cudaMemcpy(dt.p, t, (size_t)n * plane * sizeof(float), cudaMemcpyHostToDevice));
-    CKR(cudaMemcpy(dm.p, m, (size_t)n * plane * sizeof(float), cudaMemcpyHostToDevice));
-    CKR(cudaMemset(dmo.p, 0, np * sizeof(float)));
-    CKR(cudaMemset(dv.p, 0, np * sizeof(float)));
+    Bufs b_;
+    const size_t fb = sizeof(float), np_ = (size_t)n * plane, bp = (size_t)batch * plane;
+    const size_t oth = b_.want(np * fb), ox = b_.want(np_ * kCnnIn * fb), ot = b_.want(np_ * fb), om = b_.want(np_ * fb),
+                 ows = b_.want(cnn_workspace_floats(batch, h, w) * fb), og = b_.want(np * fb), ol = b_.want(sizeof(double)),
+                 omo = b_.want(np * fb), ov = b_.want(np * fb), obx = b_.want(bp * kCnnIn * fb), obt = b_.want(bp * fb),
+                 obm = b_.want(bp * fb);
+    CKR(b_.alloc());
+    float *const dth = b_.at<float>(oth), *const dx = b_.at<float>(ox), *const dt = b_.at<float>(ot), *const dm = b_.at<float>(om);
+    float *const dg = b_.at<float>(og), *const dmo = b_.at<float>(omo), *const dv = b_.at<float>(ov);
+    float *const bx = b_.at<float>(obx), *const bt = b_.at<float>(obt), *const bm = b_.at<float>(obm);
+    double *const dl = b_.at<double>(ol);
+    CKR(cudaMemcpy(dth, theta, np * sizeof(float), cudaMemcpyHostToDevice));
+    CKR(cudaMemcpy(dx, x, (size_t)n * plane * kCnnIn * sizeof(float), cudaMemcpyHostToDevice));
+    CKR(cudaMemcpy(dt, t, (size_t)n * plane * sizeof(float), cudaMemcpyHostToDevice));
+    CKR(cudaMemcpy(dm, m, (size_t)n * plane * sizeof(float), cudaMemcpyHostToDevice));
+    CKR(cudaMemset(dmo, 0, np * sizeof(float)));
+    CKR(cudaMemset(dv, 0, np * sizeof(float)));
     std::vector<double> cnt(n, 0.0);
     for (int k = 0; k < n; k++)
         for (size_t q = 0; q < plane; q++) cnt[k] += m[(size_t)k * plane + q];
@@ -117,20 +121,20 @@ extern "C" int tsu_cnn_train(float *theta, const float *x, const float *t, const
             if (pos >= (size_t)n) { std::shuffle(order.begin(), order.end(), rng); pos = 0; }
             int k = order[pos++];
             bc += cnt[k];
-            CKR(cudaMemcpyAsync(bx.as<float>() + (size_t)b * plane * kCnnIn, dx.as<float>() + (size_t)k * plane * kCnnIn,
+            CKR(cudaMemcpyAsync(bx + (size_t)b * plane * kCnnIn, dx + (size_t)k * plane * kCnnIn,
                                 plane * kCnnIn * sizeof(float), cudaMemcpyDeviceToDevice, 0));
-            CKR(cudaMemcpyAsync(bt.as<float>() + (size_t)b * plane, dt.as<float>() + (size_t)k * plane,
+            CKR(cudaMemcpyAsync(bt + (size_t)b * plane, dt + (size_t)k * plane,
                                 plane * sizeof(float), cudaMemcpyDeviceToDevice, 0));
-            CKR(cudaMemcpyAsync(bm.as<float>() + (size_t)b * plane, dm.as<float>() + (size_t)k * plane,
+            CKR(cudaMemcpyAsync(bm + (size_t)b * plane, dm + (size_t)k * plane,
                                 plane * sizeof(float), cudaMemcpyDeviceToDevice, 0));
         }
-        if (cnn_loss_grad(dth.as<float>(), bx.as<float>(), bt.as<float>(), bm.as<float>(), batch, h, w, (float)bc,
-                          dws.as<float>(), dg.as<float>(), dl.as<double>(), 0))
+        if (cnn_loss_grad(dth, bx, bt, bm, batch, h, w, (float)bc,
+                          b_.at<float>(ows), dg, dl, 0))
             return TSU_ERR_CUDA;
-        if (s == 1 && loss_first) CKR(cudaMemcpy(loss_first, dl.p, sizeof(double), cudaMemcpyDeviceToHost));
-        if (cnn_adam(dth.as<float>(), dg.as<float>(), dmo.as<float>(), dv.as<float>(), np, lr, s, 0)) return TSU_ERR_CUDA;
-        if (s == steps && loss_last) CKR(cudaMemcpy(loss_last, dl.p, sizeof(double), cudaMemcpyDeviceToHost));
+        if (s == 1 && loss_first) CKR(cudaMemcpy(loss_first, dl, sizeof(double), cudaMemcpyDeviceToHost));
+        if (cnn_adam(dth, dg, dmo, dv, np, lr, s, 0)) return TSU_ERR_CUDA;
+        if (s == steps && loss_last) CKR(cudaMemcpy(loss_last, dl, sizeof(double), cudaMemcpyDeviceToHost));
     }
-    CKR(cudaMemcpy(theta, dth.p, np * sizeof(float), cudaMemcpyDeviceToHost));
+    CKR(cudaMemcpy(theta, dth, np * sizeof(float), cudaMemcpyDeviceToHost));
     return TSU_OK;
 }
