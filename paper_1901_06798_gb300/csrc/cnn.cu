@@ -38,12 +38,12 @@ __host__ __device__ inline LayerSpec layer_spec(int l)
 // The 3x3 layers forward, and backward to their inputs, are the same product: a
 // sum over the channels and taps of a plane set, in that order.  Each output used
 // to re-read its 9 CI inputs from L1 and one weight per multiply (39 us for 16 ->
-// 16 on 4 x 128^2 cells); now a CTA of 128 threads stages an 8 x 32 tile of every
+// 16 on 4 x 128^2 cells); now a CTA of 256 threads stages an 8 x 32 tile of every
 // input channel (and the layer's weights, output channel fastest) in shared
-// memory, and a thread carries two neighbouring cells' CO sums, so a 16-byte
-// weight read serves eight multiplies, paired (__ffma2_rn) over output channels.
-// The order of every sum is the one before, so the values are too.  Tiles of 256
-// cells: 4 x 128^2 cells are 256 CTAs, enough for every SM.
+// memory, and a thread carries half of the sums of two neighbouring cells, so a
+// 16-byte weight read serves eight multiplies, paired (__ffma2_rn) over output
+// channels.  The order of every sum is the one before, so the values are too.
+// Tiles of 256 cells: 4 x 128^2 cells are 256 CTAs, enough for every SM.
 constexpr int kTy = 8, kTx = 32;                       // tile of a CTA
 constexpr int kIy = kTy + 2, kIx = kTx + 2;            // its inputs
 
@@ -63,7 +63,7 @@ __device__ __forceinline__ void stage_tile(const float *__restrict__ x, float *s
 // BACK = true: y[c] = relu'(act[c]) sum_o sum_tap w[o, c, tap] x[o, cell - tap].
 // CI planes in, CO planes out; wn, wi: the layer's own output and input channels.
 template <int CI, int CO, bool BACK>
-__global__ void __launch_bounds__(128) conv3_kernel(const float *__restrict__ x, const float *__restrict__ theta, int off_w,
+__global__ void __launch_bounds__(256) conv3_kernel(const float *__restrict__ x, const float *__restrict__ theta, int off_w,
                                                     int off_b, const float *__restrict__ act, float *__restrict__ y, int H,
                                                     int W, int tiles_x, int tiles_y)
 {
@@ -75,17 +75,19 @@ __global__ void __launch_bounds__(128) conv3_kernel(const float *__restrict__ x,
     const long long plane = (long long)H * W;
     x += (long long)img * CI * plane;
     y += (long long)img * CO * plane;
-    for (int e = threadIdx.x; e < CI * 9 * CO; e += 128) {
+    for (int e = threadIdx.x; e < CI * 9 * CO; e += 256) {
         const int o = e % CO, q = e / CO, tap = q % 9, c = q / 9;   // into [c][tap][o]
         sw[e] = theta[off_w + (BACK ? (c * CO + o) : (o * CI + c)) * 9 + tap];
     }
     stage_tile<CI>(x, sx, PS, H, W, ty, tx);
     __syncthreads();
-    const int r = threadIdx.x >> 4, c0 = 2 * (threadIdx.x & 15);   // cells (ty + r, tx + c0) and the next
-    float2 acc[2][CO / 2];
+    constexpr int CH = CO / 2;                                     // output channels of a thread
+    const int oh = (threadIdx.x >> 7) * CH;                        // the first of them
+    const int r = (threadIdx.x >> 4) & 7, c0 = 2 * (threadIdx.x & 15);   // cells (ty + r, tx + c0) and the next
+    float2 acc[2][CH / 2];
 #pragma unroll
-    for (int o = 0; o < CO / 2; o++) {
-        const float2 b = BACK ? make_float2(0.0f, 0.0f) : make_float2(theta[off_b + 2 * o], theta[off_b + 2 * o + 1]);
+    for (int o = 0; o < CH / 2; o++) {
+        const float2 b = BACK ? make_float2(0.0f, 0.0f) : make_float2(theta[off_b + oh + 2 * o], theta[off_b + oh + 2 * o + 1]);
         acc[0][o] = b;
         acc[1][o] = b;
     }
@@ -101,10 +103,10 @@ __global__ void __launch_bounds__(128) conv3_kernel(const float *__restrict__ x,
 #pragma unroll
         for (int tap = 0; tap < 9; tap++) {
             const int i = BACK ? 2 - tap / 3 : tap / 3, j = BACK ? 2 - tap % 3 : tap % 3;
-            const float4 *w4 = reinterpret_cast<const float4 *>(sw + (c * 9 + tap) * CO);
+            const float4 *w4 = reinterpret_cast<const float4 *>(sw + (c * 9 + tap) * CO + oh);
             const float2 v0 = make_float2(v[i][j], v[i][j]), v1 = make_float2(v[i][j + 1], v[i][j + 1]);
 #pragma unroll
-            for (int o = 0; o < CO / 4; o++) {
+            for (int o = 0; o < CH / 4; o++) {
                 const float4 w = w4[o];
                 const float2 wa = make_float2(w.x, w.y), wb = make_float2(w.z, w.w);
                 acc[0][2 * o] = __ffma2_rn(wa, v0, acc[0][2 * o]);
@@ -122,11 +124,11 @@ __global__ void __launch_bounds__(128) conv3_kernel(const float *__restrict__ x,
         if (xx >= W) continue;
         const long long k = (long long)yy * W + xx;
 #pragma unroll
-        for (int o = 0; o < CO; o++) {
+        for (int o = 0; o < CH; o++) {
             float v = o & 1 ? acc[q][o / 2].y : acc[q][o / 2].x;
-            if (BACK) v = act[(long long)img * CO * plane + o * plane + k] > 0.0f ? v : 0.0f;
+            if (BACK) v = act[(long long)img * CO * plane + (oh + o) * plane + k] > 0.0f ? v : 0.0f;
             else v = fmaxf(v, 0.0f);
-            y[o * plane + k] = v;
+            y[(oh + o) * plane + k] = v;
         }
     }
 }
@@ -544,9 +546,9 @@ static int hidden_forward(const float *theta, const float *x, int n, int H, int 
     if (tiles > 0x7fffffffLL) return (int)cudaErrorInvalidValue;
     const unsigned grid = (unsigned)tiles;
     float *a1 = act, *a2 = act + px * HID, *a3 = act + 2 * px * HID;
-    conv3_kernel<kCnnIn, HID, false><<<grid, 128, 0, st>>>(x, theta, L0.woff, L0.boff, nullptr, a1, H, W, txs, tys);
-    conv3_kernel<HID, HID, false><<<grid, 128, 0, st>>>(a1, theta, L1.woff, L1.boff, nullptr, a2, H, W, txs, tys);
-    conv3_kernel<HID, HID, false><<<grid, 128, 0, st>>>(a2, theta, L2.woff, L2.boff, nullptr, a3, H, W, txs, tys);
+    conv3_kernel<kCnnIn, HID, false><<<grid, 256, 0, st>>>(x, theta, L0.woff, L0.boff, nullptr, a1, H, W, txs, tys);
+    conv3_kernel<HID, HID, false><<<grid, 256, 0, st>>>(a1, theta, L1.woff, L1.boff, nullptr, a2, H, W, txs, tys);
+    conv3_kernel<HID, HID, false><<<grid, 256, 0, st>>>(a2, theta, L2.woff, L2.boff, nullptr, a3, H, W, txs, tys);
     return (int)cudaGetLastError();
 }
 
@@ -600,10 +602,10 @@ int cnn_loss_grad(const float *theta, const float *x, const float *t, const floa
     const int grid = n * txs * tys, wb = std::min(grid, 152 * 2);
     // layer 3 (3x3, 16 -> 16): input a2
     wgrad3_kernel<HID><<<wb, 256, 0, st>>>(ga, a2, n, H, W, txs, tys, grad + L2.woff, grad + L2.boff);
-    conv3_kernel<HID, HID, true><<<grid, 128, 0, st>>>(ga, theta, L2.woff, 0, a2, gb, H, W, txs, tys);
+    conv3_kernel<HID, HID, true><<<grid, 256, 0, st>>>(ga, theta, L2.woff, 0, a2, gb, H, W, txs, tys);
     // layer 2: input a1
     wgrad3_kernel<HID><<<wb, 256, 0, st>>>(gb, a1, n, H, W, txs, tys, grad + L1.woff, grad + L1.boff);
-    conv3_kernel<HID, HID, true><<<grid, 128, 0, st>>>(gb, theta, L1.woff, 0, a1, ga, H, W, txs, tys);
+    conv3_kernel<HID, HID, true><<<grid, 256, 0, st>>>(gb, theta, L1.woff, 0, a1, ga, H, W, txs, tys);
     // layer 1: input x (no ReLU before it, no input gradient needed)
     wgrad3_kernel<kCnnIn><<<wb, 256, 0, st>>>(ga, x, n, H, W, txs, tys, grad + L0.woff, grad + L0.boff);
     return (int)cudaGetLastError();

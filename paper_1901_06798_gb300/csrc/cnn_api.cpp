@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstring>
 #include <algorithm>
+#include <mutex>
 #include <random>
 #include <vector>
 
@@ -16,19 +17,60 @@ using namespace tsu;
 
 namespace {
 
-// The device buffers of one call, cut out of one allocation (each cudaMalloc and
-// cudaFree takes tens of microseconds, and the calls used up to twelve)
+// The device buffers of one call, cut out of one allocation from a memory pool of
+// the process: cudaMalloc and cudaFree take tens of microseconds each and wait for
+// the device, and the calls used up to twelve of both.  The pool (one per device,
+// stream-ordered, safe from several threads) keeps at most kPoolKeep bytes between
+// calls; what is above that goes back to the device at the next synchronisation.
+constexpr unsigned long long kPoolKeep = 64ull << 20;
+constexpr int kMaxDevices = 64;
+
+cudaError_t pool_of_device(cudaMemPool_t *out)
+{
+    static std::mutex mu;
+    static cudaMemPool_t pools[kMaxDevices] = {nullptr};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!pools[dev]) {
+        cudaMemPoolProps p{};
+        p.allocType = cudaMemAllocationTypePinned;
+        p.location.type = cudaMemLocationTypeDevice;
+        p.location.id = dev;
+        cudaMemPool_t q = nullptr;
+        e = cudaMemPoolCreate(&q, &p);
+        if (e != cudaSuccess) return e;
+        unsigned long long keep = kPoolKeep;
+        e = cudaMemPoolSetAttribute(q, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(q);
+            return e;
+        }
+        pools[dev] = q;
+    }
+    *out = pools[dev];
+    return cudaSuccess;
+}
+
 struct Bufs {
     char *p = nullptr;
     size_t used = 0;
-    ~Bufs() { if (p) cudaFree(p); }
+    ~Bufs() { if (p) cudaFreeAsync(p, 0); }
     size_t want(size_t bytes)   // offset of a buffer; all are asked for before alloc()
     {
         const size_t o = used;
         used += (bytes + 255) & ~(size_t)255;
         return o;
     }
-    cudaError_t alloc() { return cudaMalloc((void **)&p, used < 256 ? 256 : used); }
+    cudaError_t alloc()
+    {
+        cudaMemPool_t pool = nullptr;
+        const cudaError_t e = pool_of_device(&pool);
+        if (e != cudaSuccess) return e;
+        return cudaMallocFromPoolAsync((void **)&p, used < 256 ? 256 : used, pool, 0);
+    }
     template <typename T> T *at(size_t off) const { return reinterpret_cast<T *>(p + off); }
 };
 
