@@ -164,12 +164,23 @@ int k_halo(int prec, const LevelView &L, const HaloMsg *msgs, int n, int cur, vo
 
 // rate of a level from the cell speeds of new patches (smax, cleared)
 int k_post_rate(const CtrlView &cv, int level, int nscen, double R, double dx, double dy, cudaStream_t st);
+// start of a step of one grid in the caller's memory (scratch pointers on the device)
+struct GridStart {
+    PatchDesc *desc;
+    double *dt;
+    float *dtf;
+    unsigned long long *smax;   // [2]
+    unsigned *count;
+    double dt_value;
+    int bc[4];
+};
+int k_grid_start(int prec, const PatchDesc &P, void *block, int cur, const GridStart &gs, cudaStream_t st);
 // what ends a level step (a.tail), as a launch of its own
 int k_tail(int prec, const StepArgs &a, cudaStream_t st);
 // end of a coarse step of a refined run: t += dt^1, gauge samples
 int k_end_step(int prec, const GaugeArgs &ga, const CtrlView &cv, cudaStream_t st);
 // maxpts: an upper bound on the output points one patch covers (sizes the grid)
-int k_read_field(int prec, const LevelView &L, int npatch, int maxpts, int cur, int scen, int field, double *dst, int nx,
+int k_read_field(int prec, const LevelView &L, int p0, int npatch, int maxpts, int cur, int scen, int field, double *dst, int nx,
                  int ny, double x0, double y0, double dx, double dy, double X0, double Y0, double dxl, double dyl,
                  cudaStream_t st);
 int k_fill(double *p, long long n, double v, cudaStream_t st);

@@ -30,54 +30,58 @@ namespace {
 
 constexpr size_t kScratchBytes = 512;               // per GPU
 constexpr size_t kDescOff = 0;                      // PatchDesc
-constexpr size_t kListOff = 256;                    // int bclist[1]
-constexpr size_t kDtOff = 272;                      // double dt
-constexpr size_t kDtfOff = 280;                     // float dt
-constexpr size_t kSmaxOff = 288;                    // unsigned long long smax[2]
-static_assert(sizeof(PatchDesc) <= kListOff, "the descriptor fits its slot");
+constexpr size_t kDtOff = 256;                      // double dt
+constexpr size_t kDtfOff = 264;                     // float dt
+constexpr size_t kCountOff = 268;                   // unsigned, CTAs done
+constexpr size_t kSmaxOff = 272;                    // unsigned long long smax[2]
+static_assert(sizeof(PatchDesc) <= kDtOff, "the descriptor fits its slot");
 constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
-std::mutex g_mu;
-void *g_scratch_ptr[kMaxDevices] = {nullptr};
+// Where the last CTA of a small grid's update leaves the two largest speeds: this
+// page of the library's own, page-locked in place (a copy of 16 bytes to pageable
+// memory costs 6 us of a 32 us call).  Calls are serialised by their caller, as for
+// the scratch; each device has its own pair.
+alignas(4096) double g_speeds[512];
 
-// Address of the scratch array on the current device, looked up once per
-// device (the host-side name of a __device__ array is not a device address).
-cudaError_t scratch_for_current_device(void **out)
+struct DeviceState {
+    void *scratch = nullptr;
+    double *speeds = nullptr;   // the device's pointer to its pair in g_speeds; null: copied instead
+};
+std::mutex g_mu;
+DeviceState g_state[kMaxDevices];
+bool g_registered = false, g_tried = false;
+
+// The scratch array's address on the current device (the host-side name of a
+// __device__ array is not a device address) and its pair of speeds, looked up once
+// per device.
+cudaError_t state_of_device(DeviceState *out, double **host_speeds)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(g_mu);
-    if (!g_scratch_ptr[dev]) {
+    DeviceState &d = g_state[dev];
+    if (!d.scratch) {
         void *p = nullptr;
         e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
         if (e != cudaSuccess) return e;
-        g_scratch_ptr[dev] = p;
+        if (!g_tried) {
+            g_tried = true;
+            g_registered = cudaHostRegister(g_speeds, sizeof g_speeds, cudaHostRegisterPortable | cudaHostRegisterMapped) == cudaSuccess;
+            if (!g_registered) cudaGetLastError();   // the copy serves as well
+        }
+        void *q = nullptr;
+        if (g_registered && cudaHostGetDevicePointer(&q, g_speeds, 0) == cudaSuccess)
+            d.speeds = static_cast<double *>(q) + 2 * dev;
+        else cudaGetLastError();
+        d.scratch = p;
     }
-    *out = g_scratch_ptr[dev];
+    *out = d;
+    *host_speeds = g_speeds + 2 * dev;
     return cudaSuccess;
-}
-
-__global__ void noalloc_prepare_kernel(unsigned char *scratch, long long fstride, int nx, int ny, int pitch, double dt)
-{
-    if (threadIdx.x != 0) return;
-    PatchDesc d;
-    memset(&d, 0, sizeof d);
-    d.off = 0;
-    d.fs = fstride;
-    d.i0 = 0; d.j0 = 0; d.nx = nx; d.ny = ny; d.pitch = pitch;
-    d.scen = 0;
-    d.bcmask = 15;
-    *reinterpret_cast<PatchDesc *>(scratch + kDescOff) = d;
-    *reinterpret_cast<int *>(scratch + kListOff) = 0;
-    *reinterpret_cast<double *>(scratch + kDtOff) = dt;
-    *reinterpret_cast<float *>(scratch + kDtfOff) = (float)dt;
-    unsigned long long *sm = reinterpret_cast<unsigned long long *>(scratch + kSmaxOff);
-    sm[0] = 0ull;
-    sm[1] = 0ull;
 }
 
 }  // namespace
@@ -105,22 +109,26 @@ extern "C" int tsu_grid_step_noalloc(int precision, void *block, int nx, int ny,
     const int nsx = (nx + W - 1) / W, nsy = (ny + rows - 1) / rows;
 
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    void *sp = nullptr;
-    if (scratch_for_current_device(&sp) != cudaSuccess) return TSU_ERR_CUDA;
-    unsigned char *scratch = reinterpret_cast<unsigned char *>(sp);
+    DeviceState ds;
+    double *host_speeds = nullptr;
+    if (state_of_device(&ds, &host_speeds) != cudaSuccess) return TSU_ERR_CUDA;
+    unsigned char *scratch = reinterpret_cast<unsigned char *>(ds.scratch);
 
-    noalloc_prepare_kernel<<<1, 32, 0, st>>>(scratch, field_stride, nx, ny, pitch, dt);
-    if (cudaGetLastError() != cudaSuccess) return TSU_ERR_CUDA;
-
-    const PatchDesc *desc = reinterpret_cast<const PatchDesc *>(scratch + kDescOff);
-    LevelView L{};
-    L.descs = desc;
-    L.arena = block;
-    L.nxl = nx;
-    L.nyl = ny;
-    BcArgs ba{reinterpret_cast<const int *>(scratch + kListOff), {bc[0], bc[1], bc[2], bc[3]}};
-    const int ring = (nx + 4) * (ny + 4) - nx * ny;
-    if (k_bc(precision, L, ba, 1, ring, cur, 1, 1, st) != 0) return TSU_ERR_CUDA;
+    PatchDesc d;
+    std::memset(&d, 0, sizeof d);
+    d.fs = field_stride;
+    d.nx = nx; d.ny = ny; d.pitch = pitch;
+    d.bcmask = 15;
+    GridStart gs{};
+    gs.desc = reinterpret_cast<PatchDesc *>(scratch + kDescOff);
+    gs.dt = reinterpret_cast<double *>(scratch + kDtOff);
+    gs.dtf = reinterpret_cast<float *>(scratch + kDtfOff);
+    gs.smax = reinterpret_cast<unsigned long long *>(scratch + kSmaxOff);
+    gs.count = reinterpret_cast<unsigned *>(scratch + kCountOff);
+    gs.dt_value = dt;
+    for (int k = 0; k < 4; k++) gs.bc[k] = bc[k];
+    if (k_grid_start(precision, d, block, cur, gs, st) != 0) return TSU_ERR_CUDA;
+    const PatchDesc *desc = gs.desc;
 
     StepArgs a{};
     a.descs = desc;
@@ -137,9 +145,20 @@ extern "C" int tsu_grid_step_noalloc(int precision, void *block, int nx, int ny,
     a.drytol = drytol;
     a.dt1f = reinterpret_cast<const float *>(scratch + kDtfOff);
     set_f32_constants(a);
+    const bool direct = ds.speeds != nullptr && nsx * nsy <= kTailMaxCtas;
+    if (direct) {
+        a.tail.count = gs.count;
+        a.tail.speeds_out = ds.speeds;
+    }
     int e = precision == TSU_F64 ? launch_step_f64(a, nsx * nsy, nt, st) : launch_step_f32p(a, nsx * nsy, nt, st);
     if (e != 0) return TSU_ERR_CUDA;
 
+    if (direct) {
+        if (cudaStreamSynchronize(st) != cudaSuccess) return TSU_ERR_CUDA;
+        max_speeds[0] = host_speeds[0];
+        max_speeds[1] = host_speeds[1];
+        return TSU_OK;
+    }
     unsigned long long bits[2] = {0ull, 0ull};
     if (cudaMemcpyAsync(bits, scratch + kSmaxOff, sizeof bits, cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return TSU_ERR_CUDA;

@@ -74,7 +74,7 @@ template <int NW> int launch_tile_nw(const StepArgs &a, int n, cudaStream_t st)
 int tile_rows_f32p(int n, const int *nx, const int *ny, int threads)
 {
     static const int cand[] = {4, 6, 8, 10, 12, 16, 20, 24, 30, 36, 44, 60};
-    constexpr double kOver = 10.0, kShare = 0.2;
+    constexpr double kOver = 16.0, kShare = 0.15;
     int best = 44;
     double bc = 1e300;
     for (int R : cand) {

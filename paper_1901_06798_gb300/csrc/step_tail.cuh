@@ -88,6 +88,11 @@ __device__ __forceinline__ bool launch_live(const StepArgs &a)
 template <typename T, bool PERT> __device__ __forceinline__ void end_level(const StepArgs &a)
 {
     const TailArgs &tl = a.tail;
+    if (tl.speeds_out != nullptr) {
+        if (threadIdx.x < 2)
+            tl.speeds_out[threadIdx.x] = __longlong_as_double((long long)atomicExch(a.smax + threadIdx.x, 0ull));
+        return;
+    }
     bool any = false;
     for (int s = threadIdx.x; s < tl.nscen; s += blockDim.x) {
         const double sx = __longlong_as_double((long long)atomicExch(tl.cv.smax + 2 * s, 0ull));

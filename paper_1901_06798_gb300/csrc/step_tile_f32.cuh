@@ -148,7 +148,7 @@ template <int NW, bool GEO, bool BULK> __device__ __forceinline__ void tile_item
     }
 
     // ---- x sweep, a row per warp
-    const float *kapP = GEO ? a.kapf + (P.j0 + 2) : nullptr;   // capacity of patch row j at kapP[j]
+    const float *rkapP = GEO ? a.rkapf + (P.j0 + 2) : nullptr;   // 1 / capacity of patch row j at rkapP[j]
     const float dtdx = dt1 * a.rdx;
     float smx = 0.0f;
     {
@@ -166,7 +166,7 @@ template <int NW, bool GEO, bool BULK> __device__ __forceinline__ void tile_item
             const int j = y0 - 2 + k;
             const bool rowint = j >= 0 && j < P.ny;
             float rk = 1.0f;
-            if (GEO) rk = 1.0f / kapP[j];
+            if (GEO) rk = rkapP[j];
             const float2 dtdxr = f2(GEO ? dtdx * rk : dtdx);
             z.h = sub(z.q0, z.B);
             W2 xw;
@@ -266,7 +266,8 @@ template <int NW, bool GEO, bool BULK> __device__ __forceinline__ void tile_item
     const int sl = (h + NW - 1) / NW;   // rows of a segment
     const int s0 = warp * sl, hs = min(sl, h - s0);
     const float dtdy = dt1 * a.rdy;
-    const float *cedP = GEO ? a.cedf + (P.j0 + 2) : nullptr;   // relative length of the y-edge below patch row j
+    const float *cedP = GEO ? a.cedf + (P.j0 + 2) : nullptr;    // relative length of the y-edge below patch row j
+    const float *cratP = GEO ? a.cratf + (P.j0 + 2) : nullptr;  // the same over the mean capacity of its two cells
     float smy = 0.0f;
     if (hs > 0) {
         const int c0 = 2 * lane;
@@ -283,7 +284,7 @@ template <int NW, bool GEO, bool BULK> __device__ __forceinline__ void tile_item
             c.q0 = ld2(r); c.ht = ld2(r + kTileRing); c.hn = ld2(r + 2 * kTileRing); c.B = ld2(r + 3 * kTileRing);
             c.h = sub(c.q0, c.B);
         };
-        auto ratio = [&](int k) { return cedP[jr + k] / (0.5f * (kapP[jr + k - 1] + kapP[jr + k])); };   // GEO, edge k >= 1
+        auto ratio = [&](int k) { return cratP[jr + k]; };   // GEO, edge k >= 1
         auto speed = [&](int k, float2 n0, float2 s2) {   // edge k bounds a row of the segment: 2 .. hs + 2
             const float cr = GEO ? ratio(k) : 1.0f;
             sp.x = fmaxf(sp.x, fmaxf(n0.x, s2.x) * cr);
@@ -303,7 +304,7 @@ template <int NW, bool GEO, bool BULK> __device__ __forceinline__ void tile_item
             load(r, c);
             float2 dtk = f2(dtdy), m0 = add(Dl[0], Su[0]);
             if (GEO) {
-                dtk = f2(dtdy / kapP[jr + k]);
+                dtk = f2(dtdy * rkapP[jr + k]);
                 m0 = fma(f2(cedP[jr + k + 1] - cedP[jr + k]), c.hn, m0);   // divergence of the edge length
             }
             float2 n0 = fnma(dtk, m0, c.q0);

@@ -344,7 +344,7 @@ struct Lvl {
     // latitude-longitude grids: physical equatorial cell sizes and the row tables
     double dxp = 0, dyp = 0;
     DevBuf<double> dKap, dCed;
-    DevBuf<float> dKapF, dCedF;
+    DevBuf<float> dKapF, dCedF, dRkapF, dCratF;
 };
 
 
@@ -479,6 +479,7 @@ struct tsu_ctx {
         a.dy = pdy(l);
         if (c.spherical) {
             a.kap = lv[l].dKap.p; a.ced = lv[l].dCed.p; a.kapf = lv[l].dKapF.p; a.cedf = lv[l].dCedF.p;
+            a.rkapf = lv[l].dRkapF.p; a.cratf = lv[l].dCratF.p;
         }
         a.tile_rows = lv[l].tile_rows;
         a.err = derr.p;
@@ -1789,7 +1790,7 @@ struct tsu_ctx {
         for (auto &L : lv) {
             L.dP.release(); L.dItems.release(); L.dNbrs.release(); L.dCmap.release(); L.dCcand.release(); L.dBc.release();
             L.dOlds.release(); L.dList.release();
-            L.dKap.release(); L.dCed.release(); L.dKapF.release(); L.dCedF.release();
+            L.dKap.release(); L.dCed.release(); L.dKapF.release(); L.dCedF.release(); L.dRkapF.release(); L.dCratF.release();
             L.dGmap.release(); L.dGoff.release(); L.dGinterp.release(); L.dGcount.release();
         }
         for (auto &g : grids) if (g.dev) cudaFreeAsync(g.dev, st);
@@ -1893,7 +1894,7 @@ int tsu_create(const tsu_config *cfg, void *cuda_stream, tsu_ctx **out)
                 L.dxp = Re * (L.dx * d2r);
                 L.dyp = Re * (L.dy * d2r);
                 std::vector<double> kap(L.nyl + 4), ced(L.nyl + 5);
-                std::vector<float> kapf(L.nyl + 4), cedf(L.nyl + 5);
+                std::vector<float> kapf(L.nyl + 4), cedf(L.nyl + 5), rkapf(L.nyl + 4), cratf(L.nyl + 4);
                 for (int J = -2; J < L.nyl + 2; J++) {
                     const double a = (c.y0 + (double)J * L.dy) * d2r, b = (c.y0 + (double)(J + 1) * L.dy) * d2r;
                     kap[J + 2] = (std::sin(b) - std::sin(a)) / (L.dy * d2r);
@@ -1903,7 +1904,12 @@ int tsu_create(const tsu_config *cfg, void *cuda_stream, tsu_ctx **out)
                     ced[J + 2] = std::cos((c.y0 + (double)J * L.dy) * d2r);
                     cedf[J + 2] = (float)ced[J + 2];
                 }
+                for (size_t k = 0; k < rkapf.size(); k++) {
+                    rkapf[k] = (float)(1.0 / kap[k]);
+                    cratf[k] = k > 0 ? (float)(ced[k] / (0.5 * (kap[k - 1] + kap[k]))) : 0.0f;
+                }
                 L.dKap.upload(kap, x->st); L.dCed.upload(ced, x->st); L.dKapF.upload(kapf, x->st); L.dCedF.upload(cedf, x->st);
+                L.dRkapF.upload(rkapf, x->st); L.dCratF.upload(cratf, x->st);
             }
         }
         const int S = x->nscen;
@@ -2169,12 +2175,18 @@ int tsu_read_field(tsu_ctx *ctx, int scen, int level, int field, double *dst, in
             // output points a patch can cover: its extent in output spacings, plus the edges
             const double sx = L.dx / dx, sy = L.dy / dy;
             long long maxpts = 1;
-            for (const auto &P : L.P) {
+            int pa = -1, pb = 0;   // the scenario's patches lie in [pa, pb)
+            for (int k = 0; k < (int)L.P.size(); k++) {
+                const PatchDesc &P = L.P[k];
+                if (P.scen != scen) continue;
+                if (pa < 0) pa = k;
+                pb = k + 1;
                 long long w = std::min<long long>(nx, (long long)std::ceil(P.nx * sx) + 3);
                 long long h = std::min<long long>(ny, (long long)std::ceil(P.ny * sy) + 3);
                 maxpts = std::max(maxpts, w * h);
             }
-            ctx->kl(k_read_field(ctx->prec, ctx->view(l), (int)L.P.size(), (int)std::min<long long>(maxpts, 1LL << 30),
+            if (pa < 0) continue;
+            ctx->kl(k_read_field(ctx->prec, ctx->view(l), pa, pb - pa, (int)std::min<long long>(maxpts, 1LL << 30),
                                  L.cur, scen, field, ctx->dstage.p, nx, ny, x0, y0, dx, dy, ctx->c.x0, ctx->c.y0, L.dx,
                                  L.dy, ctx->st),
                     "read field");

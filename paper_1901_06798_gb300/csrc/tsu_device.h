@@ -64,6 +64,7 @@ struct TailArgs {
     double *geta, *gt;
     long long *nsamp;
     double x0, y0, gdx, gdy;     // the level's origin and cell size in the gauges' coordinates
+    double *speeds_out;          // set: only the two largest speeds go there (host memory)
 };
 
 // the most CTAs of a launch that are counted: two waves of the FP32 split
@@ -92,6 +93,9 @@ struct StepArgs {
     // length of the latitude edge below row J at ced[J + 2]; null on Cartesian grids
     const double *kap, *ced;
     const float *kapf, *cedf;
+    // FP32: 1 / capacity of row J at [J + 2]; length of the edge below row J over the mean capacity of its
+    // two cells at [J + 2] (J >= -1)
+    const float *rkapf, *cratf;
     // split update (step_tile_f32.cuh, step_tile_f64.cuh): the most rows of a work item, and,
     // with null items, the tile columns of the one patch the launch covers
     int tile_rows, tile_nsx;
