@@ -38,10 +38,12 @@ template <int NW> int launch_geo(const StepArgs &a, int n, cudaStream_t st)
 int step_threads_f64(int transverse) { return transverse ? kThreadsUnsplitF64 : kThreadsF64; }
 int step_strip_width_f64(int threads, int transverse) { return transverse ? threads - 4 : d1::kCols; }
 
-// The tile height with the least FP64 work on the busiest SM.  A tile of R rows
-// costs about 2 (R + 4) warp rows of x sweep and 2 (R / 2 + 3) of y march on each
-// half of its columns (two segments); an SM's tiles share its FP64 pipe, so they
-// add up however many run at once.  At most 32 rows: three CTAs then fit on an SM.
+// The tile height with the least time on the busiest SM.  A tile of R rows costs
+// about 2 (R + 4) warp rows of x sweep and 2 (R / 2 + 3) of y march on each half of
+// its columns (two segments); an SM's tiles share its FP64 pipe, so they add up.
+// The four warps of one CTA leave the pipe idle between dependent instructions:
+// alone it takes about 1.75 times, two take 1.2 times as long per unit of work as
+// three or more, which is what fits.
 int tile_rows_f64(int n, const int *nx, const int *ny)
 {
     int best = 32;
@@ -49,7 +51,8 @@ int tile_rows_f64(int n, const int *nx, const int *ny)
     for (int R = 32; R >= 4; R -= 2) {
         double items = 0.0;
         for (int k = 0; k < n; k++) items += (double)((nx[k] + d1::kCols - 1) / d1::kCols) * ((ny[k] + R - 1) / R);
-        const double c = std::ceil(items / kSMs) * (2.0 * (R + 4) + 4.0 * (R / 2 + 3));
+        const double per = std::ceil(items / kSMs);
+        const double c = per * (2.0 * (R + 4) + 4.0 * (R / 2 + 3)) * (per <= 1 ? 1.75 : (per <= 2 ? 1.2 : 1.0));
         if (c < bc) { bc = c; best = R; }
     }
     return best;

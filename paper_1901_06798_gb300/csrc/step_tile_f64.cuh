@@ -167,6 +167,41 @@ __device__ __forceinline__ void limit_ocean(const Wave<double> &r, const double 
     F[2] = (c0 * r.Z[0][2] + c1 * z1) + c2 * r.Z[2][2];
 }
 
+// limit() of any edge.  Waves go to a side by selection (half each at speed 0); the
+// contact wave has only a transverse component here too.
+__device__ __forceinline__ void share(double z, double s, double &l, double &r)
+{
+    l = neg(s) ? z : 0.0;
+    r = neg(s) ? 0.0 : z;
+    if (zero(s)) { l = 0.5 * z; r = l; }
+}
+__device__ __forceinline__ void limit_any(const Wave<double> &r, const double (&I0)[3], double t1, const double (&I2)[3],
+                                          double dtdx, double (&am)[3], double (&ap)[3], double (&F)[3])
+{
+    double l0[3], r0[3], l2[3], r2[3], l1, r1;
+#pragma unroll
+    for (int m = 0; m < 3; m++) { share(r.Z[0][m], r.s[0], l0[m], r0[m]); share(r.Z[2][m], r.s[2], l2[m], r2[m]); }
+    const double z1 = r.Z[1][2];
+    share(z1, r.s[1], l1, r1);
+    double c0 = 0.0, c1 = 0.0, c2 = 0.0;
+    if (r.wall == 0) {
+        if (!zero(r.s[0])) c0 = factor(r.s[0], dtdx, mc_half(dot3(I0, r.Z[0]), dot3(r.Z[0], r.Z[0])));
+        if (!zero(r.s[1])) c1 = factor(r.s[1], dtdx, mc_half(t1 * z1, z1 * z1));
+        if (!zero(r.s[2])) c2 = factor(r.s[2], dtdx, mc_half(dot3(I2, r.Z[2]), dot3(r.Z[2], r.Z[2])));
+    }
+#pragma unroll
+    for (int m = 0; m < 2; m++) {
+        am[m] = l0[m] + l2[m];
+        ap[m] = r0[m] + r2[m];
+        F[m] = c0 * r.Z[0][m] + c2 * r.Z[2][m];
+    }
+    am[2] = (l0[2] + l1) + l2[2];
+    ap[2] = (r0[2] + r1) + r2[2];
+    F[2] = (c0 * r.Z[0][2] + c1 * z1) + c2 * r.Z[2][2];
+    if (r.wall == 2) { ap[0] = 0.0; ap[1] = 0.0; ap[2] = 0.0; }
+    if (r.wall == 1) { am[0] = 0.0; am[1] = 0.0; am[2] = 0.0; }
+}
+
 __device__ __forceinline__ double shfl_up1(double v) { return __shfl_up_sync(0xffffffffu, v, 1); }      // lane 0: its own
 __device__ __forceinline__ double shfl_down1(double v) { return __shfl_down_sync(0xffffffffu, v, 1); }  // lane 31: its own
 
@@ -277,7 +312,9 @@ template <int NW, bool GEO> __device__ __forceinline__ void tile64_item(const St
             L.su = shfl_up1(z[1].su); L.um = shfl_up1(z[1].um); L.pn = shfl_up1(z[1].pn); L.pt = shfl_up1(z[1].pt);
             Wave<double> e[2];
             double am[2][3], ap[2][3], F[2][3];
-            const bool oc = riemann_ocean(hg, L, z[0], e[0]) & riemann_ocean(hg, z[0], z[1], e[1]);
+            // (a row with a dry cell goes to the general solver at once)
+            const bool tried = __all_sync(ALL, wet);
+            const bool oc = tried && (riemann_ocean(hg, L, z[0], e[0]) & riemann_ocean(hg, z[0], z[1], e[1]));
             if (__all_sync(ALL, oc)) {
                 double rt[3], lt[3];
 #pragma unroll
@@ -290,17 +327,18 @@ template <int NW, bool GEO> __device__ __forceinline__ void tile64_item(const St
                     riemann<double, false>(g, L.z, z[0].z, e[0]);
                     riemann<double, false>(g, z[0].z, z[1].z, e[1]);
                 }
-                double Z0[3][3], Z1[3][3];   // upwind waves of the two edges
+                double I00[3], I02[3], I10[3], I12[3];   // upwind waves of the two edges
+                auto pick = [&](int p, int m, double &x0, double &x1) {
+                    const double l = shfl_up1(e[1].Z[p][m]), r = shfl_down1(e[0].Z[p][m]);
+                    x0 = neg(e[0].s[p]) ? e[1].Z[p][m] : l;
+                    x1 = neg(e[1].s[p]) ? r : e[0].Z[p][m];
+                };
+                double t0, t1;
 #pragma unroll
-                for (int p = 0; p < 3; p++)
-#pragma unroll
-                    for (int m = 0; m < 3; m++) {
-                        const double l = shfl_up1(e[1].Z[p][m]), r = shfl_down1(e[0].Z[p][m]);
-                        Z0[p][m] = e[0].s[p] >= 0.0 ? l : e[1].Z[p][m];
-                        Z1[p][m] = e[1].s[p] >= 0.0 ? e[0].Z[p][m] : r;
-                    }
-                limit<double>(e[0], Z0, dtdx, am[0], ap[0], F[0]);
-                limit<double>(e[1], Z1, dtdx, am[1], ap[1], F[1]);
+                for (int m = 0; m < 3; m++) { pick(0, m, I00[m], I10[m]); pick(2, m, I02[m], I12[m]); }
+                pick(1, 2, t0, t1);
+                limit_any(e[0], I00, t0, I02, dtdx, am[0], ap[0], F[0]);
+                limit_any(e[1], I10, t1, I12, dtdx, am[1], ap[1], F[1]);
             }
             if (rowint) {
 #pragma unroll
@@ -379,7 +417,9 @@ template <int NW, bool GEO> __device__ __forceinline__ void tile64_item(const St
                     if (!pder) derive(p, g);
                     derive(c, g);
                     cder = true;
-                    const bool oc = riemann_ocean(hg, p, c, wn);
+                    // (with a dry cell among the warp's, the general solver at once)
+                    const bool tried = __all_sync(ALL, c.z.wet && p.z.wet);
+                    const bool oc = tried && riemann_ocean(hg, p, c, wn);
                     okn = __all_sync(ALL, oc);
                     if (!oc) riemann<double, false>(g, p.z, c.z, wn);
                     if (counts) {
@@ -399,12 +439,13 @@ template <int NW, bool GEO> __device__ __forceinline__ void tile64_item(const St
                     if (okm) {
                         limit_ocean(wm, wn.Z[0], neg(wm.s[1]) ? wn.Z[1][2] : wo.Z[1][2], wo.Z[2], dtdy, am, ap, F);
                     } else {
-                        double ZI[3][3];
+                        double I0[3], I2[3];
 #pragma unroll
-                        for (int q = 0; q < 3; q++)
-#pragma unroll
-                            for (int m = 0; m < 3; m++) ZI[q][m] = wm.s[q] >= 0.0 ? wo.Z[q][m] : wn.Z[q][m];
-                        limit<double>(wm, ZI, dtdy, am, ap, F);
+                        for (int m = 0; m < 3; m++) {
+                            I0[m] = neg(wm.s[0]) ? wn.Z[0][m] : wo.Z[0][m];
+                            I2[m] = neg(wm.s[2]) ? wn.Z[2][m] : wo.Z[2][m];
+                        }
+                        limit_any(wm, I0, neg(wm.s[1]) ? wn.Z[1][2] : wo.Z[1][2], I2, dtdy, am, ap, F);
                     }
                 }
                 if (k >= 4) {
@@ -474,7 +515,7 @@ template <int NW, bool GEO> __device__ __forceinline__ void tile64_item(const St
     }
 }
 
-template <int NW, bool GEO> __global__ void __launch_bounds__(NW * 32) step_tile_f64(StepArgs a)
+template <int NW, bool GEO> __global__ void __launch_bounds__(NW * 32, NW >= 8 ? 1 : 12 / NW) step_tile_f64(StepArgs a)
 {
     if (!launch_live(a)) return;
     tile64_item<NW, GEO>(a, blockIdx.x);
