@@ -226,6 +226,7 @@ __global__ void ghost_map_kernel(LevelView L, GhostSrc *gmap, int2 *ilist, int *
 template <typename T>
 __global__ void ghost_copy_kernel(LevelView L, int cur, int *err)
 {
+    chain_begin();
     const PatchDesc P = L.descs[blockIdx.x];
     const int n = ring_count(P);
     Acc<T> a = acc<T>(L.arena, P);
@@ -251,6 +252,7 @@ template <typename T, bool PERT>
 __global__ void ghost_interp_kernel(LevelView L, LevelView C, int cur, int cur_c, int ratio, double alpha,
                                     double drytol, int *err)
 {
+    chain_begin();
     const int ni = *L.icount;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < ni; e += gridDim.x * blockDim.x) {
         const int2 pg = L.ilist[e];
@@ -316,6 +318,7 @@ __device__ __forceinline__ void begin_step(const CtrlView &cv, const BeginArgs &
 template <typename T>
 __global__ void bc_kernel(LevelView L, int cur, BcArgs bcs, int do_state, int do_B, CtrlView cv, BeginArgs bg)
 {
+    chain_begin();
     if (bg.nscen > 0 && blockIdx.x + 1 == gridDim.x) {
         if (blockIdx.y == 0) begin_step(cv, bg);
         return;
@@ -346,6 +349,7 @@ __global__ void bc_kernel(LevelView L, int cur, BcArgs bcs, int do_state, int do
 template <typename T>
 __global__ void grid_start_kernel(PatchDesc P, void *block, int cur, GridStart gs)
 {
+    chain_begin();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *gs.desc = P;
         *gs.dt = gs.dt_value;
@@ -976,7 +980,11 @@ __global__ void post_rate_kernel(CtrlView cv, int level, int nscen, double R, do
 }
 
 // the end of a level step whose update launch does not count its CTAs
-template <typename T, bool PERT> __global__ void tail_kernel(StepArgs a) { end_level<T, PERT>(a); }
+template <typename T, bool PERT> __global__ void tail_kernel(StepArgs a)
+{
+    chain_begin();
+    end_level<T, PERT>(a);
+}
 
 // ---------------------------------------------------------------- gauges, fields
 
@@ -1196,13 +1204,12 @@ int k_ghost_fill(int prec, const LevelView &L, const LevelView &C, int npatch, i
 {
     if (npatch <= 0) return 0;
     dim3 g = npatch >= 152 * 8 ? dim3(npatch, 1) : grid_for(maxring, npatch, 128);
-    if (prec == 0) ghost_copy_kernel<double><<<g, 128, 0, st>>>(L, cur, err);
-    else ghost_copy_kernel<float><<<g, 128, 0, st>>>(L, cur, err);
-    int e = (int)cudaGetLastError();
+    int e = prec == 0 ? launch_chained(ghost_copy_kernel<double>, g, 128, 0, st, L, cur, err)
+                      : launch_chained(ghost_copy_kernel<float>, g, 128, 0, st, L, cur, err);
     if (e != 0 || ratio <= 0) return e;
     // the list's length is known on the device only: a fixed grid strides over it
-    TSU_DISPATCH(prec, ghost_interp_kernel, <<<152 * 8, 128, 0, st>>>(L, C, cur, cur_c, ratio, alpha, drytol, err));
-    return (int)cudaGetLastError();
+    if (prec == 0) return launch_chained(ghost_interp_kernel<double, false>, 152 * 8, 128, 0, st, L, C, cur, cur_c, ratio, alpha, drytol, err);
+    return launch_chained(ghost_interp_kernel<float, true>, 152 * 8, 128, 0, st, L, C, cur, cur_c, ratio, alpha, drytol, err);
 }
 
 int k_bc(int prec, const LevelView &L, const BcArgs &b, int nlist, int maxring, int cur, int do_state, int do_B,
@@ -1213,9 +1220,8 @@ int k_bc(int prec, const LevelView &L, const BcArgs &b, int nlist, int maxring, 
     if (bg) g.x++;
     const CtrlView c = cv ? *cv : CtrlView{};
     const BeginArgs a = bg ? *bg : BeginArgs{};
-    if (prec == 0) bc_kernel<double><<<g, 128, 0, st>>>(L, cur, b, do_state, do_B, c, a);
-    else bc_kernel<float><<<g, 128, 0, st>>>(L, cur, b, do_state, do_B, c, a);
-    return (int)cudaGetLastError();
+    if (prec == 0) return launch_chained(bc_kernel<double>, g, 128, 0, st, L, cur, b, do_state, do_B, c, a);
+    return launch_chained(bc_kernel<float>, g, 128, 0, st, L, cur, b, do_state, do_B, c, a);
 }
 
 int k_average(int prec, const LevelView &F, const LevelView &C, int npatch, int maxcells, int cur_f, int cur_c, int r,
@@ -1453,15 +1459,14 @@ int k_grid_start(int prec, const PatchDesc &P, void *block, int cur, const GridS
 {
     const long long ring = (long long)(P.nx + 4) * (P.ny + 4) - (long long)P.nx * P.ny;
     const int blocks = (int)std::min<long long>((ring + 127) / 128, 152 * 16);
-    if (prec == 0) grid_start_kernel<double><<<blocks, 128, 0, st>>>(P, block, cur, gs);
-    else grid_start_kernel<float><<<blocks, 128, 0, st>>>(P, block, cur, gs);
-    return (int)cudaGetLastError();
+    if (prec == 0) return launch_chained(grid_start_kernel<double>, blocks, 128, 0, st, P, block, cur, gs);
+    return launch_chained(grid_start_kernel<float>, blocks, 128, 0, st, P, block, cur, gs);
 }
 
 int k_tail(int prec, const StepArgs &a, cudaStream_t st)
 {
-    TSU_DISPATCH(prec, tail_kernel, <<<1, 128, 0, st>>>(a));
-    return (int)cudaGetLastError();
+    if (prec == 0) return launch_chained(tail_kernel<double, false>, 1, 128, 0, st, a);
+    return launch_chained(tail_kernel<float, true>, 1, 128, 0, st, a);
 }
 
 int k_post_rate(const CtrlView &cv, int level, int nscen, double R, double dx, double dy, cudaStream_t st)

@@ -42,8 +42,7 @@ template <int NW, bool GEO, bool BULK> int launch_tile(const StepArgs &a, int n,
     static unsigned long long told = 0;
     const int e = allow_smem(step_tile_f32<NW, GEO, BULK>, told);
     if (e) return e;
-    step_tile_f32<NW, GEO, BULK><<<n, NW * 32, tile_smem(a.tile_rows), st>>>(a);
-    return (int)cudaGetLastError();
+    return launch_chained(step_tile_f32<NW, GEO, BULK>, n, NW * 32, tile_smem(a.tile_rows), st, a);
 }
 
 template <bool GEO> int launch_retake(const StepArgs &a, int n, cudaStream_t st)
@@ -53,8 +52,8 @@ template <bool GEO> int launch_retake(const StepArgs &a, int n, cudaStream_t st)
     if (e) return e;
     StepArgs b = a;
     b.n_items = n;
-    retake_tile_f32<GEO><<<std::min(n, kSMs * tile_ctas(a.tile_rows, 128)), 128, tile_smem(a.tile_rows), st>>>(b);
-    return (int)cudaGetLastError();
+    return launch_chained(retake_tile_f32<GEO>, std::min(n, kSMs * tile_ctas(a.tile_rows, 128)), 128, tile_smem(a.tile_rows),
+                          st, b);
 }
 
 template <int NW> int launch_tile_nw(const StepArgs &a, int n, cudaStream_t st)

@@ -24,8 +24,13 @@ template <int NW, bool GEO> int launch_tile(const StepArgs &a, int n, cudaStream
         if (e != cudaSuccess) return (int)e;
         if (dev < 64) told |= 1ull << dev;
     }
-    step_tile_f64<NW, GEO><<<n, NW * 32, tile_smem(a.tile_rows), st>>>(a);
-    return (int)cudaGetLastError();
+    // (not launched ahead of the boundaries' end: placed around CTAs that are still
+    // there, the tiles spread unevenly over the SMs, 0.33 -> 0.52 ms on 512^2 cells)
+    if (a.gate == nullptr) {
+        step_tile_f64<NW, GEO><<<n, NW * 32, tile_smem(a.tile_rows), st>>>(a);
+        return (int)cudaGetLastError();
+    }
+    return launch_chained(step_tile_f64<NW, GEO>, n, NW * 32, tile_smem(a.tile_rows), st, a);
 }
 
 template <int NW> int launch_geo(const StepArgs &a, int n, cudaStream_t st)

@@ -9,6 +9,7 @@
 // more than with none.
 #pragma once
 #include <cuda_runtime.h>
+#include "chain.cuh"
 #include "tsu_device.h"
 
 namespace tsu {
@@ -78,10 +79,11 @@ __device__ __forceinline__ double gauge_eta(const PatchDesc &P, const T *blk, in
     return __dadd_rn(a, __dmul_rn(ty, __dadd_rn(b, -a)));
 }
 
-// whether this launch has anything to do: a retake launch (a.gate set) has not
+// First call of every patch-update kernel: whether this launch has anything to do: a retake launch (a.gate set) has not
 // when no scenario is marked
 __device__ __forceinline__ bool launch_live(const StepArgs &a)
 {
+    chain_begin();
     return a.gate == nullptr || a.tail.any_retake == nullptr || *a.tail.any_retake != 0;
 }
 

@@ -350,8 +350,7 @@ int launch_unsplit_f32_nt(const StepArgs &a, int n_items, cudaStream_t st)
         if (e != cudaSuccess) return (int)e;
         configured = true;
     }
-    step_unsplit_f32_kernel<NT, RING><<<n_items, NT, bytes, st>>>(a);
-    return (int)cudaGetLastError();
+    return launch_chained(step_unsplit_f32_kernel<NT, RING>, n_items, NT, bytes, st, a);
 }
 
 }  // namespace tsu
