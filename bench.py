@@ -86,15 +86,15 @@ def peaks():
 
 def kernel_hash():
     h = hashlib.sha256()
-    for f in ("step_kernel.cuh", "step_f32x2.cuh", "step_split_f32.cuh", "step_f32p.cu", "step_f64.cu", "tsu_device.h"):
+    for f in ("step_kernel.cuh", "step_f32x2.cuh", "step_tile_f32.cuh", "step_tile_f64.cuh", "step_f32p.cu", "step_f64.cu",
+              "tsu_device.h"):
         h.update(open(os.path.join(ROOT, "paper_1901_06798_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
 
 def ncu_traffic(prec):
-    """DRAM bytes of one patch update (the x- and y-sweep kernels of the FP32
-    split update together) from the committed ncu summary, only if it was taken
-    on the current kernel sources."""
+    """DRAM bytes of one patch update from the committed ncu summary, only if it
+    was taken on the current kernel sources."""
     p = os.path.join(ROOT, "profiles", "step_kernel_traffic.json")
     if not os.path.exists(p):
         return None
@@ -466,7 +466,6 @@ def run_config4(args, stream, torch):
         if use:
             ctx.cnn_set_weights(theta)
         W.load(ctx, dict(w, cfg=cfg))
-        ctx.set_tuning(64 if prec == B.TSU_F64 else 32, 32)
         torch.cuda.synchronize()
         t0 = time.perf_counter()
         misses, checked, done = 0, 0, 0
@@ -677,7 +676,7 @@ def main():
                                "the CFL check, the level-1 retake launch and its check, gauge sampling"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm, "traffic": traffic,
-                         "kernel": "patch update = step_x_f32x2 + step_y_f32x2 (one launch each per step)",
+                         "kernel": "patch update = step_tile_f32 (one launch per step) and the retake launch, which leaves at once",
                          "kernel_ms": r["kernel_ms"],
                          "bytes_per_launch": bpl, "peak_source": src},
             # the other roof of the same update: algorithmic flops against the FP32 pipes; neither

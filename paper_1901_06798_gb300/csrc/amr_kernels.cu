@@ -224,15 +224,16 @@ __global__ void ghost_map_kernel(LevelView L, GhostSrc *gmap, int2 *ilist, int *
 // the map names.  The interpolated cells are left to the kernel below, so
 // that no CTA here waits on their long chains of dependent loads.
 template <typename T>
-__global__ void ghost_copy_kernel(LevelView L, int cur, int *err)
+__global__ void ghost_copy_kernel(LevelView L, int cur, int *err, const int *list)
 {
     chain_begin();
-    const PatchDesc P = L.descs[blockIdx.x];
+    const int patch = list ? list[blockIdx.x] : blockIdx.x;
+    const PatchDesc P = L.descs[patch];
     const int n = ring_count(P);
     Acc<T> a = acc<T>(L.arena, P);
     T *q0 = a.f(cur, 0), *q1 = a.f(cur, 1), *q2 = a.f(cur, 2);
     const T *ar = reinterpret_cast<const T *>(L.arena);
-    const GhostSrc *gm = L.gmap + L.goff[blockIdx.x];
+    const GhostSrc *gm = L.gmap + L.goff[patch];
     for (int g = blockIdx.y * blockDim.x + threadIdx.x; g < n; g += gridDim.y * blockDim.x) {
         const GhostSrc s = gm[g];
         if (s.src == kGhostSkip || s.src == kGhostInterp) continue;
@@ -1200,12 +1201,16 @@ int k_ghost_map(const LevelView &L, GhostSrc *gmap, int2 *ilist, int *icount, in
 }
 
 int k_ghost_fill(int prec, const LevelView &L, const LevelView &C, int npatch, int maxring, int cur, int cur_c,
-                 int ratio, double alpha, double drytol, int *err, cudaStream_t st)
+                 int ratio, double alpha, double drytol, int *err, const int *list, int nlist, cudaStream_t st)
 {
     if (npatch <= 0) return 0;
-    dim3 g = npatch >= 152 * 8 ? dim3(npatch, 1) : grid_for(maxring, npatch, 128);
-    int e = prec == 0 ? launch_chained(ghost_copy_kernel<double>, g, 128, 0, st, L, cur, err)
-                      : launch_chained(ghost_copy_kernel<float>, g, 128, 0, st, L, cur, err);
+    const int nc = list ? nlist : npatch;
+    int e = 0;
+    if (nc > 0) {
+        dim3 g = nc >= 152 * 8 ? dim3(nc, 1) : grid_for(maxring, nc, 128);
+        e = prec == 0 ? launch_chained(ghost_copy_kernel<double>, g, 128, 0, st, L, cur, err, list)
+                      : launch_chained(ghost_copy_kernel<float>, g, 128, 0, st, L, cur, err, list);
+    }
     if (e != 0 || ratio <= 0) return e;
     // the list's length is known on the device only: a fixed grid strides over it
     if (prec == 0) return launch_chained(ghost_interp_kernel<double, false>, 152 * 8, 128, 0, st, L, C, cur, cur_c, ratio, alpha, drytol, err);

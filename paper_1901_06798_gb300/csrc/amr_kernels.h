@@ -8,19 +8,6 @@ namespace tsu {
 
 constexpr int kMaxLevels = 8;
 
-// Where one ghost cell of a patch takes its value from, found once per patch
-// table (the search over the neighbour boxes does not run at every fill):
-// src >= 0 is the element offset in the arena of the same-level neighbour's
-// interior cell in field 0 of buffer 0, sfs that patch's field stride; the
-// negative codes below mark the other cases.
-struct __align__(16) GhostSrc {
-    long long src;
-    long long sfs;
-};
-constexpr long long kGhostSkip = -1;     // outside the level's index space (physical boundary)
-constexpr long long kGhostInterp = -2;   // no same-level neighbour: space-time interpolation from the coarser level
-constexpr long long kGhostNone = -3;     // no neighbour on the coarsest level: a tiling error
-
 // Device view of one level's tables (all scenarios).
 struct LevelView {
     const PatchDesc *descs;
@@ -114,8 +101,10 @@ struct GaugeArgs {
 // (ilist, icount: the interpolated cells' list and its length, zeroed here; ilist holds one entry per ghost cell)
 int k_ghost_map(const LevelView &L, GhostSrc *gmap, int2 *ilist, int *icount, int npatch, int maxring, int ratio,
                 cudaStream_t st);
+// list (set: nlist entries): copy the ghost cells of these patches only (the FP32 split update reads the others'
+// from their sources); the interpolation always runs over the whole level
 int k_ghost_fill(int prec, const LevelView &L, const LevelView &C, int npatch, int maxring, int cur, int cur_c,
-                 int ratio, double alpha, double drytol, int *err, cudaStream_t st);
+                 int ratio, double alpha, double drytol, int *err, const int *list, int nlist, cudaStream_t st);
 // bg (level 1): the same launch starts the coarse step (dt^1 from the rates)
 int k_bc(int prec, const LevelView &L, const BcArgs &b, int nlist, int maxring, int cur, int do_state, int do_B,
          cudaStream_t st, const CtrlView *cv = nullptr, const BeginArgs *bg = nullptr);

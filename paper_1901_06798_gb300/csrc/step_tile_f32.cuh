@@ -135,7 +135,67 @@ template <int NW, bool GEO, bool BULK> __device__ __forceinline__ void tile_item
             }
         }
         cp_async_commit();
+    }
+    if (!BULK && a.gmap != nullptr && P.bcmask == 0) {
+        // Ghost cells from the cells that hold them (16 level-3 steps between regrids
+        // used to copy them to the patches' rings first: 94 us a step of 7000 patches,
+        // bound by 8 bytes of every 32-byte sector).  The first ones of a thread are
+        // on their way while the rows land.  Cells without such a source
+        // (interpolated) are in the ring already.
+        const int nb = y0 == 0 ? 2 : 0, nt = y0 + h == P.ny ? 2 : 0, nl = x0 == 0 ? 2 : 0, nr = x0 + w == P.nx ? 2 : 0;
+        const int rows2 = nb + nt, cols2 = nl + nr, nrow = rows2 * ncols, total = nrow + (nrows - rows2) * cols2;
+        const GhostSrc *gm = a.gmap + a.goff[it.patch];
+        const float *ar = reinterpret_cast<const float *>(a.arena);
+        // ghost cell e of the tile: its place in the tile and its source (null: none)
+        auto find = [&](int e, float *&to, long long &sf) -> const float * {
+            int k, c;
+            if (e < nrow) {
+                const int r = e / ncols;
+                c = e - r * ncols;
+                k = r < nb ? r : nrows - nt + (r - nb);
+            } else {
+                const int r = (e - nrow) / cols2, q = (e - nrow) - r * cols2;
+                k = nb + r;
+                c = q < nl ? q : ncols - nr + (q - nl);
+            }
+            const int i = x0 - 2 + c, j = y0 - 2 + k, Wr = P.nx + 4;
+            const int gi = j < 0 ? (j + 2) * Wr + i + 2 : (j >= P.ny ? (2 + j - P.ny) * Wr + i + 2 : 4 * Wr + 4 * j + (i < 0 ? i + 2 : 2 + i - P.nx));
+            const GhostSrc s = gm[gi];
+            to = tile + k * kTileRow + c;
+            sf = s.sfs;
+            if (s.src == kGhostNone && a.err) atomicOr(a.err, 1);
+            return s.src >= 0 ? ar + s.src + (long long)(cur * 3) * s.sfs : nullptr;
+        };
+        constexpr int HOLD = 4;
+        float *to[HOLD];
+        float v[HOLD][3];
+#pragma unroll
+        for (int q = 0; q < HOLD; q++) {
+            const int e = t + q * NT;
+            to[q] = nullptr;
+            if (e < total) {
+                float *p;
+                long long sf;
+                const float *s = find(e, p, sf);
+                if (s != nullptr) {
+                    to[q] = p;
+                    v[q][0] = s[0]; v[q][1] = s[sf]; v[q][2] = s[2 * sf];
+                }
+            }
+        }
         cp_async_wait<0>();
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < HOLD; q++)
+            if (to[q] != nullptr) { to[q][0] = v[q][0]; to[q][kTileRing] = v[q][1]; to[q][2 * kTileRing] = v[q][2]; }
+        for (int e = t + HOLD * NT; e < total; e += NT) {
+            float *p;
+            long long sf;
+            const float *s = find(e, p, sf);
+            if (s != nullptr) { p[0] = s[0]; p[kTileRing] = s[sf]; p[2 * kTileRing] = s[2 * sf]; }
+        }
+    } else {
+        if (!BULK) cp_async_wait<0>();
     }
     __syncthreads();
     if (ncols < kTileRing) {   // columns past a narrow tile repeat its last: no waves between them

@@ -463,6 +463,21 @@ struct tsu_ctx {
 
     // ------------------------------------------------------------ helpers
     bool split_f32() const { return prec != TSU_F64 && c.transverse == 0; }
+    // the update's tiles read their ghost cells from the cells that hold them (bulk
+    // copies bring whole rows of the patch's own storage)
+    bool gathers() const { return split_f32() && !bulk_rows; }
+    // ghost cells of level l before a step: copies from same-level patches (where the
+    // update does not read them itself: it does for patches away from the domain's
+    // edges, whose boundary rules need the ring in place) and interpolation
+    void fill_ghosts(int l, double alpha)
+    {
+        Lvl &L = lv[l];
+        const LevelView Cv = l > 0 ? view(l - 1) : view(l);
+        const int nc = gathers() ? (int)L.bclist.size() : (int)L.P.size();
+        kl(k_ghost_fill(prec, view(l), Cv, (int)L.P.size(), L.maxring, L.cur, l > 0 ? lv[l - 1].cur : 0,
+                        l > 0 ? ratio[l - 1] : 0, alpha, c.drytol, derr.p, gathers() ? L.dBc.p : nullptr, nc, st), "ghost fill");
+        launches += (nc > 0 ? 1 : 0) + (l > 0 ? 1 : 0) - 1;   // the copies' and the interpolated cells' kernels
+    }
     int nt() const
     {
         if (step_nt > 0) return step_nt;
@@ -482,6 +497,10 @@ struct tsu_ctx {
             a.rkapf = lv[l].dRkapF.p; a.cratf = lv[l].dCratF.p;
         }
         a.tile_rows = lv[l].tile_rows;
+        if (gathers()) {
+            a.gmap = lv[l].dGmap.p;
+            a.goff = lv[l].dGoff.p;
+        }
         a.err = derr.p;
         a.bulk_rows = bulk_rows;
         a.wait_polls = wait_polls;
@@ -1215,11 +1234,7 @@ struct tsu_ctx {
         const int n = (int)L.P.size();
         if (n == 0) return;
         if (l > 0 || n > 1) {
-            double alpha = l > 0 ? (double)k / (double)ratio[l - 1] : 0.0;
-            LevelView Cv = l > 0 ? view(l - 1) : view(l);
-            kl(k_ghost_fill(prec, view(l), Cv, n, L.maxring, L.cur, l > 0 ? lv[l - 1].cur : 0,
-                            l > 0 ? ratio[l - 1] : 0, alpha, c.drytol, derr.p, st), "ghost fill");
-            if (l > 0) launches++;   // the interpolated cells' kernel
+            fill_ghosts(l, l > 0 ? (double)k / (double)ratio[l - 1] : 0.0);
         }
         if (!L.bclist.empty()) {   // never empty on level 1, which covers the domain
             BcArgs ba{L.dBc.p, {c.bc[0], c.bc[1], c.bc[2], c.bc[3]}};
@@ -2492,10 +2507,7 @@ int tsu_time_level1_steps(tsu_ctx *ctx, int warmup, int n, double *kernel_ms_out
         for (int k = 0; k < n; k++) {
             // the kernels of level_step and coarse_step, with an event on either side of
             // the update (its retake launch included)
-            if (L.P.size() > 1) {
-                ctx->kl(k_ghost_fill(ctx->prec, ctx->view(0), ctx->view(0), (int)L.P.size(), L.maxring, L.cur, 0, 0, 0.0,
-                                     ctx->c.drytol, ctx->derr.p, ctx->st), "ghost fill");
-            }
+            if (L.P.size() > 1) ctx->fill_ghosts(0, 0.0);
             BcArgs ba{L.dBc.p, {ctx->c.bc[0], ctx->c.bc[1], ctx->c.bc[2], ctx->c.bc[3]}};
             const CtrlView cv = ctx->ctrl();
             const BeginArgs bg{ctx->nscen, ctx->nlev, ctx->Rl.p, ctx->c.cfl_desired, ctx->c.dt_max};

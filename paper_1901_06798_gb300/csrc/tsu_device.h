@@ -23,6 +23,19 @@ struct PatchDesc {
     int old_off, old_cnt;      // old same-level patches overlapping (regrid initialisation)
 };
 
+// Where one ghost cell of a patch takes its value from, found once per patch
+// table (the search over the neighbour boxes does not run at every fill):
+// src >= 0 is the element offset in the arena of the same-level neighbour's
+// interior cell in field 0 of buffer 0, sfs that patch's field stride; the
+// negative codes below mark the other cases.
+struct __align__(16) GhostSrc {
+    long long src;
+    long long sfs;
+};
+constexpr long long kGhostSkip = -1;     // outside the level's index space (physical boundary)
+constexpr long long kGhostInterp = -2;   // no same-level neighbour: space-time interpolation from the coarser level
+constexpr long long kGhostNone = -3;     // no neighbour on the coarsest level: a tiling error
+
 // One work item of the patch update: a strip of columns [x0, x0+w) and a row
 // segment [y0, y0+h) of one patch (patch-local interior indices).
 struct StepItem {
@@ -99,6 +112,11 @@ struct StepArgs {
     // split update (step_tile_f32.cuh, step_tile_f64.cuh): the most rows of a work item, and,
     // with null items, the tile columns of the one patch the launch covers
     int tile_rows, tile_nsx;
+    // FP32 split update: ghost-cell sources of the level's patches in ghost-ring order, patch k's from
+    // gmap[goff[k]]; a tile of a patch inside the domain takes its ghost cells from there (null: from the
+    // patch's own ghost ring)
+    const GhostSrc *gmap;
+    const long long *goff;
     // CFL retake of a level-1 step: when set, a work item of scenario s runs
     // only if gate[s] != 0 (null: every item runs)
     const int *gate;
