@@ -142,7 +142,8 @@ template <int NW, bool GEO, bool BULK> __device__ __forceinline__ void tile_item
         // bound by 8 bytes of every 32-byte sector).  The first ones of a thread are
         // on their way while the rows land.  Cells without such a source
         // (interpolated) are in the ring already.
-        const int nb = y0 == 0 ? 2 : 0, nt = y0 + h == P.ny ? 2 : 0, nl = x0 == 0 ? 2 : 0, nr = x0 + w == P.nx ? 2 : 0;
+        // (a strip or segment one cell short of the patch's edge has one ghost column or row)
+        const int nb = max(0, 2 - y0), nt = max(0, y0 + h + 2 - P.ny), nl = max(0, 2 - x0), nr = max(0, x0 + w + 2 - P.nx);
         const int rows2 = nb + nt, cols2 = nl + nr, nrow = rows2 * ncols, total = nrow + (nrows - rows2) * cols2;
         const GhostSrc *gm = a.gmap + a.goff[it.patch];
         const float *ar = reinterpret_cast<const float *>(a.arena);
