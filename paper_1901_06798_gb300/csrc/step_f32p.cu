@@ -3,6 +3,7 @@
 // is formed from eta' directly, so still water is exactly still and the
 // ocean-depth cancellation of h + B never enters the flux.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include "step_tile_f32.cuh"
 
@@ -26,12 +27,12 @@ int tile_ctas(int rows, int threads)
 }
 
 // above 48 KiB of dynamic shared memory a kernel has to be told so, once per device
-template <typename K> int allow_smem(K kernel, unsigned long long &told)
+template <typename K> int allow_smem(K kernel, std::atomic<unsigned long long> &told)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return (int)e;
-    if (dev < 64 && (told >> dev & 1)) return 0;
+    if (dev < 64 && (told.load() >> dev & 1)) return 0;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_smem(kTileRowsMax));
     if (e == cudaSuccess && dev < 64) told |= 1ull << dev;
     return (int)e;
@@ -39,7 +40,7 @@ template <typename K> int allow_smem(K kernel, unsigned long long &told)
 
 template <int NW, bool GEO, bool BULK> int launch_tile(const StepArgs &a, int n, cudaStream_t st)
 {
-    static unsigned long long told = 0;
+    static std::atomic<unsigned long long> told{0};
     const int e = allow_smem(step_tile_f32<NW, GEO, BULK>, told);
     if (e) return e;
     return launch_chained(step_tile_f32<NW, GEO, BULK>, n, NW * 32, tile_smem(a.tile_rows), st, a);
@@ -47,7 +48,7 @@ template <int NW, bool GEO, bool BULK> int launch_tile(const StepArgs &a, int n,
 
 template <bool GEO> int launch_retake(const StepArgs &a, int n, cudaStream_t st)
 {
-    static unsigned long long told = 0;
+    static std::atomic<unsigned long long> told{0};
     const int e = allow_smem(retake_tile_f32<GEO>, told);
     if (e) return e;
     StepArgs b = a;
@@ -74,11 +75,11 @@ int tile_rows_f32p(int n, const int *nx, const int *ny, int threads)
 {
     static const int cand[] = {4, 6, 8, 10, 12, 16, 20, 24, 30, 36, 44, 60};
     constexpr double kOver = 16.0, kShare = 0.15;
+    const std::vector<double> strips = strips_by_height(n, nx, ny, kTileCols);
     int best = 44;
     double bc = 1e300;
     for (int R : cand) {
-        double items = 0.0;
-        for (int k = 0; k < n; k++) items += (double)((nx[k] + kTileCols - 1) / kTileCols) * ((ny[k] + R - 1) / R);
+        const double items = tile_count(strips, R);
         const int occ = tile_ctas(R, threads);
         const double per = items / kSMs, full = std::floor(per / occ), rest = std::ceil(per - full * occ - 1e-9);
         const double one = R + kOver;
@@ -97,11 +98,11 @@ int unsplit_rows(int n, const int *nx, const int *ny, int threads, int precision
     static const int cand[] = {8, 12, 16, 24, 32, 48, 64};
     const bool f64 = precision == 0;
     const int W = threads - 4, occ = std::max(1, 512 / threads);
+    const std::vector<double> strips = strips_by_height(n, nx, ny, W);
     int best = f64 ? 128 : 64;
     double bc = 1e300;
     for (int R : cand) {
-        double items = 0.0;
-        for (int k = 0; k < n; k++) items += (double)((nx[k] + W - 1) / W) * ((ny[k] + R - 1) / R);
+        const double items = tile_count(strips, R);
         const double per = items / kSMs, full = std::floor(per / occ), rest = std::ceil(per - full * occ - 1e-9);
         const double one = R + 6;
         const double c = f64 ? std::ceil(per) * one

@@ -1,6 +1,7 @@
 // step_f64.cu -- FP64 split update (step_tile_f64.cuh).  Built with --fmad=false so
 // every multiply and add rounds exactly as the FP64 oracle's.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include "step_tile_f64.cuh"
 
@@ -15,11 +16,11 @@ int tile_smem(int rows) { return (rows + 4) * d1::kRow * (int)sizeof(double); }
 template <int NW, bool GEO> int launch_tile(const StepArgs &a, int n, cudaStream_t st)
 {
     // above 48 KiB of dynamic shared memory a kernel has to be told so, once per device
-    static unsigned long long told = 0;
+    static std::atomic<unsigned long long> told{0};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return (int)e;
-    if (dev >= 64 || !(told >> dev & 1)) {
+    if (dev >= 64 || !(told.load() >> dev & 1)) {
         e = cudaFuncSetAttribute(step_tile_f64<NW, GEO>, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_smem(kTileRowsMaxF64));
         if (e != cudaSuccess) return (int)e;
         if (dev < 64) told |= 1ull << dev;
@@ -51,12 +52,11 @@ int step_strip_width_f64(int threads, int transverse) { return transverse ? thre
 // three or more, which is what fits.
 int tile_rows_f64(int n, const int *nx, const int *ny)
 {
+    const std::vector<double> strips = strips_by_height(n, nx, ny, d1::kCols);
     int best = 32;
     double bc = 1e300;
     for (int R = 32; R >= 4; R -= 2) {
-        double items = 0.0;
-        for (int k = 0; k < n; k++) items += (double)((nx[k] + d1::kCols - 1) / d1::kCols) * ((ny[k] + R - 1) / R);
-        const double per = std::ceil(items / kSMs);
+        const double per = std::ceil(tile_count(strips, R) / kSMs);
         const double c = per * (2.0 * (R + 4) + 4.0 * (R / 2 + 3)) * (per <= 1 ? 1.75 : (per <= 2 ? 1.2 : 1.0));
         if (c < bc) { bc = c; best = R; }
     }
