@@ -261,17 +261,17 @@ int tsu_get_stats(tsu_ctx *ctx, int scenario, tsu_stats *out);
 /* Launch shape of the patch update (the autotuner's knobs): step_threads
  * threads per CTA and seg_rows rows per CTA (patches taller than that are cut
  * into row segments).  step_threads is 64, 128 or 256, or also 32 for the
- * split FP32 update.  A CTA updates a strip of 2 step_threads - 4 columns in
- * the split FP32 update (two columns per thread), step_threads - 4 otherwise.
- * The split FP32 update runs as two kernels: the knobs shape its x-sweep
- * kernel (rows counted over the patch's ghost rows too); its y-sweep kernel
- * always takes strips of 64 columns and 64 rows.  0 restores the defaults.
- * Results do not depend on either.  Returns TSU_ERR_ARG for any other value. */
+ * split FP32 update.  A CTA updates a tile of 60 columns in the split updates
+ * and a strip of step_threads - 4 columns in the unsplit ones.  In the split
+ * FP32 update seg_rows (up to 124) sets the tiles' height, in the other updates
+ * it bounds the height that the size of the level suggests.  0 restores the
+ * defaults.  Results do not depend on either.  Returns TSU_ERR_ARG for any
+ * other value. */
 int tsu_set_tuning(tsu_ctx *ctx, int step_threads, int seg_rows);
 
-/* How the FP32 split update's x-sweep kernel brings rows into shared memory.
- * enable = 0 (the default): every thread copies its own columns with
- * cp.async.  enable = 1: one thread copies each field's row segment with a
+/* How the FP32 split update brings its tiles into shared memory.
+ * enable = 0 (the default): every thread copies its share of the rows with
+ * cp.async, ghost cells from the patches that hold them.  enable = 1: one thread copies each field's row segment with a
  * bulk copy (cp.async.bulk) that completes on an mbarrier, and every thread
  * polls that barrier at most `polls` times before it gives up (2^22 is far
  * above what a copy takes).  A wait that runs out stops the work item's
@@ -321,9 +321,8 @@ int tsu_level1_buffers(tsu_ctx *ctx, void **h, void **hu, void **hv, void **B, i
 
 /* Per-level timing of the patch update, for measurement.  enable != 0 starts
  * recording a pair of CUDA events on the library's stream around the update
- * launches of every level step (the x- and y-sweep kernels of the FP32 split
- * update, the fused FP64 kernel, and on level 1 the retake launch with its
- * bookkeeping kernel); coarse steps then run without graphs.  Either call
+ * launch of every level step (and on level 1 the retake launch with the end of
+ * the step); coarse steps then run without graphs.  Either call
  * drops what was recorded so far.  Synchronises the stream. */
 int tsu_profile_levels(tsu_ctx *ctx, int enable);
 
@@ -432,10 +431,11 @@ int tsu_cnn_features(tsu_ctx *ctx, int scenario, int level, float *features, uns
  * stream) before it returns, so it must not be issued while that stream is
  * being captured into a CUDA graph.
  *
- * It allocates nothing: its scratch (about 1 MiB, mostly the work-item table)
- * is a file-scope __device__ array that every GPU loading the library holds
- * until the process exits.  The first call on a device looks up that array's
- * address (once per device, with that device current).  Every call shares the
+ * It allocates nothing: its scratch is a file-scope __device__ array of 512
+ * bytes that every GPU loading the library holds until the process exits, and
+ * a host page of the library's that the device writes the speeds to.  The
+ * first call looks up that array's address (once per device, with that device
+ * current) and page-locks the host page.  Every call shares the
  * array and leaves its contents behind; each call rewrites what it uses and
  * clears the speed accumulator, but calls that overlap on the GPU (other
  * streams or host threads) race on it -- serialise them.

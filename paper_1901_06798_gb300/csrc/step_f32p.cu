@@ -71,6 +71,11 @@ template <int NW> int launch_tile_nw(const StepArgs &a, int n, cudaStream_t st)
 // the y march); a second to fourth CTA on an SM slows the others by kShare each
 // (they share the issue slots that one leaves free); tiles come in waves of as
 // many CTAs as fit.
+// Both sides of its choices, update alone, developed sea unless noted (us at rows 44 / 20 / 8):
+// 4096^2 259 / 309 / 466 (it takes 44), 1531 x 1213 69.5 / 59.2 / 72.7 (24: 60.5),
+// 500^2 41.0 / 30.0 / 29.3 (16: 27.2), 200^2 25.0 / 19.4 / 16.8 (12: 17.3); 7000 patches of
+// 60^2, 16 steps: 6.7 ms at 60, 7.7 at 20, 8.8 at 16.  With 64 or 256 threads in place of 128
+// the best heights take 269 and 289 us at 4096^2.
 int tile_rows_f32p(int n, const int *nx, const int *ny, int threads)
 {
     static const int cand[] = {4, 6, 8, 10, 12, 16, 20, 24, 30, 36, 44, 60};
@@ -93,6 +98,8 @@ int tile_rows_f32p(int n, const int *nx, const int *ny, int threads)
 // of which sweeps 4 more and fills its pipeline.  FP32: about 16 warps run on an
 // SM, which share its issue slots as the tiles' do.  FP64: an SM's CTAs share its
 // FP64 pipe, so their times add up.
+// Both sides (us): FP32 1024^2 took 172 with rows by a fixed 64, 70 with the rule's, 86 with 12;
+// FP32 300^2 37 with the rule's and 45 with 64 threads; 2500^2 289 (rule), 286 to 298 at others.
 int unsplit_rows(int n, const int *nx, const int *ny, int threads, int precision)
 {
     static const int cand[] = {8, 12, 16, 24, 32, 48, 64};

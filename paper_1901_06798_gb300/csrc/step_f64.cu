@@ -50,6 +50,10 @@ int step_strip_width_f64(int threads, int transverse) { return transverse ? thre
 // The four warps of one CTA leave the pipe idle between dependent instructions:
 // alone it takes about 1.75 times, two take 1.2 times as long per unit of work as
 // three or more, which is what fits.
+// Both sides (us, developed sea): 771 x 602 543 with the rule's height, 941 with 16 rows,
+// 687 with 12; 512^2 325 and 380 with 12; 2048^2 3972 and 4124 with 24.  256 threads in place
+// of 128: 350 at 512^2, 595 at 771 x 602, but 115 against 127 at 200^2 and 241 against 333 where
+// most of 512^2 is at rest; 64 threads: 398, 568, 191, 467.
 int tile_rows_f64(int n, const int *nx, const int *ny)
 {
     const std::vector<double> strips = strips_by_height(n, nx, ny, d1::kCols);
