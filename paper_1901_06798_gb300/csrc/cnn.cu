@@ -13,6 +13,7 @@
 #include <cstdint>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include "chain.cuh"
 #include "cnn.h"
 
 namespace tsu {
@@ -62,15 +63,17 @@ __device__ __forceinline__ void stage_tile(const float *__restrict__ x, float *s
 // BACK = false: y[o] = relu(b[o] + sum_c sum_tap w[o, c, tap] x[c, cell + tap]);
 // BACK = true: y[c] = relu'(act[c]) sum_o sum_tap w[o, c, tap] x[o, cell - tap].
 // CI planes in, CO planes out; wn, wi: the layer's own output and input channels.
+// s: kConvSmem<CI, CO> floats, 16-byte aligned.
+template <int CI, int CO> constexpr int kConvSmem = CI * kIy * kIx + CI * 9 * CO;
 template <int CI, int CO, bool BACK>
-__global__ void __launch_bounds__(256) conv3_kernel(const float *__restrict__ x, const float *__restrict__ theta, int off_w,
-                                                    int off_b, const float *__restrict__ act, float *__restrict__ y, int H,
-                                                    int W, int tiles_x, int tiles_y)
+__device__ __forceinline__ void conv3_tile(float *s, int tile, const float *__restrict__ x, const float *__restrict__ theta,
+                                           int off_w, int off_b, const float *__restrict__ act, float *__restrict__ y, int H,
+                                           int W, int tiles_x, int tiles_y)
 {
     constexpr int PS = kIy * kIx;
-    __shared__ __align__(16) float sx[CI * PS];
-    __shared__ __align__(16) float sw[CI * 9 * CO];
-    const int img = blockIdx.x / (tiles_x * tiles_y), tq = blockIdx.x - img * (tiles_x * tiles_y);
+    static_assert(CI * PS % 4 == 0, "the weights are read 16 bytes at a time");
+    float *sx = s, *sw = s + CI * PS;
+    const int img = tile / (tiles_x * tiles_y), tq = tile - img * (tiles_x * tiles_y);
     const int ty = (tq / tiles_x) * kTy, tx = (tq % tiles_x) * kTx;
     const long long plane = (long long)H * W;
     x += (long long)img * CI * plane;
@@ -133,6 +136,15 @@ __global__ void __launch_bounds__(256) conv3_kernel(const float *__restrict__ x,
     }
 }
 
+template <int CI, int CO>
+__global__ void __launch_bounds__(256) conv3_kernel(const float *__restrict__ x, const float *__restrict__ theta, int off_w,
+                                                    int off_b, float *__restrict__ y, int H, int W, int tiles_x, int tiles_y)
+{
+    __shared__ __align__(16) float s[kConvSmem<CI, CO>];
+    chain_begin();
+    conv3_tile<CI, CO, false>(s, blockIdx.x, x, theta, off_w, off_b, nullptr, y, H, W, tiles_x, tiles_y);
+}
+
 // The 1x1 head on its own (inference in FP32)
 __global__ void head_kernel(const float *__restrict__ a3, const float *__restrict__ theta, int off_w, int off_b,
                             float *__restrict__ z, int n, long long plane)
@@ -156,6 +168,7 @@ __global__ void __launch_bounds__(128) head_loss_kernel(const float *__restrict_
                                                         long long total, long long plane, float inv_count, float *ga, float *gw,
                                                         float *gb, double *loss)
 {
+    chain_begin();
     float w[HID], dw[HID], db = 0.0f;
     double part = 0.0;
 #pragma unroll
@@ -213,16 +226,18 @@ __global__ void __launch_bounds__(128) head_loss_kernel(const float *__restrict_
 // units of 16 cells, 18 paired multiply-adds for one 16-byte and three 4-byte reads.
 // The threads that are left over split the units.  A CTA adds up several tiles
 // before it adds its sums to the result, one atomic per weight.
+// CTA `block` of `blocks`; s: kGradSmem<CI> floats, 16-byte aligned.
+template <int CI> constexpr int kGradSmem = kTy * kTx * HID + CI * (kIy * kIx + 1);
 template <int CI>
-__global__ void __launch_bounds__(256) wgrad3_kernel(const float *__restrict__ g, const float *__restrict__ a, int n, int H,
-                                                     int W, int tiles_x, int tiles_y, float *gw, float *gb)
+__device__ __forceinline__ void wgrad3_tiles(float *s, int block, int blocks, const float *__restrict__ g,
+                                             const float *__restrict__ a, int n, int H, int W, int tiles_x, int tiles_y,
+                                             float *gw, float *gb)
 {
     constexpr int PS = kIy * kIx + 1;          // odd: channels fall on different banks
     constexpr int NC = 4 * CI;                 // (channel, four outputs) pairs
     constexpr int SUB = 256 / NC;              // threads per pair
     constexpr int UNITS = kTy * kTx / 16;      // units of 16 cells of a row
-    __shared__ float sa[CI * PS];
-    __shared__ __align__(16) float sg[kTy * kTx * HID];
+    float *sg = s, *sa = s + kTy * kTx * HID;
     const long long plane = (long long)H * W;
     const int pair = threadIdx.x % NC, sub = threadIdx.x / NC;
     const int c = pair % CI, og = pair / CI;
@@ -231,7 +246,7 @@ __global__ void __launch_bounds__(256) wgrad3_kernel(const float *__restrict__ g
     for (int q = 0; q < 9; q++) { acc[q][0] = make_float2(0.0f, 0.0f); acc[q][1] = make_float2(0.0f, 0.0f); }
     bs[0] = make_float2(0.0f, 0.0f); bs[1] = make_float2(0.0f, 0.0f);
     const int ntile = n * tiles_x * tiles_y;
-    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+    for (int tile = block; tile < ntile; tile += blocks) {
         const int img = tile / (tiles_x * tiles_y), q = tile - img * (tiles_x * tiles_y);
         const int ty = (q / tiles_x) * kTy, tx = (q % tiles_x) * kTx;
         __syncthreads();   // the last tile has been used
@@ -272,9 +287,9 @@ __global__ void __launch_bounds__(256) wgrad3_kernel(const float *__restrict__ g
     float *red = sg;   // [HID][CI][9] and the bias sums: fits in the g tile
     static_assert(HID * CI * 9 + HID <= kTy * kTx * HID, "the sums fit");
     for (int e = threadIdx.x; e < HID * CI * 9 + HID; e += 256) red[e] = 0.0f;
-    for (int s = 0; s < SUB; s++) {
+    for (int q = 0; q < SUB; q++) {
         __syncthreads();
-        if (sub == s) {
+        if (sub == q) {
 #pragma unroll
             for (int t = 0; t < 9; t++) {
                 float *d = red + ((4 * og) * CI + c) * 9 + t;
@@ -292,6 +307,31 @@ __global__ void __launch_bounds__(256) wgrad3_kernel(const float *__restrict__ g
     __syncthreads();
     for (int e = threadIdx.x; e < HID * CI * 9; e += 256) atomicAdd(gw + e, red[e]);
     if (threadIdx.x < HID) atomicAdd(gb + threadIdx.x, red[HID * CI * 9 + threadIdx.x]);
+}
+
+template <int CI>
+__global__ void __launch_bounds__(256) wgrad3_kernel(const float *__restrict__ g, const float *__restrict__ a, int n, int H,
+                                                     int W, int tiles_x, int tiles_y, float *gw, float *gb)
+{
+    __shared__ __align__(16) float s[kGradSmem<CI>];
+    chain_begin();
+    wgrad3_tiles<CI>(s, blockIdx.x, gridDim.x, g, a, n, H, W, tiles_x, tiles_y, gw, gb);
+}
+
+// A hidden layer's backward pass in one launch: the first wb CTAs sum its weight
+// gradients, the others form the gradient of its input.  Both only read g, and each
+// alone leaves an SM waiting most of the time (1.7 CTAs of 8 warps an SM).  With the
+// launches of the pass overlapping their starts (chain.cuh), the gradient of four
+// 128^2 images takes 261 us where it took 270, the copies from the host included.
+__global__ void __launch_bounds__(256) back3_kernel(const float *__restrict__ g, const float *__restrict__ a,
+                                                    const float *__restrict__ theta, int off_w, float *__restrict__ gx, int n,
+                                                    int H, int W, int tiles_x, int tiles_y, float *gw, float *gb, int wb)
+{
+    constexpr int S1 = kGradSmem<HID>, S2 = kConvSmem<HID, HID>;
+    __shared__ __align__(16) float s[S1 > S2 ? S1 : S2];
+    chain_begin();
+    if ((int)blockIdx.x < wb) wgrad3_tiles<HID>(s, blockIdx.x, wb, g, a, n, H, W, tiles_x, tiles_y, gw, gb);
+    else conv3_tile<HID, HID, true>(s, blockIdx.x - wb, g, theta, off_w, 0, a, gx, H, W, tiles_x, tiles_y);
 }
 
 __global__ void adam_kernel(float *theta, const float *grad, float *m, float *v, int np, float lr, float b1, float b2,
@@ -546,10 +586,11 @@ static int hidden_forward(const float *theta, const float *x, int n, int H, int 
     if (tiles > 0x7fffffffLL) return (int)cudaErrorInvalidValue;
     const unsigned grid = (unsigned)tiles;
     float *a1 = act, *a2 = act + px * HID, *a3 = act + 2 * px * HID;
-    conv3_kernel<kCnnIn, HID, false><<<grid, 256, 0, st>>>(x, theta, L0.woff, L0.boff, nullptr, a1, H, W, txs, tys);
-    conv3_kernel<HID, HID, false><<<grid, 256, 0, st>>>(a1, theta, L1.woff, L1.boff, nullptr, a2, H, W, txs, tys);
-    conv3_kernel<HID, HID, false><<<grid, 256, 0, st>>>(a2, theta, L2.woff, L2.boff, nullptr, a3, H, W, txs, tys);
-    return (int)cudaGetLastError();
+    int e = launch_chained(conv3_kernel<kCnnIn, HID>, grid, 256, 0, st, x, theta, L0.woff, L0.boff, a1, H, W, txs, tys);
+    if (e) return e;
+    e = launch_chained(conv3_kernel<HID, HID>, grid, 256, 0, st, a1, theta, L1.woff, L1.boff, a2, H, W, txs, tys);
+    if (e) return e;
+    return launch_chained(conv3_kernel<HID, HID>, grid, 256, 0, st, a2, theta, L2.woff, L2.boff, a3, H, W, txs, tys);
 }
 
 int cnn_forward(const float *theta, const float *x, int n, int H, int W, bool fp16, float *act, float *logits,
@@ -596,19 +637,22 @@ int cnn_loss_grad(const float *theta, const float *x, const float *t, const floa
     const int e = hidden_forward(theta, x, n, H, W, act, st);
     if (e) return e;
     // head (1x1, 16 -> 1)
-    head_loss_kernel<<<(int)std::min<long long>((px + 127) / 128, 152 * 8), 128, 0, st>>>(
-        a3, theta, L3.woff, L3.boff, t, m, px, plane, mcount > 0 ? 1.0f / mcount : 0.0f, ga, grad + L3.woff, grad + L3.boff, loss);
+    int r = launch_chained(head_loss_kernel, (unsigned)std::min<long long>((px + 127) / 128, 152 * 8), 128, 0, st, a3, theta, L3.woff,
+                           L3.boff, t, m, px, plane, mcount > 0 ? 1.0f / mcount : 0.0f, ga, grad + L3.woff, grad + L3.boff, loss);
+    if (r) return r;
     const int txs = (W + kTx - 1) / kTx, tys = (H + kTy - 1) / kTy;
-    const int grid = n * txs * tys, wb = std::min(grid, 152 * 2);
+    const int grid = n * txs * tys, wb = std::min(grid, 152 * 2);   // hidden_forward has refused grids above 2^31 - 1
+    if (grid > 0x7fffffff - wb) return (int)cudaErrorInvalidValue;
     // layer 3 (3x3, 16 -> 16): input a2
-    wgrad3_kernel<HID><<<wb, 256, 0, st>>>(ga, a2, n, H, W, txs, tys, grad + L2.woff, grad + L2.boff);
-    conv3_kernel<HID, HID, true><<<grid, 256, 0, st>>>(ga, theta, L2.woff, 0, a2, gb, H, W, txs, tys);
+    r = launch_chained(back3_kernel, grid + wb, 256, 0, st, ga, a2, theta, L2.woff, gb, n, H, W, txs, tys, grad + L2.woff,
+                           grad + L2.boff, wb);
+    if (r) return r;
     // layer 2: input a1
-    wgrad3_kernel<HID><<<wb, 256, 0, st>>>(gb, a1, n, H, W, txs, tys, grad + L1.woff, grad + L1.boff);
-    conv3_kernel<HID, HID, true><<<grid, 256, 0, st>>>(gb, theta, L1.woff, 0, a1, ga, H, W, txs, tys);
+    r = launch_chained(back3_kernel, grid + wb, 256, 0, st, gb, a1, theta, L1.woff, ga, n, H, W, txs, tys, grad + L1.woff,
+                       grad + L1.boff, wb);
+    if (r) return r;
     // layer 1: input x (no ReLU before it, no input gradient needed)
-    wgrad3_kernel<kCnnIn><<<wb, 256, 0, st>>>(ga, x, n, H, W, txs, tys, grad + L0.woff, grad + L0.boff);
-    return (int)cudaGetLastError();
+    return launch_chained(wgrad3_kernel<kCnnIn>, wb, 256, 0, st, ga, x, n, H, W, txs, tys, grad + L0.woff, grad + L0.boff);
 }
 
 int cnn_adam(float *theta, const float *grad, float *m, float *v, int np, float lr, int t, cudaStream_t st)
