@@ -12,7 +12,11 @@
 
 namespace tsu {
 
-// first statement of every kernel that is launched by launch_chained
+// First statement of every kernel that is launched by launch_chained.  Such a kernel
+// runs while the kernel before it still writes, so no pointer of it, or of a function
+// it calls, is __restrict__: that would promise data that never changes while the
+// kernel runs, and let the compiler load it ahead of the wait or past the coherent
+// caches.
 __device__ __forceinline__ void chain_begin()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -50,7 +50,7 @@ constexpr int kIy = kTy + 2, kIx = kTx + 2;            // its inputs
 
 // a tile of CI planes with its margin, zero outside the plane; plane stride ps floats
 template <int CI>
-__device__ __forceinline__ void stage_tile(const float *__restrict__ x, float *s, int ps, int H, int W, int ty, int tx)
+__device__ __forceinline__ void stage_tile(const float *x, float *s, int ps, int H, int W, int ty, int tx)
 {
     const long long plane = (long long)H * W;
     for (int e = threadIdx.x; e < CI * kIy * kIx; e += blockDim.x) {
@@ -66,9 +66,8 @@ __device__ __forceinline__ void stage_tile(const float *__restrict__ x, float *s
 // s: kConvSmem<CI, CO> floats, 16-byte aligned.
 template <int CI, int CO> constexpr int kConvSmem = CI * kIy * kIx + CI * 9 * CO;
 template <int CI, int CO, bool BACK>
-__device__ __forceinline__ void conv3_tile(float *s, int tile, const float *__restrict__ x, const float *__restrict__ theta,
-                                           int off_w, int off_b, const float *__restrict__ act, float *__restrict__ y, int H,
-                                           int W, int tiles_x, int tiles_y)
+__device__ __forceinline__ void conv3_tile(float *s, int tile, const float *x, const float *theta, int off_w, int off_b,
+                                           const float *act, float *y, int H, int W, int tiles_x, int tiles_y)
 {
     constexpr int PS = kIy * kIx;
     static_assert(CI * PS % 4 == 0, "the weights are read 16 bytes at a time");
@@ -126,19 +125,20 @@ __device__ __forceinline__ void conv3_tile(float *s, int tile, const float *__re
         const int xx = tx + c0 + q;
         if (xx >= W) continue;
         const long long k = (long long)yy * W + xx;
+        float v[CH], a[CH];   // (all loads before the first store: the compiler may not move one past the other)
 #pragma unroll
         for (int o = 0; o < CH; o++) {
-            float v = o & 1 ? acc[q][o / 2].y : acc[q][o / 2].x;
-            if (BACK) v = act[(long long)img * CO * plane + (oh + o) * plane + k] > 0.0f ? v : 0.0f;
-            else v = fmaxf(v, 0.0f);
-            y[(oh + o) * plane + k] = v;
+            v[o] = o & 1 ? acc[q][o / 2].y : acc[q][o / 2].x;
+            a[o] = BACK ? act[((long long)img * CO + oh + o) * plane + k] : 0.0f;
         }
+#pragma unroll
+        for (int o = 0; o < CH; o++) y[(oh + o) * plane + k] = BACK ? (a[o] > 0.0f ? v[o] : 0.0f) : fmaxf(v[o], 0.0f);
     }
 }
 
 template <int CI, int CO>
-__global__ void __launch_bounds__(256) conv3_kernel(const float *__restrict__ x, const float *__restrict__ theta, int off_w,
-                                                    int off_b, float *__restrict__ y, int H, int W, int tiles_x, int tiles_y)
+__global__ void __launch_bounds__(256) conv3_kernel(const float *x, const float *theta, int off_w, int off_b, float *y, int H,
+                                                    int W, int tiles_x, int tiles_y)
 {
     __shared__ __align__(16) float s[kConvSmem<CI, CO>];
     chain_begin();
@@ -163,9 +163,8 @@ __global__ void head_kernel(const float *__restrict__ a3, const float *__restric
 // the logit z, g = dL/dz = (sigmoid(z) - t) m / M and the loss, the head's weight
 // and bias gradients, and dL/d(a3) times ReLU'.  As four kernels they read a3 three
 // times, and the weight gradient alone took 381 us.
-__global__ void __launch_bounds__(128) head_loss_kernel(const float *__restrict__ a3, const float *__restrict__ theta, int off_w,
-                                                        int off_b, const float *__restrict__ t, const float *__restrict__ m,
-                                                        long long total, long long plane, float inv_count, float *ga, float *gw,
+__global__ void __launch_bounds__(128) head_loss_kernel(const float *a3, const float *theta, int off_w, int off_b,
+                                                        const float *t, const float *m, long long total, long long plane, float inv_count, float *ga, float *gw,
                                                         float *gb, double *loss)
 {
     chain_begin();
@@ -229,8 +228,7 @@ __global__ void __launch_bounds__(128) head_loss_kernel(const float *__restrict_
 // CTA `block` of `blocks`; s: kGradSmem<CI> floats, 16-byte aligned.
 template <int CI> constexpr int kGradSmem = kTy * kTx * HID + CI * (kIy * kIx + 1);
 template <int CI>
-__device__ __forceinline__ void wgrad3_tiles(float *s, int block, int blocks, const float *__restrict__ g,
-                                             const float *__restrict__ a, int n, int H, int W, int tiles_x, int tiles_y,
+__device__ __forceinline__ void wgrad3_tiles(float *s, int block, int blocks, const float *g, const float *a, int n, int H, int W, int tiles_x, int tiles_y,
                                              float *gw, float *gb)
 {
     constexpr int PS = kIy * kIx + 1;          // odd: channels fall on different banks
@@ -310,8 +308,8 @@ __device__ __forceinline__ void wgrad3_tiles(float *s, int block, int blocks, co
 }
 
 template <int CI>
-__global__ void __launch_bounds__(256) wgrad3_kernel(const float *__restrict__ g, const float *__restrict__ a, int n, int H,
-                                                     int W, int tiles_x, int tiles_y, float *gw, float *gb)
+__global__ void __launch_bounds__(256) wgrad3_kernel(const float *g, const float *a, int n, int H, int W,
+                                                     int tiles_x, int tiles_y, float *gw, float *gb)
 {
     __shared__ __align__(16) float s[kGradSmem<CI>];
     chain_begin();
@@ -323,9 +321,8 @@ __global__ void __launch_bounds__(256) wgrad3_kernel(const float *__restrict__ g
 // alone leaves an SM waiting most of the time (1.7 CTAs of 8 warps an SM).  With the
 // launches of the pass overlapping their starts (chain.cuh), the gradient of four
 // 128^2 images takes 261 us where it took 270, the copies from the host included.
-__global__ void __launch_bounds__(256) back3_kernel(const float *__restrict__ g, const float *__restrict__ a,
-                                                    const float *__restrict__ theta, int off_w, float *__restrict__ gx, int n,
-                                                    int H, int W, int tiles_x, int tiles_y, float *gw, float *gb, int wb)
+__global__ void __launch_bounds__(256) back3_kernel(const float *g, const float *a, const float *theta, int off_w,
+                                                    float *gx, int n, int H, int W, int tiles_x, int tiles_y, float *gw, float *gb, int wb)
 {
     constexpr int S1 = kGradSmem<HID>, S2 = kConvSmem<HID, HID>;
     __shared__ __align__(16) float s[S1 > S2 ? S1 : S2];
