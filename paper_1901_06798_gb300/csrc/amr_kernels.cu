@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 #include <type_traits>
 #include "amr_kernels.h"
+#include "boundary.h"
 #include "step_tail.cuh"
 
 namespace tsu {
@@ -281,24 +282,11 @@ __global__ void ghost_interp_kernel(LevelView L, LevelView C, int cur, int cur_c
 __device__ __forceinline__ bool bc_source(const PatchDesc &P, int nxl, int nyl, const int *bc, int i, int j, int &si,
                                           int &sj, bool &negx, bool &negy)
 {
-    int I = P.i0 + i, J = P.j0 + j;
-    bool out = false;
-    si = i; sj = j; negx = false; negy = false;
-    if (I < 0) {
-        out = true;
-        if (bc[0] == 0) { si = (-1 - I) - P.i0; negx = true; } else si = -P.i0;
-    } else if (I >= nxl) {
-        out = true;
-        if (bc[1] == 0) { si = (2 * nxl - 1 - I) - P.i0; negx = true; } else si = nxl - 1 - P.i0;
-    }
-    if (J < 0) {
-        out = true;
-        if (bc[2] == 0) { sj = (-1 - J) - P.j0; negy = true; } else sj = -P.j0;
-    } else if (J >= nyl) {
-        out = true;
-        if (bc[3] == 0) { sj = (2 * nyl - 1 - J) - P.j0; negy = true; } else sj = nyl - 1 - P.j0;
-    }
-    return out;
+    const bool ox = boundary_source(P.i0 + i, nxl, bc[0], bc[1], si, negx);
+    const bool oy = boundary_source(P.j0 + j, nyl, bc[2], bc[3], sj, negy);
+    si -= P.i0;
+    sj -= P.j0;
+    return ox || oy;
 }
 
 // Start of a coarse step: dt^1 = min(dt_max, nu_d / max_l(rate_l / R_l)).
