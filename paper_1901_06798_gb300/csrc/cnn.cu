@@ -162,14 +162,15 @@ __global__ void head_kernel(const float *__restrict__ a3, const float *__restric
 // The head, its loss and its backward pass in one pass over the last activations:
 // the logit z, g = dL/dz = (sigmoid(z) - t) m / M and the loss, the head's weight
 // and bias gradients, and dL/d(a3) times ReLU'.  As four kernels they read a3 three
-// times, and the weight gradient alone took 381 us.
+// times, and the weight gradient alone took 381 us.  A CTA's sums go to its own place
+// in part (weights, then the bias) and lpart (grad_sum_kernel adds them up).
 __global__ void __launch_bounds__(128) head_loss_kernel(const float *a3, const float *theta, int off_w, int off_b,
-                                                        const float *t, const float *m, long long total, long long plane, float inv_count, float *ga, float *gw,
-                                                        float *gb, double *loss)
+                                                        const float *t, const float *m, long long total, long long plane, float inv_count, float *ga, float *part,
+                                                        double *lpart)
 {
     chain_begin();
     float w[HID], dw[HID], db = 0.0f;
-    double part = 0.0;
+    double ls = 0.0;
 #pragma unroll
     for (int c = 0; c < HID; c++) { w[c] = theta[off_w + c]; dw[c] = 0.0f; }
     const float b = theta[off_b];
@@ -184,7 +185,7 @@ __global__ void __launch_bounds__(128) head_loss_kernel(const float *a3, const f
         const float sg = 1.0f / (1.0f + __expf(-zz));
         const float g = (sg - tt) * mm * inv_count;
         const float l = fmaxf(zz, 0.0f) - zz * tt + log1pf(__expf(-fabsf(zz)));
-        part += (double)(l * mm);
+        ls += (double)(l * mm);
         db += g;
 #pragma unroll
         for (int c = 0; c < HID; c++) {
@@ -197,7 +198,7 @@ __global__ void __launch_bounds__(128) head_loss_kernel(const float *a3, const f
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        part += __shfl_xor_sync(0xffffffffu, part, o);
+        ls += __shfl_xor_sync(0xffffffffu, ls, o);
         db += __shfl_xor_sync(0xffffffffu, db, o);
 #pragma unroll
         for (int c = 0; c < HID; c++) dw[c] += __shfl_xor_sync(0xffffffffu, dw[c], o);
@@ -206,14 +207,13 @@ __global__ void __launch_bounds__(128) head_loss_kernel(const float *a3, const f
 #pragma unroll
         for (int c = 0; c < HID; c++) red[warp][c] = dw[c];
         red[warp][HID] = db;
-        redl[warp] = part;
+        redl[warp] = ls;
     }
     __syncthreads();
-    if (threadIdx.x <= HID) {
-        const float v = (red[0][threadIdx.x] + red[1][threadIdx.x]) + (red[2][threadIdx.x] + red[3][threadIdx.x]);
-        atomicAdd(threadIdx.x < HID ? gw + threadIdx.x : gb, v);
-    }
-    if (threadIdx.x == 32) atomicAdd(loss, ((redl[0] + redl[1]) + (redl[2] + redl[3])) * (double)inv_count);
+    if (threadIdx.x <= HID)
+        part[blockIdx.x * (HID + 1) + threadIdx.x] =
+            (red[0][threadIdx.x] + red[1][threadIdx.x]) + (red[2][threadIdx.x] + red[3][threadIdx.x]);
+    if (threadIdx.x == 32) lpart[blockIdx.x] = ((redl[0] + redl[1]) + (redl[2] + redl[3])) * (double)inv_count;
 }
 
 // Weight and bias gradients of a 3x3 layer: dW[o, c, tap] = sum over cells of g[o,
@@ -223,13 +223,14 @@ __global__ void __launch_bounds__(128) head_loss_kernel(const float *a3, const f
 // (g with the channels together), and a thread owns one input channel and four
 // output channels: their 36 sums stay in registers while a 3 x 3 window slides along
 // units of 16 cells, 18 paired multiply-adds for one 16-byte and three 4-byte reads.
-// The threads that are left over split the units.  A CTA adds up several tiles
-// before it adds its sums to the result, one atomic per weight.
+// The threads that are left over split the units.  A CTA's sums, over several tiles
+// where there are more than kGradCtas, go to its own place in part (weights, then
+// biases: the layer's slice of the parameter vector); grad_sum_kernel adds them up.
 // CTA `block` of `blocks`; s: kGradSmem<CI> floats, 16-byte aligned.
 template <int CI> constexpr int kGradSmem = kTy * kTx * HID + CI * (kIy * kIx + 1);
 template <int CI>
 __device__ __forceinline__ void wgrad3_tiles(float *s, int block, int blocks, const float *g, const float *a, int n, int H, int W, int tiles_x, int tiles_y,
-                                             float *gw, float *gb)
+                                             float *part)
 {
     constexpr int PS = kIy * kIx + 1;          // odd: channels fall on different banks
     constexpr int NC = 4 * CI;                 // (channel, four outputs) pairs
@@ -303,17 +304,16 @@ __device__ __forceinline__ void wgrad3_tiles(float *s, int block, int blocks, co
         }
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < HID * CI * 9; e += 256) atomicAdd(gw + e, red[e]);
-    if (threadIdx.x < HID) atomicAdd(gb + threadIdx.x, red[HID * CI * 9 + threadIdx.x]);
+    for (int e = threadIdx.x; e < HID * CI * 9 + HID; e += 256) part[(long long)block * (HID * CI * 9 + HID) + e] = red[e];
 }
 
 template <int CI>
 __global__ void __launch_bounds__(256) wgrad3_kernel(const float *g, const float *a, int n, int H, int W,
-                                                     int tiles_x, int tiles_y, float *gw, float *gb)
+                                                     int tiles_x, int tiles_y, float *part)
 {
     __shared__ __align__(16) float s[kGradSmem<CI>];
     chain_begin();
-    wgrad3_tiles<CI>(s, blockIdx.x, gridDim.x, g, a, n, H, W, tiles_x, tiles_y, gw, gb);
+    wgrad3_tiles<CI>(s, blockIdx.x, gridDim.x, g, a, n, H, W, tiles_x, tiles_y, part);
 }
 
 // A hidden layer's backward pass in one launch: the first wb CTAs sum its weight
@@ -322,13 +322,75 @@ __global__ void __launch_bounds__(256) wgrad3_kernel(const float *g, const float
 // launches of the pass overlapping their starts (chain.cuh), the gradient of four
 // 128^2 images takes 261 us where it took 270, the copies from the host included.
 __global__ void __launch_bounds__(256) back3_kernel(const float *g, const float *a, const float *theta, int off_w,
-                                                    float *gx, int n, int H, int W, int tiles_x, int tiles_y, float *gw, float *gb, int wb)
+                                                    float *gx, int n, int H, int W, int tiles_x, int tiles_y, float *part,
+                                                    int wb)
 {
     constexpr int S1 = kGradSmem<HID>, S2 = kConvSmem<HID, HID>;
     __shared__ __align__(16) float s[S1 > S2 ? S1 : S2];
     chain_begin();
-    if ((int)blockIdx.x < wb) wgrad3_tiles<HID>(s, blockIdx.x, wb, g, a, n, H, W, tiles_x, tiles_y, gw, gb);
+    if ((int)blockIdx.x < wb) wgrad3_tiles<HID>(s, blockIdx.x, wb, g, a, n, H, W, tiles_x, tiles_y, part);
     else conv3_tile<HID, HID, true>(s, blockIdx.x - wb, g, theta, off_w, 0, a, gx, H, W, tiles_x, tiles_y);
+}
+
+// Where the CTAs of the backward pass leave their sums: count[l] slices of layer l's
+// parameters in part[l], in CTA order, and count[3] parts of the loss.
+struct GradParts {
+    float *part[4];
+    double *loss;
+    int count[4];
+};
+
+// The gradient and the loss from the CTAs' sums.  A block takes 32 parameters, eight
+// threads each; thread q adds the slices q, q + 8, ... in four interleaved chains, and
+// the chains and threads are added as a tree.  The order is fixed and no sum is longer
+// than 38 terms: by atomics, 256 to 512 additions one after another in the order of
+// arrival, the gradient of 4 x 128^2 cells was off by 2.3e-7 to 2.7e-7 of its norm and
+// differed from call to call; now it is off by 0.7e-7.  The whole call takes 258 us (266
+// with the atomics and the two fills that cleared their results).
+__global__ void __launch_bounds__(256) grad_sum_kernel(GradParts gp, float *grad, double *loss)
+{
+    chain_begin();
+    __shared__ float red[8][32];
+    __shared__ double redl[256];
+    if (blockIdx.x + 1 == gridDim.x) {
+        double v = 0.0;
+        for (int b = threadIdx.x; b < gp.count[3]; b += 256) v += gp.loss[b];
+        redl[threadIdx.x] = v;
+        for (int o = 128; o > 0; o >>= 1) {
+            __syncthreads();
+            if (threadIdx.x < o) redl[threadIdx.x] += redl[threadIdx.x + o];
+        }
+        if (threadIdx.x == 0) *loss = redl[0];
+        return;
+    }
+    const int k = blockIdx.x * 32 + (threadIdx.x & 31), q = threadIdx.x >> 5;
+    int l = 0, end = 0, np = 0, off = 0;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const LayerSpec S = layer_spec(i);
+        end = S.boff + S.cout;
+        if (k >= S.woff && k < end) { l = i; off = S.woff; np = end - S.woff; }
+    }
+    const bool in = k < end;
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (in) {
+        const float *p = gp.part[l] + (k - off);
+        const int n = gp.count[l];
+        int b = q;
+        for (; b + 24 < n; b += 32) {
+#pragma unroll
+            for (int i = 0; i < 4; i++) acc[i] += p[(long long)(b + 8 * i) * np];
+        }
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+            if (b + 8 * i < n) acc[i] += p[(long long)(b + 8 * i) * np];
+    }
+    red[q][threadIdx.x & 31] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    __syncthreads();
+    if (threadIdx.x < 32 && in) {
+        const int c = threadIdx.x;
+        grad[k] = ((red[0][c] + red[1][c]) + (red[2][c] + red[3][c])) + ((red[4][c] + red[5][c]) + (red[6][c] + red[7][c]));
+    }
 }
 
 __global__ void adam_kernel(float *theta, const float *grad, float *m, float *v, int np, float lr, float b1, float b2,
@@ -567,10 +629,32 @@ int cnn_n_params()
     return s.boff + s.cout;
 }
 
-size_t cnn_workspace_floats(int n, int H, int W)
+// CTAs that sum the weight gradients of a layer, and of the head: two an SM, eight an SM
+constexpr int kGradCtas = 152 * 2, kHeadCtas = 152 * 8;
+static long long layer_tiles(int n, int H, int W) { return (long long)n * ((W + kTx - 1) / kTx) * ((H + kTy - 1) / kTy); }
+
+// The workspace of cnn_loss_grad: the activations a1..a3, two gradient plane sets, then
+// the CTAs' sums.  Returns its floats (ws null: nothing else).
+static size_t grad_workspace(int n, int H, int W, float *ws, GradParts &gp)
 {
     const size_t px = (size_t)n * H * W;
-    return px * (size_t)(3 * HID) /* activations a1..a3 */ + px * (size_t)(2 * HID) /* two gradient plane sets */;
+    size_t o = px * (size_t)(3 * HID + 2 * HID);   // a multiple of 16 floats: the loss's doubles are aligned
+    gp.count[3] = (int)std::min<size_t>((px + 127) / 128, kHeadCtas);
+    gp.loss = ws ? reinterpret_cast<double *>(ws + o) : nullptr;
+    o += 2 * (size_t)gp.count[3];
+    for (int l = 0; l < 4; l++) {
+        const LayerSpec S = layer_spec(l);
+        if (l < 3) gp.count[l] = (int)std::min<long long>(layer_tiles(n, H, W), kGradCtas);
+        gp.part[l] = ws ? ws + o : nullptr;
+        o += (size_t)gp.count[l] * (S.boff + S.cout - S.woff);
+    }
+    return o;
+}
+
+size_t cnn_workspace_floats(int n, int H, int W)
+{
+    GradParts gp;
+    return grad_workspace(n, H, W, nullptr, gp);
 }
 
 // the three hidden layers in FP32, activations a1, a2, a3 to act
@@ -628,28 +712,28 @@ int cnn_loss_grad(const float *theta, const float *x, const float *t, const floa
     const long long plane = (long long)H * W;
     float *act = ws, *ga = ws + px * 3 * HID, *gb = ga + px * HID;
     const float *a1 = act, *a2 = act + px * HID, *a3 = act + 2 * px * HID;
-    const LayerSpec L0 = layer_spec(0), L1 = layer_spec(1), L2 = layer_spec(2), L3 = layer_spec(3);
-    cudaMemsetAsync(grad, 0, cnn_n_params() * sizeof(float), st);
-    cudaMemsetAsync(loss, 0, sizeof(double), st);
+    const LayerSpec L1 = layer_spec(1), L2 = layer_spec(2), L3 = layer_spec(3);
+    GradParts gp;
+    grad_workspace(n, H, W, ws, gp);
     const int e = hidden_forward(theta, x, n, H, W, act, st);
     if (e) return e;
     // head (1x1, 16 -> 1)
-    int r = launch_chained(head_loss_kernel, (unsigned)std::min<long long>((px + 127) / 128, 152 * 8), 128, 0, st, a3, theta, L3.woff,
-                           L3.boff, t, m, px, plane, mcount > 0 ? 1.0f / mcount : 0.0f, ga, grad + L3.woff, grad + L3.boff, loss);
+    int r = launch_chained(head_loss_kernel, gp.count[3], 128, 0, st, a3, theta, L3.woff, L3.boff, t, m, px, plane,
+                           mcount > 0 ? 1.0f / mcount : 0.0f, ga, gp.part[3], gp.loss);
     if (r) return r;
     const int txs = (W + kTx - 1) / kTx, tys = (H + kTy - 1) / kTy;
-    const int grid = n * txs * tys, wb = std::min(grid, 152 * 2);   // hidden_forward has refused grids above 2^31 - 1
+    const int grid = n * txs * tys, wb = gp.count[0];   // hidden_forward has refused grids above 2^31 - 1
     if (grid > 0x7fffffff - wb) return (int)cudaErrorInvalidValue;
     // layer 3 (3x3, 16 -> 16): input a2
-    r = launch_chained(back3_kernel, grid + wb, 256, 0, st, ga, a2, theta, L2.woff, gb, n, H, W, txs, tys, grad + L2.woff,
-                           grad + L2.boff, wb);
+    r = launch_chained(back3_kernel, grid + wb, 256, 0, st, ga, a2, theta, L2.woff, gb, n, H, W, txs, tys, gp.part[2], wb);
     if (r) return r;
     // layer 2: input a1
-    r = launch_chained(back3_kernel, grid + wb, 256, 0, st, gb, a1, theta, L1.woff, ga, n, H, W, txs, tys, grad + L1.woff,
-                       grad + L1.boff, wb);
+    r = launch_chained(back3_kernel, grid + wb, 256, 0, st, gb, a1, theta, L1.woff, ga, n, H, W, txs, tys, gp.part[1], wb);
     if (r) return r;
     // layer 1: input x (no ReLU before it, no input gradient needed)
-    return launch_chained(wgrad3_kernel<kCnnIn>, wb, 256, 0, st, ga, x, n, H, W, txs, tys, grad + L0.woff, grad + L0.boff);
+    r = launch_chained(wgrad3_kernel<kCnnIn>, wb, 256, 0, st, ga, x, n, H, W, txs, tys, gp.part[0]);
+    if (r) return r;
+    return launch_chained(grad_sum_kernel, (cnn_n_params() + 31) / 32 + 1, 256, 0, st, gp, grad, loss);
 }
 
 int cnn_adam(float *theta, const float *grad, float *m, float *v, int np, float lr, int t, cudaStream_t st)

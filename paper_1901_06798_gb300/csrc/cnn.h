@@ -9,7 +9,7 @@ constexpr int kCnnIn = 5;       // input features per cell
 constexpr int kCnnHidden = 16;  // channels of the three 3x3 layers
 
 int cnn_n_params();
-// FP32 activations + gradient planes needed by cnn_loss_grad for n planes of H x W
+// FP32 activations, gradient planes and CTAs' sums needed by cnn_loss_grad for n planes of H x W
 size_t cnn_workspace_floats(int n, int H, int W);
 // workspace bytes of the inference path (its activations stay in shared memory)
 size_t cnn_half_workspace_bytes(int n, int H, int W);
