@@ -8,7 +8,7 @@
 // behind its back, and latency-critical loops cannot afford a cudaMalloc that
 // may block or fail.  The context-based entry points allocate (the patch
 // arena, tables, flags); this one keeps its few bytes of scratch -- patch
-// descriptor, boundary list, dt and the wave-speed accumulator --
+// descriptor, dt, the CTA count and the wave-speed accumulator --
 // in one file-scope __device__ array instead.
 //
 // The scratch array is shared by every call in the process on a given GPU
@@ -22,6 +22,7 @@
 
 #include "../../include/tsunami.h"
 #include "amr_kernels.h"
+#include "tile_rules.h"
 #include "tsu_device.h"
 
 namespace tsu {
@@ -105,7 +106,7 @@ extern "C" int tsu_grid_step_noalloc(int precision, void *block, int nx, int ny,
     // tiles found from the CTA's index
     const int nt = precision == TSU_F64 ? step_threads_f64(0) : step_threads_f32p();
     const int W = precision == TSU_F64 ? step_strip_width_f64(nt, 0) : step_strip_width_f32p(nt, 0);
-    const int rows = tile_cut(ny, precision == TSU_F64 ? tile_rows_f64(1, &nx, &ny) : tile_rows_f32p(1, &nx, &ny, nt));
+    const int rows = tile_cut(ny, work_rows(1, &nx, &ny, W, nt, true, precision == TSU_F64));
     const int nsx = (nx + W - 1) / W, nsy = (ny + rows - 1) / rows;
 
     cudaStream_t st = (cudaStream_t)cuda_stream;

@@ -48,6 +48,7 @@
 #pragma once
 #include <type_traits>
 #include "step_f32x2.cuh"
+#include "tile_rules.h"
 
 namespace tsu {
 

@@ -33,6 +33,7 @@
 // (ced_{j+1} - ced_j) hv_j of the varying edge length.
 #pragma once
 #include "step_kernel.cuh"
+#include "tile_rules.h"
 
 namespace tsu {
 namespace d1 {

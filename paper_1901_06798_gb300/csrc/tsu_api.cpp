@@ -28,6 +28,7 @@
 #include "amr_kernels.h"
 #include "cnn.h"
 #include "host_pool.h"
+#include "tile_rules.h"
 #include "tsu_device.h"
 
 namespace tsu {
@@ -634,9 +635,7 @@ struct tsu_ctx {
             } else {
                 std::vector<int> px(n), py(n);
                 for (int k = 0; k < n; k++) { px[k] = L.P[k].nx; py[k] = L.P[k].ny; }
-                L.tile_rows = !split ? unsplit_rows(n, px.data(), py.data(), nt(), prec)
-                                     : (prec == TSU_F64 ? tile_rows_f64(n, px.data(), py.data())
-                                                        : tile_rows_f32p(n, px.data(), py.data(), nt()));
+                L.tile_rows = work_rows(n, px.data(), py.data(), W, nt(), split, prec == TSU_F64);
                 if (seg_rows > 0) L.tile_rows = std::min(L.tile_rows, seg_rows);
             }
             std::vector<std::vector<StepItem>> xi(16);

@@ -1,7 +1,6 @@
 // tsu_device.h -- structures shared by the library's host code and kernels.
 #pragma once
 #include <cstdint>
-#include <vector>
 #include <cuda_runtime.h>
 
 namespace tsu {
@@ -159,34 +158,5 @@ int step_threads_f32p();
 // per CTA (the unsplit kernels take one column per thread in both precisions)
 int step_strip_width_f64(int threads, int transverse);
 int step_strip_width_f32p(int threads, int transverse);
-// Split update: rows of a tile for n patches of nx[k] x ny[k] cells advanced
-// together (FP32: by CTAs of `threads`), and rows of a patch's tiles (of at most
-// `cap` rows): equal and even
-int tile_rows_f32p(int n, const int *nx, const int *ny, int threads);
-int tile_rows_f64(int n, const int *nx, const int *ny);
-// tiles of at most R rows over patches sorted by height: strips[ny] strips of ny rows
-inline double tile_count(const std::vector<double> &strips, int R)
-{
-    double items = 0.0;
-    for (size_t ny = 1; ny < strips.size(); ny++)
-        if (strips[ny] > 0.0) items += strips[ny] * (double)((ny + R - 1) / R);
-    return items;
-}
-inline std::vector<double> strips_by_height(int n, const int *nx, const int *ny, int W)
-{
-    int top = 0;
-    for (int k = 0; k < n; k++) top = ny[k] > top ? ny[k] : top;
-    std::vector<double> s((size_t)top + 1, 0.0);
-    for (int k = 0; k < n; k++) s[ny[k]] += (double)((nx[k] + W - 1) / W);
-    return s;
-}
-inline int tile_cut(int ny, int cap)
-{
-    const int nt = (ny + cap - 1) / cap, r = (ny + nt - 1) / nt;
-    return r + (r & 1) <= cap ? r + (r & 1) : r;
-}
-constexpr int kTileRowsMax = 124, kTileRowsMaxF64 = 104;   // a tile row takes 1 KiB (FP64: 2 KiB) of shared memory
-// unsplit update: rows of its row segments, by the same reasoning
-int unsplit_rows(int n, const int *nx, const int *ny, int threads, int precision);
 
 }  // namespace tsu

@@ -1,0 +1,115 @@
+"""Heights of the patch update's work items (csrc/tile_rules.h), compiled for the host:
+what one patch gets is what the rule over many patches gives it, the rules are those
+of a restatement that looks at the patches one by one, and a step of a grid in the
+caller's memory, which asks on every call, allocates nothing for it.
+"""
+import ctypes
+import math
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1901_06798_gb300", "csrc")
+
+HARNESS = r"""
+#include <cstdlib>
+#include <new>
+#include "tile_rules.h"
+static long allocations = 0;
+void *operator new(std::size_t n) { allocations++; void *p = std::malloc(n ? n : 1); if (!p) throw std::bad_alloc(); return p; }
+void operator delete(void *p) noexcept { std::free(p); }
+void operator delete(void *p, std::size_t) noexcept { std::free(p); }
+extern "C" long rows(int n, const int *nx, const int *ny, int W, int threads, int split, int f64, long *allocs)
+{
+    const long a = allocations;
+    const int r = tsu::work_rows(n, nx, ny, W, threads, split != 0, f64 != 0);
+    *allocs = allocations - a;
+    return r;
+}
+extern "C" long cut(int ny, int cap) { return tsu::tile_cut(ny, cap); }
+"""
+
+# (threads, split, f64) of the library's launches, with their strips' columns
+KINDS = [(128, 1, 0), (32, 1, 0), (256, 1, 0), (128, 1, 1), (64, 1, 1), (128, 0, 0), (64, 0, 1)]
+
+
+def _width(threads, split):
+    return 60 if split else threads - 4
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rules")
+    (d / "h.cpp").write_text(HARNESS)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(d / "h.cpp"), "-o", str(d / "h.so")],
+                   check=True)
+    L = ctypes.CDLL(str(d / "h.so"))
+    L.rows.restype = L.cut.restype = ctypes.c_long
+    return L
+
+
+def _rows(lib, patches, threads, split, f64):
+    nx, ny = (np.array(v, dtype=np.intc) for v in zip(*patches))
+    p = [v.ctypes.data_as(ctypes.POINTER(ctypes.c_int)) for v in (nx, ny)]
+    allocs = ctypes.c_long()
+    r = lib.rows(len(patches), *p, _width(threads, split), threads, split, f64, ctypes.byref(allocs))
+    return r, allocs.value
+
+
+def _restated(patches, threads, split, f64):
+    W = _width(threads, split)
+
+    def cost(R):
+        per = sum(-(-x // W) * -(-y // R) for x, y in patches) / 152
+        if split and f64:
+            return math.ceil(per) * (2.0 * (R + 4) + 4.0 * (R // 2 + 3)) * (1.75 if per <= 1 else 1.2 if per <= 2 else 1.0)
+        one, share = (R + 16.0, 0.15) if split else (R + 6.0, 0.4)
+        if f64:
+            return math.ceil(per) * one
+        occ = 512 // threads
+        if split:
+            occ = max(1, min(occ, 228 * 1024 // ((R + 4) * 1024 + 1024)))
+        full = math.floor(per / occ)
+        rest = math.ceil(per - full * occ - 1e-9)
+        return full * one * (1.0 + share * (occ - 1)) + (one * (1.0 + share * (rest - 1)) if rest > 0 else 0.0)
+
+    if split:
+        cand = range(32, 3, -2) if f64 else (4, 6, 8, 10, 12, 16, 20, 24, 30, 36, 44, 60)
+    else:
+        cand = (8, 12, 16, 24, 32, 48, 64)
+    return min(cand, key=cost)
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("nx,ny", [(1, 1), (2, 3), (48, 40), (60, 61), (771, 602), (4096, 4096), (64, 16384), (16384, 16384)])
+def test_one_patch(lib, nx, ny, kind):
+    r, allocs = _rows(lib, [(nx, ny)], *kind)
+    assert r == _restated([(nx, ny)], *kind)
+    assert allocs == 0
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("n", [2, 30, 4000])
+def test_many_patches(lib, n, kind):
+    rng = np.random.default_rng(n)
+    patches = [(int(a), int(b)) for a, b in rng.integers(1, 65, (n, 2))]
+    r, allocs = _rows(lib, patches, *kind)
+    assert r == _restated(patches, *kind)
+    assert allocs > 0   # (the counter counts)
+
+
+def test_a_patch_cut_into_strips_is_one_patch(lib):
+    for kind in KINDS:
+        W = _width(kind[0], kind[1])
+        for ny in (5, 129, 1537):
+            assert _rows(lib, [(7 * W, ny)], *kind)[0] == _rows(lib, [(W, ny)] * 7, *kind)[0]
+
+
+def test_tiles_are_equal_even_and_within_the_cap(lib):
+    for ny in range(1, 400):
+        for cap in (1, 2, 3, 12, 44, 59, 60, 124):
+            r = lib.cut(ny, cap)
+            assert 1 <= r <= cap and -(-ny // r) <= -(-ny // cap)
+            assert r % 2 == 0 or r == -(-ny // -(-ny // cap))
