@@ -262,9 +262,8 @@ int tsu_get_stats(tsu_ctx *ctx, int scenario, tsu_stats *out);
  * threads per CTA and seg_rows rows per CTA (patches taller than that are cut
  * into row segments).  step_threads is 64, 128 or 256, or also 32 for the
  * split FP32 update.  A CTA updates a tile of 60 columns in the split updates
- * and a strip of step_threads - 4 columns in the unsplit ones.  In the split
- * FP32 update seg_rows (up to 124) sets the tiles' height, in the other updates
- * it bounds the height that the size of the level suggests.  0 restores the
+ * (of at most 124 rows in FP32 and 104 in FP64: what shared memory holds) and a
+ * strip of step_threads - 4 columns in the unsplit ones.  0 restores the
  * defaults.  Results do not depend on either.  Returns TSU_ERR_ARG for any
  * other value. */
 int tsu_set_tuning(tsu_ctx *ctx, int step_threads, int seg_rows);

@@ -151,4 +151,12 @@ inline int work_rows(int n, const int *nx, const int *ny, int W, int threads, bo
     return work_rows(s.data(), (int)s.size(), threads, split, f64);
 }
 
+// The most rows of a work item: what the caller asks for (seg_rows > 0; tiles no taller
+// than shared memory holds), else the rule's
+inline int item_rows(int seg_rows, int n, const int *nx, const int *ny, int W, int threads, bool split, bool f64)
+{
+    if (seg_rows <= 0) return work_rows(n, nx, ny, W, threads, split, f64);
+    return split ? std::min(seg_rows, f64 ? kTileRowsMaxF64 : kTileRowsMax) : seg_rows;
+}
+
 }  // namespace tsu

@@ -628,16 +628,9 @@ struct tsu_ctx {
         // host threads and joined in range order
         {
             // split update: tiles of equal heights within a patch; unsplit: row segments
-            // (seg_rows caps them; it sets them in the FP32 split update, whose issue-bound
-            // tiles can be worth other heights than the rule's)
-            if (seg_rows > 0 && split_f32()) {
-                L.tile_rows = std::min(seg_rows, kTileRowsMax);
-            } else {
-                std::vector<int> px(n), py(n);
-                for (int k = 0; k < n; k++) { px[k] = L.P[k].nx; py[k] = L.P[k].ny; }
-                L.tile_rows = work_rows(n, px.data(), py.data(), W, nt(), split, prec == TSU_F64);
-                if (seg_rows > 0) L.tile_rows = std::min(L.tile_rows, seg_rows);
-            }
+            std::vector<int> px(n), py(n);
+            for (int k = 0; k < n; k++) { px[k] = L.P[k].nx; py[k] = L.P[k].ny; }
+            L.tile_rows = item_rows(seg_rows, n, px.data(), py.data(), W, nt(), split, prec == TSU_F64);
             std::vector<std::vector<StepItem>> xi(16);
             parallel_ranges(n, [&](int q, int b, int e) {
                 std::vector<StepItem> &ox = xi[q];

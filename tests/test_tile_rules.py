@@ -28,6 +28,10 @@ extern "C" long rows(int n, const int *nx, const int *ny, int W, int threads, in
     *allocs = allocations - a;
     return r;
 }
+extern "C" long item(int seg_rows, int nx, int ny, int W, int threads, int split, int f64)
+{
+    return tsu::item_rows(seg_rows, 1, &nx, &ny, W, threads, split != 0, f64 != 0);
+}
 extern "C" long cut(int ny, int cap) { return tsu::tile_cut(ny, cap); }
 """
 
@@ -46,7 +50,7 @@ def lib(tmp_path_factory):
     subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(d / "h.cpp"), "-o", str(d / "h.so")],
                    check=True)
     L = ctypes.CDLL(str(d / "h.so"))
-    L.rows.restype = L.cut.restype = ctypes.c_long
+    L.rows.restype = L.cut.restype = L.item.restype = ctypes.c_long
     return L
 
 
@@ -113,3 +117,40 @@ def test_tiles_are_equal_even_and_within_the_cap(lib):
             r = lib.cut(ny, cap)
             assert 1 <= r <= cap and -(-ny // r) <= -(-ny // cap)
             assert r % 2 == 0 or r == -(-ny // -(-ny // cap))
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_the_caller_sets_the_height(lib, kind):
+    """Also above what the rule would take, up to what a tile can hold."""
+    threads, split, f64 = kind
+    most = (104 if f64 else 124) if split else 1 << 31
+    for nx, ny in ((48, 40), (771, 602), (4096, 4096)):
+        for rows in (1, 2, 9, 33, 48, 64, 104, 124, 256, (1 << 31) - 1):
+            assert lib.item(rows, nx, ny, _width(threads, split), threads, split, f64) == min(rows, most)
+        assert lib.item(0, nx, ny, _width(threads, split), threads, split, f64) == _rows(lib, [(nx, ny)], *kind)[0]
+
+
+def _run(nx, ny, prec, transverse, tuning):
+    from paper_1901_06798_gb300 import binding, workloads as W
+    w = W.hump200()
+    cfg = dict(w["cfg"], nx=nx, ny=ny, dx=2000.0 / nx, dy=2000.0 / ny, bc=[0, 1, 1, 0], transverse=transverse)
+    w = dict(w, cfg=cfg)
+    g = W.load(binding.Tsunami(cfg, precision=prec), w)
+    if tuning:
+        g.set_tuning(*tuning)
+    g.step(8)
+    out = [g.level_array(0, 1, f) for f in ("eta", "hu", "hv")]
+    g.close()
+    return out
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec,transverse", [(0, 0), (0, 1), (1, 1)])
+@pytest.mark.parametrize("nx,ny", [(61, 105), (130, 333)])
+def test_tall_work_items_same_bits(nx, ny, prec, transverse):
+    """Heights that the rules do not take: one row, FP64 tiles of all the shared memory of
+    an SM, row segments of the whole grid."""
+    ref = _run(nx, ny, prec, transverse, None)
+    for tuning in ((64, 1), (128, 48), (128, 104), (256, 105), (64, 1 << 20)):
+        for a, b in zip(_run(nx, ny, prec, transverse, tuning), ref):
+            assert np.array_equal(a, b), tuning
