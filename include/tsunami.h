@@ -281,12 +281,15 @@ int tsu_set_tuning(tsu_ctx *ctx, int step_threads, int seg_rows);
  * or polls outside [0, 2^32 - 1]. */
 int tsu_set_bulk_copies(tsu_ctx *ctx, int enable, long long polls);
 
-/* Autotuner: time every launch shape of the patch update (threads per CTA
- * 64/128/256, and 32 for the split FP32 update, x rows per work item
- * 32/64/128/256, or 16/32/64/128 for the split FP32 update) on the context's current
- * levels with `reps` zero-length steps each -- the kernels do all their work
- * but the state is unchanged -- and keep the fastest.  Outputs (any may be
- * NULL): the chosen shape and its time per step of all levels in ms. */
+/* Autotuner: time launch shapes of the patch update (threads per CTA 64/128/256,
+ * and 32 for the split FP32 update, x rows per work item: the library's own
+ * choice for each level's size, 32, 64, and 16/124 in the split FP32 update or
+ * 128 in the unsplit ones) on the context's current levels with `reps`
+ * zero-length steps each -- the kernels do all their work but the state is
+ * unchanged -- and keep the fastest.  Outputs (any may be NULL): the chosen
+ * shape and its time per step of all levels in ms.  Where the library's own
+ * heights were the fastest, the rows are a bound on them (32, 64 or 128): set
+ * them elsewhere by seg_rows = 0. */
 int tsu_autotune(tsu_ctx *ctx, int reps, int *best_threads, int *best_seg_rows, double *best_ms);
 
 /* Checkpoint and restart of a whole simulation, between tsu_step calls

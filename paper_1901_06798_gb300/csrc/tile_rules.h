@@ -151,6 +151,31 @@ inline int work_rows(int n, const int *nx, const int *ny, int W, int threads, bo
     return work_rows(s.data(), (int)s.size(), threads, split, f64);
 }
 
+// The launch shapes the autotuner times (threads, seg_rows): the library's own heights
+// (0) and set ones.  None is another one under a second name: every set height is within
+// what a tile can hold.
+struct LaunchShape {
+    int threads, seg_rows;
+};
+inline std::vector<LaunchShape> launch_shapes(bool split, bool f64)
+{
+    std::vector<LaunchShape> out;
+    const bool tile32 = split && !f64;
+    for (int t : {64, 128, 256, 32}) {
+        if (t == 32 && !tile32) continue;
+        for (int r : {0, 16, 32, 64, 128})
+            if ((r != 16 || tile32) && !(split && r == 128)) out.push_back({t, r});
+        if (tile32) out.push_back({t, kTileRowsMax});
+    }
+    return out;
+}
+// The rows the autotuner reports: those set, else a bound on the library's own, the most
+// rows of a work item on any level: 32, 64 or 128 (they never exceed 64)
+inline int reported_rows(int seg_rows, int most)
+{
+    return seg_rows > 0 ? seg_rows : (most <= 32 ? 32 : (most <= 64 ? 64 : 128));
+}
+
 // The most rows of a work item: what the caller asks for (seg_rows > 0; tiles no taller
 // than shared memory holds), else the rule's
 inline int item_rows(int seg_rows, int n, const int *nx, const int *ny, int W, int threads, bool split, bool f64)

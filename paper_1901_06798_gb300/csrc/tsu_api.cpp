@@ -2327,22 +2327,15 @@ int tsu_autotune(tsu_ctx *ctx, int reps, int *best_threads, int *best_seg_rows, 
         ctx->zero_dtf.ensure(ctx->nscen, ctx->st);
         CK(cudaMemsetAsync(ctx->zero_dt.p, 0, ctx->nscen * sizeof(double), ctx->st));
         CK(cudaMemsetAsync(ctx->zero_dtf.p, 0, ctx->nscen * sizeof(float), ctx->st));
-        // threads x rows per work item; the FP32 split update's items are tiles held
-        // in shared memory: shorter ones, and also by 32 threads
-        const bool split = ctx->split_f32();
-        const int nts[4] = {64, 128, 256, 32};
-        const int segs[4] = {split ? 16 : 32, split ? 32 : 64, split ? 64 : 128, split ? 128 : 256};
-        const int n_nt = split ? 4 : 3;
+        const std::vector<LaunchShape> shapes = launch_shapes(ctx->c.transverse == 0, ctx->prec == TSU_F64);
         cudaEvent_t e0, e1;
         CK(cudaEventCreate(&e0));
         CK(cudaEventCreate(&e1));
         double best = 1e30;
         int bt = 0, bs = 0;
-        // (the FP32 split update's own choice, 0 x 0, comes last)
-        const int n_shapes = 4 * n_nt + (split ? 1 : 0);
-        for (int q = 0; q < n_shapes; q++) {
-            ctx->step_nt = q < 4 * n_nt ? nts[q / 4] : 0;
-            ctx->seg_rows = q < 4 * n_nt ? segs[q % 4] : 0;
+        for (const LaunchShape &q : shapes) {
+            ctx->step_nt = q.threads;
+            ctx->seg_rows = q.seg_rows;
             for (int l = 0; l < ctx->nlev; l++)
                 if (!ctx->lv[l].P.empty()) ctx->finish_level(l);
             auto run = [&] {
@@ -2373,7 +2366,10 @@ int tsu_autotune(tsu_ctx *ctx, int reps, int *best_threads, int *best_seg_rows, 
             if (!ctx->lv[l].P.empty()) ctx->finish_level(l);
         ctx->sync();
         if (best_threads) *best_threads = ctx->nt();
-        if (best_seg_rows) *best_seg_rows = bs > 0 ? bs : ctx->lv[0].tile_rows;
+        int most = 0;
+        for (int l = 0; l < ctx->nlev; l++)
+            if (!ctx->lv[l].P.empty()) most = std::max(most, ctx->lv[l].tile_rows);
+        if (best_seg_rows) *best_seg_rows = reported_rows(bs, most);
         if (best_ms) *best_ms = best;
     });
 }

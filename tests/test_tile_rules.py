@@ -32,6 +32,13 @@ extern "C" long item(int seg_rows, int nx, int ny, int W, int threads, int split
 {
     return tsu::item_rows(seg_rows, 1, &nx, &ny, W, threads, split != 0, f64 != 0);
 }
+extern "C" long shapes(int split, int f64, int *out)   // (threads, rows) pairs
+{
+    long n = 0;
+    for (const tsu::LaunchShape &s : tsu::launch_shapes(split != 0, f64 != 0)) { out[2 * n] = s.threads; out[2 * n + 1] = s.seg_rows; n++; }
+    return n;
+}
+extern "C" long reported(int seg_rows, int most) { return tsu::reported_rows(seg_rows, most); }
 extern "C" long cut(int ny, int cap) { return tsu::tile_cut(ny, cap); }
 """
 
@@ -50,7 +57,7 @@ def lib(tmp_path_factory):
     subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(d / "h.cpp"), "-o", str(d / "h.so")],
                    check=True)
     L = ctypes.CDLL(str(d / "h.so"))
-    L.rows.restype = L.cut.restype = L.item.restype = ctypes.c_long
+    L.rows.restype = L.cut.restype = L.item.restype = L.shapes.restype = L.reported.restype = ctypes.c_long
     return L
 
 
@@ -128,6 +135,21 @@ def test_the_caller_sets_the_height(lib, kind):
         for rows in (1, 2, 9, 33, 48, 64, 104, 124, 256, (1 << 31) - 1):
             assert lib.item(rows, nx, ny, _width(threads, split), threads, split, f64) == min(rows, most)
         assert lib.item(0, nx, ny, _width(threads, split), threads, split, f64) == _rows(lib, [(nx, ny)], *kind)[0]
+
+
+@pytest.mark.parametrize("split,f64", [(1, 0), (1, 1), (0, 0), (0, 1)])
+def test_the_autotuner_times_shapes_that_differ_and_reports_their_rows(lib, split, f64):
+    out = (ctypes.c_int * 64)()
+    n = lib.shapes(split, f64, out)
+    shapes = [(out[2 * k], out[2 * k + 1]) for k in range(n)]
+    threads = {64, 128, 256} | ({32} if split and not f64 else set())
+    assert {t for t, _ in shapes} == threads and {(t, 0) for t in threads} <= set(shapes)
+    launched = [(t, lib.item(r, 4096, 4096, _width(t, split), t, split, f64) if r else 0) for t, r in shapes]
+    assert len(set(launched)) == len(shapes)
+    for (t, r), (_, rows) in zip(shapes, launched):
+        assert rows == r and (r == 0 or lib.reported(r, 7) == r)
+    for most in range(1, 125):
+        assert lib.reported(0, most) == min(r for r in (32, 64, 128) if r >= most)
 
 
 def _run(nx, ny, prec, transverse, tuning):
