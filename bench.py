@@ -21,6 +21,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -84,10 +85,21 @@ def peaks():
     return 6800.0, "fallback"
 
 
+def kernel_sources():
+    """The sources of the split update: its two translation units and what they include."""
+    d = os.path.join(ROOT, "paper_1901_06798_gb300", "csrc")
+    out, todo = [], ["step_f64.cu", "step_f32p.cu"]
+    while todo:
+        f = todo.pop()
+        if f not in out:
+            out.append(f)
+            todo += re.findall(r'^#include "([\w.]+)"', open(os.path.join(d, f)).read(), re.M)
+    return sorted(out)
+
+
 def kernel_hash():
     h = hashlib.sha256()
-    for f in ("step_kernel.cuh", "step_f32x2.cuh", "step_tile_f32.cuh", "step_tile_f64.cuh", "step_f32p.cu", "step_f64.cu",
-              "tsu_device.h"):
+    for f in kernel_sources():
         h.update(open(os.path.join(ROOT, "paper_1901_06798_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
