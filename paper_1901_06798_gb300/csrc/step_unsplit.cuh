@@ -444,6 +444,14 @@ int launch_unsplit_nt(const StepArgs &a, int n_items, cudaStream_t st)
         if (e != cudaSuccess) return (int)e;
         configured = true;
     }
+    // Not launched ahead of its predecessor's end: placed around CTAs that are still
+    // there, several segments share an SM's FP64 pipe while others idle.  Behind the
+    // interpolation of a 3-level run's ghost cells (150 patches, a segment each) a coarse
+    // step took 104 ms launched ahead and takes 68 ms; uniform grids take the same.
+    if (a.gate == nullptr) {
+        step_unsplit_kernel<T, PERT, NT, RING><<<n_items, NT, bytes, st>>>(a);
+        return (int)cudaGetLastError();
+    }
     return launch_chained(step_unsplit_kernel<T, PERT, NT, RING>, n_items, NT, bytes, st, a);
 }
 

@@ -64,3 +64,14 @@ def test_chained_kernels_wait_first_and_promise_no_constant_data(kernel):
     assert re.search(r"chain_begin\(\)|launch_live\(", FUNCTIONS[kernel][1])
     for f in sorted(_reached(kernel, set())):
         assert "__restrict__" not in FUNCTIONS[f][0] + FUNCTIONS[f][1], f
+
+
+@pytest.mark.parametrize("source,kernel", [("step_f64.cu", "step_tile_f64"), ("step_unsplit.cuh", "step_unsplit_kernel")])
+def test_fp64_updates_are_launched_after_their_predecessor(source, kernel):
+    """Launched ahead of its end they share SMs unevenly, and each SM's FP64 pipe is what
+    bounds them (a 3-level unsplit run took 1.5 times as long).  Only the retake launch,
+    which mostly finds nothing to do, overlaps."""
+    text = open(os.path.join(CSRC, source)).read()
+    plain = text.index("if (a.gate == nullptr) {")
+    assert re.match(r"if \(a\.gate == nullptr\) \{\s+" + kernel + r"<[^;]*<<<", text[plain:])
+    assert text.index("launch_chained(" + kernel) > plain
