@@ -112,24 +112,46 @@ inline int tile_rows_f64(const HeightStrips *s, int m)
     return best;
 }
 
-// Unsplit update: rows of its row segments (strips of threads - 4 columns), each
-// of which sweeps 4 more and fills its pipeline.  FP32: about 16 warps run on an
-// SM, which share its issue slots as the tiles' do.  FP64: an SM's CTAs share its
-// FP64 pipe, so their times add up.
-// Both sides (us): FP32 1024^2 took 172 with rows by a fixed 64, 70 with the rule's, 86 with 12;
-// FP32 300^2 37 with the rule's and 45 with 64 threads; 2500^2 289 (rule), 286 to 298 at others.
-inline int unsplit_rows(const HeightStrips *s, int m, int threads, bool f64)
+// Unsplit update, FP32: rows of its row segments (strips of threads - 4 columns), each
+// of which sweeps 4 more and fills its pipeline.  About 16 warps run on an SM, which
+// share its issue slots as the tiles' do.
+// Both sides (us): 1024^2 took 172 with rows by a fixed 64, 70 with the rule's, 86 with 12;
+// 300^2 37 with the rule's and 45 with 64 threads; 2500^2 289 (rule), 286 to 298 at others.
+inline int unsplit_rows_f32p(const HeightStrips *s, int m, int threads)
 {
     static const int cand[] = {8, 12, 16, 24, 32, 48, 64};
     const int occ = std::max(1, 512 / threads);
-    int best = f64 ? 128 : 64;
+    int best = 64;
     double bc = 1e300;
     for (int R : cand) {
         const double items = tile_count(s, m, R);
         const double per = items / kSMs, full = std::floor(per / occ), rest = std::ceil(per - full * occ - 1e-9);
         const double one = R + 6;
-        const double c = f64 ? std::ceil(per) * one
-                             : full * one * (1.0 + 0.4 * (occ - 1)) + (rest > 0 ? one * (1.0 + 0.4 * (rest - 1)) : 0.0);
+        const double c = full * one * (1.0 + 0.4 * (occ - 1)) + (rest > 0 ? one * (1.0 + 0.4 * (rest - 1)) : 0.0);
+        if (c < bc) { bc = c; best = R; }
+    }
+    return best;
+}
+
+// Unsplit update, FP64: the same segments.  Eight warps fit on an SM (shared memory); in
+// units of two warps, a row of one, two or three alone takes 2.1, 2.25 and 3.1 times what
+// it takes of the full four, where the FP64 pipe is busy.  Beyond that the SMs take
+// segments as they finish: the work shared out, and the end of the last ones (1.3).
+// Both sides (us a step, developed sea, heights 16 / 32 / 64 / 128, then the rule's):
+// 771 x 602 1447 / 1569 / 2852 / 5575 (16), 1024^2 2800 / 2727 / 3037 / 5588 (32), 2000^2
+// 9699 / 10358 / 10295 / 10398 (128), 2400^2 13689 / 13076 / 15179 / 18085 (32), 4096 x
+// 1000 9978 / 10403 / 10149 / 10388 (128).  Counting whole segments an SM, whatever the
+// number in flight, took 48 rows for the last two: 13674 and 11401.
+inline int unsplit_rows_f64(const HeightStrips *s, int m, int threads)
+{
+    static const int cand[] = {8, 12, 16, 24, 32, 48, 64, 96, 128};
+    static const double alone[] = {0.0, 2.1, 2.25, 3.1, 4.0};
+    const double unit = threads / 64.0;
+    int best = 64;
+    double bc = 1e300;
+    for (int R : cand) {
+        const double per = tile_count(s, m, R) / kSMs * unit, in_flight = std::ceil(per / unit - 1e-9) * unit;
+        const double c = (R + 2) * (in_flight <= 4.0 ? alone[(int)in_flight] : per + 1.3);
         if (c < bc) { bc = c; best = R; }
     }
     return best;
@@ -139,7 +161,8 @@ inline int unsplit_rows(const HeightStrips *s, int m, int threads, bool f64)
 // in strips of W columns by CTAs of `threads`
 inline int work_rows(const HeightStrips *s, int m, int threads, bool split, bool f64)
 {
-    return !split ? unsplit_rows(s, m, threads, f64) : (f64 ? tile_rows_f64(s, m) : tile_rows_f32p(s, m, threads));
+    if (split) return f64 ? tile_rows_f64(s, m) : tile_rows_f32p(s, m, threads);
+    return f64 ? unsplit_rows_f64(s, m, threads) : unsplit_rows_f32p(s, m, threads);
 }
 inline int work_rows(int n, const int *nx, const int *ny, int W, int threads, bool split, bool f64)
 {
@@ -170,7 +193,7 @@ inline std::vector<LaunchShape> launch_shapes(bool split, bool f64)
     return out;
 }
 // The rows the autotuner reports: those set, else a bound on the library's own, the most
-// rows of a work item on any level: 32, 64 or 128 (they never exceed 64)
+// rows of a work item on any level: 32, 64 or 128 (which they never exceed)
 inline int reported_rows(int seg_rows, int most)
 {
     return seg_rows > 0 ? seg_rows : (most <= 32 ? 32 : (most <= 64 ? 64 : 128));

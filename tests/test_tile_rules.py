@@ -76,9 +76,10 @@ def _restated(patches, threads, split, f64):
         per = sum(-(-x // W) * -(-y // R) for x, y in patches) / 152
         if split and f64:
             return math.ceil(per) * (2.0 * (R + 4) + 4.0 * (R // 2 + 3)) * (1.75 if per <= 1 else 1.2 if per <= 2 else 1.0)
-        one, share = (R + 16.0, 0.15) if split else (R + 6.0, 0.4)
         if f64:
-            return math.ceil(per) * one
+            n = math.ceil(per - 1e-9) * threads / 64
+            return (R + 2) * ((0.0, 2.1, 2.25, 3.1, 4.0)[int(n)] if n <= 4 else per * threads / 64 + 1.3)
+        one, share = (R + 16.0, 0.15) if split else (R + 6.0, 0.4)
         occ = 512 // threads
         if split:
             occ = max(1, min(occ, 228 * 1024 // ((R + 4) * 1024 + 1024)))
@@ -89,7 +90,7 @@ def _restated(patches, threads, split, f64):
     if split:
         cand = range(32, 3, -2) if f64 else (4, 6, 8, 10, 12, 16, 20, 24, 30, 36, 44, 60)
     else:
-        cand = (8, 12, 16, 24, 32, 48, 64)
+        cand = (8, 12, 16, 24, 32, 48, 64, 96, 128) if f64 else (8, 12, 16, 24, 32, 48, 64)
     return min(cand, key=cost)
 
 
@@ -109,6 +110,35 @@ def test_many_patches(lib, n, kind):
     r, allocs = _rows(lib, patches, *kind)
     assert r == _restated(patches, *kind)
     assert allocs > 0   # (the counter counts)
+
+
+# us of an FP64 unsplit step at each height, measured on a GB300: a developed sea, and one
+# mostly at rest
+HEIGHTS = (8, 12, 16, 24, 32, 48, 64, 96, 128)
+MEASURED = [
+    ((300, 300), (471, 618, 791, 1132, 1470, 2156, 2840, 4207, 5567)),
+    ((771, 602), (1556, 1661, 1447, 1618, 1569, 2305, 2852, 4219, 5575)),
+    ((1024, 1024), (3051, 3165, 2800, 3616, 2727, 3100, 3037, 4493, 5588)),
+    ((1213, 1531), (5039, 4974, 5076, 5409, 5284, 5992, 5288, 6058, 5959)),
+    ((1700, 1700), (7589, 7476, 6952, 7804, 7875, 7789, 9665, 7844, 8036)),
+    ((2000, 2000), (10597, 10141, 9699, 9985, 10358, 10512, 10295, 13643, 10398)),
+    ((2400, 2400), (14993, 14291, 13689, 13887, 13076, 13674, 15179, 15052, 18085)),
+    ((2900, 2900), (21891, 20869, 20077, 19896, 19870, 19404, 20397, 22740, 20289)),
+    ((4096, 1000), (10577, 10270, 9978, 9930, 10403, 11401, 10149, 13599, 10388)),
+    ((300, 2900), (2341, 2228, 2505, 2086, 2115, 3052, 3037, 4460, 5588)),
+    ((2900, 300), (2332, 2214, 2786, 2634, 2723, 3092, 3021, 4483, 5574)),
+    ((2000, 2000), (12430, 11914, 11422, 11846, 12450, 13315, 12326, 16152, 12440)),
+    ((2400, 2400), (17552, 16778, 16219, 16476, 15493, 17341, 18087, 18326, 22929)),
+    ((4096, 1000), (12403, 12171, 11790, 11786, 12367, 13619, 12093, 14897, 11954)),
+]
+
+
+@pytest.mark.parametrize("size,us", MEASURED)
+def test_fp64_unsplit_heights_against_measurement(lib, size, us):
+    """Never slower than the one height of 128 rows that stood before the rules (2%: what
+    runs differ by), and within 15% of the best height."""
+    t = dict(zip(HEIGHTS, us))[_rows(lib, [size], 64, 0, 1)[0]]
+    assert t <= 1.02 * us[-1] and t <= 1.15 * min(us)
 
 
 def test_a_patch_cut_into_strips_is_one_patch(lib):
