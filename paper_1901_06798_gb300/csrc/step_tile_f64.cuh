@@ -32,6 +32,7 @@
 // of its two cells), the cell update divides by kap_j, and the mass gets the term
 // (ced_{j+1} - ced_j) hv_j of the varying edge length.
 #pragma once
+#include <type_traits>
 #include "step_kernel.cuh"
 #include "tile_rules.h"
 
@@ -206,8 +207,9 @@ __device__ __forceinline__ void limit_any(const Wave<double> &r, const double (&
     if (r.wall == 1) { am[0] = 0.0; am[1] = 0.0; am[2] = 0.0; }
 }
 
-__device__ __forceinline__ double shfl_up1(double v) { return __shfl_up_sync(0xffffffffu, v, 1); }      // lane 0: its own
-__device__ __forceinline__ double shfl_down1(double v) { return __shfl_down_sync(0xffffffffu, v, 1); }  // lane 31: its own
+// the neighbour's value among GW lanes of a row; its first or last lane: its own
+template <int GW> __device__ __forceinline__ double shfl_up1(double v) { return __shfl_up_sync(0xffffffffu, v, 1, GW); }
+template <int GW> __device__ __forceinline__ double shfl_down1(double v) { return __shfl_down_sync(0xffffffffu, v, 1, GW); }
 
 // postprocess(); false where h is not a finite number (or absurd), which is left as it is
 __device__ __forceinline__ bool post(double &h, double &qn, double &qt, long long tol)
@@ -267,12 +269,18 @@ template <int NW, bool GEO> __device__ __forceinline__ void tile64_item(const St
     const double *cedP = GEO ? a.ced + (P.j0 + 2) : nullptr;   // relative length of the y-edge below it at cedP[j]
     double smx = 0.0, smy = 0.0, deep_x = 0.0, deep_y = 0.0;   // largest speeds; deepest resting cells
 
-    // ---- x sweep, a row per warp, two adjacent columns per lane and their left edges
-    {
-        const int c0 = 2 * lane;
+    // ---- x sweep, two adjacent columns per lane and their left edges: a row per warp, or
+    // two where a row fits half of one.  (Patches of 16 columns, 3600 of them: 2958 us a
+    // step with a row per warp whatever its width, 1970 us; 28 columns 1627 and 1046.  The
+    // width fixed at compile time: with it in a register wide rows lose 0.5%.)
+    auto sweep_x = [&](auto width) {
+        constexpr int GW = decltype(width)::value, RW = 32 / GW;   // lanes of a row, rows of a warp
+        const int c0 = 2 * (lane & (GW - 1));
         const bool lim[2] = {c0 >= 2 && c0 <= w + 2, c0 + 1 >= 2 && c0 + 1 <= w + 2};   // edges of updated columns
-        const bool out[2] = {c0 >= 2 && c0 < w + 2, c0 + 1 >= 2 && c0 + 1 < w + 2};     // updated columns
-        for (int k = warp; k < nrows; k += NW) {
+        for (int kw = warp * RW; kw < nrows; kw += NW * RW) {
+            const int k = RW == 1 ? kw : min(kw + lane / GW, nrows - 1);
+            const bool live = RW == 1 || kw + lane / GW < nrows;   // (past the last row: its values, unused)
+            const bool out[2] = {live && c0 >= 2 && c0 < w + 2, live && c0 + 1 >= 2 && c0 + 1 < w + 2};   // updated columns
             double *row = tile64 + k * kRow + c0;
             CellD z[2], L;
 #pragma unroll
@@ -281,12 +289,12 @@ template <int NW, bool GEO> __device__ __forceinline__ void tile64_item(const St
                 z[q].e = z[q].z.h + z[q].z.B;
             }
             const int j = y0 - 2 + k;
-            const bool rowint = j >= 0 && j < P.ny;
+            const bool rowint = live && j >= 0 && j < P.ny;
             const double kr = GEO ? kapP[j] : 1.0;
             const double dtdx = GEO ? dt / (kr * a.dx) : dtdx0;
             const bool wet = z[0].z.wet && z[1].z.wet;
-            L.e = shfl_up1(z[1].e);
-            L.z.h = shfl_up1(z[1].z.h);
+            L.e = shfl_up1<GW>(z[1].e);
+            L.z.h = shfl_up1<GW>(z[1].z.h);
             const bool flat = wet && bits(L.e) == bits(z[0].e) && bits(z[0].e) == bits(z[1].e) && still(z[0]) && still(z[1]);
             if (__all_sync(ALL, flat)) {
                 if (rowint) {
@@ -311,9 +319,9 @@ template <int NW, bool GEO> __device__ __forceinline__ void tile64_item(const St
             derive(z[0], g);
             derive(z[1], g);
             L.z.q0 = L.z.h; L.z.wet = bits(L.z.h) >= tol;
-            L.z.hn = shfl_up1(z[1].z.hn); L.z.ht = shfl_up1(z[1].z.ht); L.z.B = shfl_up1(z[1].z.B);
-            L.z.u = shfl_up1(z[1].z.u); L.z.v = shfl_up1(z[1].z.v); L.z.c = shfl_up1(z[1].z.c); L.z.sq = shfl_up1(z[1].z.sq);
-            L.su = shfl_up1(z[1].su); L.um = shfl_up1(z[1].um); L.pn = shfl_up1(z[1].pn); L.pt = shfl_up1(z[1].pt);
+            L.z.hn = shfl_up1<GW>(z[1].z.hn); L.z.ht = shfl_up1<GW>(z[1].z.ht); L.z.B = shfl_up1<GW>(z[1].z.B);
+            L.z.u = shfl_up1<GW>(z[1].z.u); L.z.v = shfl_up1<GW>(z[1].z.v); L.z.c = shfl_up1<GW>(z[1].z.c); L.z.sq = shfl_up1<GW>(z[1].z.sq);
+            L.su = shfl_up1<GW>(z[1].su); L.um = shfl_up1<GW>(z[1].um); L.pn = shfl_up1<GW>(z[1].pn); L.pt = shfl_up1<GW>(z[1].pt);
             Wave<double> e[2];
             double am[2][3], ap[2][3], F[2][3];
             // (a row with a dry cell goes to the general solver at once)
@@ -322,8 +330,8 @@ template <int NW, bool GEO> __device__ __forceinline__ void tile64_item(const St
             if (__all_sync(ALL, oc)) {
                 double rt[3], lt[3];
 #pragma unroll
-                for (int m = 0; m < 3; m++) { rt[m] = shfl_down1(e[0].Z[0][m]); lt[m] = shfl_up1(e[1].Z[2][m]); }
-                const double tl = shfl_up1(e[1].Z[1][2]), tr = shfl_down1(e[0].Z[1][2]);
+                for (int m = 0; m < 3; m++) { rt[m] = shfl_down1<GW>(e[0].Z[0][m]); lt[m] = shfl_up1<GW>(e[1].Z[2][m]); }
+                const double tl = shfl_up1<GW>(e[1].Z[1][2]), tr = shfl_down1<GW>(e[0].Z[1][2]);
                 limit_ocean(e[0], e[1].Z[0], neg(e[0].s[1]) ? e[1].Z[1][2] : tl, lt, dtdx, am[0], ap[0], F[0]);
                 limit_ocean(e[1], rt, neg(e[1].s[1]) ? tr : e[0].Z[1][2], e[0].Z[2], dtdx, am[1], ap[1], F[1]);
             } else {
@@ -333,7 +341,7 @@ template <int NW, bool GEO> __device__ __forceinline__ void tile64_item(const St
                 }
                 double I00[3], I02[3], I10[3], I12[3];   // upwind waves of the two edges
                 auto pick = [&](int p, int m, double &x0, double &x1) {
-                    const double l = shfl_up1(e[1].Z[p][m]), r = shfl_down1(e[0].Z[p][m]);
+                    const double l = shfl_up1<GW>(e[1].Z[p][m]), r = shfl_down1<GW>(e[0].Z[p][m]);
                     x0 = neg(e[0].s[p]) ? e[1].Z[p][m] : l;
                     x1 = neg(e[1].s[p]) ? r : e[0].Z[p][m];
                 };
@@ -354,7 +362,7 @@ template <int NW, bool GEO> __device__ __forceinline__ void tile64_item(const St
             }
             double amr[3], Fr[3];   // of the right lane's first edge
 #pragma unroll
-            for (int m = 0; m < 3; m++) { amr[m] = shfl_down1(am[0][m]); Fr[m] = shfl_down1(F[0][m]); }
+            for (int m = 0; m < 3; m++) { amr[m] = shfl_down1<GW>(am[0][m]); Fr[m] = shfl_down1<GW>(F[0][m]); }
 #pragma unroll
             for (int q = 0; q < 2; q++) {
                 double qs[3] = {z[q].z.q0, z[q].z.hn, z[q].z.ht};
@@ -367,7 +375,9 @@ template <int NW, bool GEO> __device__ __forceinline__ void tile64_item(const St
                 if (out[q]) { row[q] = qs[0]; row[kRing + q] = qs[1]; row[2 * kRing + q] = qs[2]; }
             }
         }
-    }
+    };
+    if (w <= 28) sweep_x(std::integral_constant<int, 16>());
+    else sweep_x(std::integral_constant<int, 32>());
     __syncthreads();
 
     // ---- y sweep: a warp takes 32 columns and a segment of rows, one column per
