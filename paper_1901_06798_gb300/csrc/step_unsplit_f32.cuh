@@ -18,6 +18,7 @@
 // terms are read from registers instead of a three-row shared ring.
 #pragma once
 #include "step_unsplit.cuh"
+#include "tile_rules.h"
 
 namespace tsu {
 
@@ -349,6 +350,10 @@ int launch_unsplit_f32_nt(const StepArgs &a, int n_items, cudaStream_t st)
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         if (e != cudaSuccess) return (int)e;
         configured = true;
+    }
+    if (a.gate == nullptr && !launch_ahead(n_items, kSMs * (512 / NT))) {
+        step_unsplit_f32_kernel<NT, RING><<<n_items, NT, bytes, st>>>(a);
+        return (int)cudaGetLastError();
     }
     return launch_chained(step_unsplit_f32_kernel<NT, RING>, n_items, NT, bytes, st, a);
 }

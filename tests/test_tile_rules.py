@@ -39,6 +39,7 @@ extern "C" long shapes(int split, int f64, int *out)   // (threads, rows) pairs
     return n;
 }
 extern "C" long reported(int seg_rows, int most) { return tsu::reported_rows(seg_rows, most); }
+extern "C" long ahead(int items, int slots) { return tsu::launch_ahead(items, slots); }
 extern "C" long cut(int ny, int cap) { return tsu::tile_cut(ny, cap); }
 """
 
@@ -57,7 +58,7 @@ def lib(tmp_path_factory):
     subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(d / "h.cpp"), "-o", str(d / "h.so")],
                    check=True)
     L = ctypes.CDLL(str(d / "h.so"))
-    L.rows.restype = L.cut.restype = L.item.restype = L.shapes.restype = L.reported.restype = ctypes.c_long
+    L.rows.restype = L.cut.restype = L.item.restype = L.shapes.restype = L.reported.restype = L.ahead.restype = ctypes.c_long
     return L
 
 
@@ -139,6 +140,18 @@ def test_fp64_unsplit_heights_against_measurement(lib, size, us):
     runs differ by), and within 15% of the best height."""
     t = dict(zip(HEIGHTS, us))[_rows(lib, [size], 64, 0, 1)[0]]
     assert t <= 1.02 * us[-1] and t <= 1.15 * min(us)
+
+
+def test_waves_that_leave_slots_free_are_not_launched_ahead(lib):
+    """Measured with 608 slots (us a step, ahead of the predecessor's end and after it): a
+    launch that is slower ahead by more than 3% is not made so, and no other costs more than
+    3%.  The last line, half a wave of 64-thread CTAs, has 1216 slots."""
+    for items, slots, ahead, after in ((40, 608, 36.5, 36.5), (114, 608, 36.9, 37.2), (200, 608, 47.4, 45.5),
+                                       (288, 608, 118.7, 96.2), (320, 608, 44.1, 41.5), (416, 608, 165.6, 148.8),
+                                       (480, 608, 113.4, 115.4), (528, 608, 64.0, 58.8), (576, 608, 67.9, 70.2),
+                                       (904, 608, 57.0, 58.3), (576, 1216, 117.2, 95.6)):
+        t = ahead if lib.ahead(items, slots) else after
+        assert t <= 1.03 * min(ahead, after), items
 
 
 def test_a_patch_cut_into_strips_is_one_patch(lib):
