@@ -134,24 +134,31 @@ inline int unsplit_rows_f32p(const HeightStrips *s, int m, int threads)
 }
 
 // Unsplit update, FP64: the same segments.  Eight warps fit on an SM (shared memory); in
-// units of two warps, a row of one, two or three alone takes 2.1, 2.25 and 3.1 times what
+// units of two warps, a row of one, two or three alone takes 2.1, 2.3 and 3.3 times what
 // it takes of the full four, where the FP64 pipe is busy.  Beyond that the SMs take
-// segments as they finish: the work shared out, and the end of the last ones (1.3).
-// Both sides (us a step, developed sea, heights 16 / 32 / 64 / 128, then the rule's):
-// 771 x 602 1447 / 1569 / 2852 / 5575 (16), 1024^2 2800 / 2727 / 3037 / 5588 (32), 2000^2
-// 9699 / 10358 / 10295 / 10398 (128), 2400^2 13689 / 13076 / 15179 / 18085 (32), 4096 x
-// 1000 9978 / 10403 / 10149 / 10388 (128).  Counting whole segments an SM, whatever the
-// number in flight, took 48 rows for the last two: 13674 and 11401.
+// segments as they finish: the rows shared out, and the end of the last segments (1.7).
+// Both sides (us a step, developed sea, heights 8 / 16 / 32 / 64 / 128, then the rule's):
+// 771 x 602 1556 / 1447 / 1569 / 2852 / 5575 (16), 1024^2 3051 / 2800 / 2727 / 3037 / 5588
+// (32), 2000^2 10597 / 9699 / 10358 / 10295 / 10398 (16), 4096 x 1000 10577 / 9978 / 10403 /
+// 10149 / 10388 (16); 1000 patches of 24^2 2771 / 3019, 2965 in one piece (8), 1600 of
+// 60^2 15224 / 14053 / 14207, 14193 in one piece (16).  Counting whole segments an SM,
+// whatever the number in flight, took 48 rows for 4096 x 1000: 11401.
 inline int unsplit_rows_f64(const HeightStrips *s, int m, int threads)
 {
     static const int cand[] = {8, 12, 16, 24, 32, 48, 64, 96, 128};
-    static const double alone[] = {0.0, 2.1, 2.25, 3.1, 4.0};
+    static const double alone[] = {0.0, 2.1, 2.3, 3.3, 4.2};
     const double unit = threads / 64.0;
+    double rows = 0.0;
+    int top = 0;
+    for (int k = 0; k < m; k++) {
+        rows += s[k].strips * s[k].ny;
+        top = std::max(top, s[k].ny);
+    }
     int best = 64;
     double bc = 1e300;
     for (int R : cand) {
-        const double per = tile_count(s, m, R) / kSMs * unit, in_flight = std::ceil(per / unit - 1e-9) * unit;
-        const double c = (R + 2) * (in_flight <= 4.0 ? alone[(int)in_flight] : per + 1.3);
+        const double items = tile_count(s, m, R), in_flight = std::ceil(items / kSMs - 1e-9) * unit, one = std::min(R, top) + 1.0;
+        const double c = in_flight <= 4.0 ? one * alone[(int)in_flight] : (rows + items) / kSMs * unit + 1.7 * one;
         if (c < bc) { bc = c; best = R; }
     }
     return best;

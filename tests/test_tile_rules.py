@@ -78,8 +78,9 @@ def _restated(patches, threads, split, f64):
         if split and f64:
             return math.ceil(per) * (2.0 * (R + 4) + 4.0 * (R // 2 + 3)) * (1.75 if per <= 1 else 1.2 if per <= 2 else 1.0)
         if f64:
-            n = math.ceil(per - 1e-9) * threads / 64
-            return (R + 2) * ((0.0, 2.1, 2.25, 3.1, 4.0)[int(n)] if n <= 4 else per * threads / 64 + 1.3)
+            n, one = math.ceil(per - 1e-9) * threads / 64, min(R, max(y for _, y in patches)) + 1.0
+            rows = sum(-(-x // W) * y for x, y in patches) / 152
+            return one * (0.0, 2.1, 2.3, 3.3, 4.2)[int(n)] if n <= 4 else (rows + per) * threads / 64 + 1.7 * one
         one, share = (R + 16.0, 0.15) if split else (R + 6.0, 0.4)
         occ = 512 // threads
         if split:
@@ -132,6 +133,19 @@ MEASURED = [
     ((2400, 2400), (17552, 16778, 16219, 16476, 15493, 17341, 18087, 18326, 22929)),
     ((4096, 1000), (12403, 12171, 11790, 11786, 12367, 13619, 12093, 14897, 11954)),
 ]
+# the same for levels of n patches of side^2 cells; the last time: in one piece
+MEASURED_PATCHES = [
+    ((1000, 24), (2771, 2991, 3019, 2965)),
+    ((300, 24), (1105, 828, 1047, 1384)),
+    ((256, 64), (5157, 5089, 5099, 5298, 5444, 5965, 6190)),
+    ((128, 64), (2894, 2906, 2979, 3110, 3181, 4650, 3599)),
+    ((900, 16), (1365, 1697, 1621)),
+    ((256, 60), (2802, 2788, 2510, 2827, 2736, 4015, 2866)),
+    ((625, 60), (6158, 5968, 5880, 5978, 6428, 6660, 7492)),
+    ((1600, 60), (15224, 14503, 14053, 13941, 14207, 14275, 14193)),
+    ((625, 40), (4351, 4179, 4089, 4086, 4644, 5962, 5962)),
+    ((1225, 40), (7999, 7693, 7517, 7478, 7844, 8246, 7947)),
+]
 
 
 @pytest.mark.parametrize("size,us", MEASURED)
@@ -139,6 +153,13 @@ def test_fp64_unsplit_heights_against_measurement(lib, size, us):
     """Never slower than the one height of 128 rows that stood before the rules (2%: what
     runs differ by), and within 15% of the best height."""
     t = dict(zip(HEIGHTS, us))[_rows(lib, [size], 64, 0, 1)[0]]
+    assert t <= 1.02 * us[-1] and t <= 1.15 * min(us)
+
+
+@pytest.mark.parametrize("level,us", MEASURED_PATCHES)
+def test_fp64_unsplit_heights_of_patches_against_measurement(lib, level, us):
+    n, side = level
+    t = dict(zip(HEIGHTS, us)).get(_rows(lib, [(side, side)] * n, 64, 0, 1)[0], us[-1])
     assert t <= 1.02 * us[-1] and t <= 1.15 * min(us)
 
 
