@@ -166,13 +166,13 @@ inline int unsplit_rows_f64(const HeightStrips *s, int m, int threads)
 
 // FP32 unsplit update: whether a launch of `items` CTAs is made ahead of its predecessor's
 // end (chain.cuh).  Placed around CTAs that are still there, those of a wave that leaves
-// slots free pile up on some SMs; a wave that fills them, or leaves most SMs one CTA at
-// most, has no choice.
+// slots free pile up on some SMs; a wave that fills them has no choice, and one of half as
+// many CTAs as SMs finds room beside the boundaries' CTAs.
 // Both sides (us a step, ahead / after): 1024^2 with 128 x 32 work items (288 CTAs of 608
 // slots) 118.7 / 96.2 and with the rule's 16 rows (576) 67.9 / 70.2; 1500^2 (416) 165.6 /
 // 148.8, 700^2 (528) 64.0 / 58.8, 512^2 (320) 44.1 / 41.5, 1213 x 1531 (480) 113.4 / 115.4;
-// 300^2 (114) 36.9 / 37.2; 900^2 (904) 57.0 / 58.3.
-inline bool launch_ahead(int items, int slots) { return items <= kSMs || 10LL * items >= 9LL * slots; }
+// 1024^2 with 64 rows (144) 177 / 170; 200^2 (50) 36.6 / 37.0; 900^2 (904) 57.0 / 58.3.
+inline bool launch_ahead(int items, int slots) { return 2 * items <= kSMs || 10LL * items >= 9LL * slots; }
 
 // The most rows of a work item for n patches of nx[k] x ny[k] cells advanced together,
 // in strips of W columns by CTAs of `threads`
