@@ -263,8 +263,9 @@ int tsu_get_stats(tsu_ctx *ctx, int scenario, tsu_stats *out);
  * into row segments).  step_threads is 64, 128 or 256, or also 32 for the
  * split FP32 update.  A CTA updates a tile of 60 columns in the split updates
  * (of at most 124 rows in FP32 and 104 in FP64: what shared memory holds) and a
- * strip of step_threads - 4 columns in the unsplit ones.  0 restores the
- * defaults.  Results do not depend on either.  Returns TSU_ERR_ARG for any
+ * strip of step_threads - 4 columns in the unsplit ones.  (A tall tile leaves
+ * an SM room for fewer CTAs: the FP64 split update is fastest at 32 rows and
+ * less.)  0 restores the defaults.  Results do not depend on either.  Returns TSU_ERR_ARG for any
  * other value. */
 int tsu_set_tuning(tsu_ctx *ctx, int step_threads, int seg_rows);
 
@@ -387,12 +388,17 @@ int tsu_time_level1_steps(tsu_ctx *ctx, int warmup, int n, double *kernel_ms_out
  * 16->16 with biases: 736 + 2,320 + 2,320; the 1x1 head 16->1: 17). */
 int tsu_cnn_num_params(void);
 
-/* Logits (n, h, w) of host inputs x (n, 5, h, w); fp16 != 0: FP16 activations
+/* The three calls below take their device buffers from a memory pool of the
+ * library's, one per device, which keeps up to 64 MiB between calls until the
+ * process exits; a call that needs more allocates the rest and gives it back.
+ *
+ * Logits (n, h, w) of host inputs x (n, 5, h, w); fp16 != 0: FP16 activations
  * and weights with FP32 accumulation (the inference path), else FP32. */
 int tsu_cnn_forward(const float *theta, const float *x, int n, int h, int w, int fp16, float *logits);
 
 /* Mean binary cross-entropy with logits over the cells where m = 1 and its
- * gradient with respect to theta (host buffers; targets t in {0, 1}). */
+ * gradient with respect to theta (host buffers; targets t in {0, 1}).  Sums are
+ * taken in a fixed order: the same inputs give the same bits. */
 int tsu_cnn_loss_grad(const float *theta, const float *x, const float *t, const float *m, int n, int h, int w,
                       double *loss, float *grad);
 

@@ -356,7 +356,7 @@ class Tsunami:
         self._check(self._L.tsu_set_tuning(self._h, step_threads, seg_rows), "tsu_set_tuning")
 
     def set_bulk_copies(self, enable: int, polls: int = 1 << 22):
-        """x-sweep rows by bulk copies on mbarriers, each wait at most `polls` polls (0: give up at once)."""
+        """Tile rows by bulk copies on mbarriers, each wait at most `polls` polls (0: give up at once)."""
         self._check(self._L.tsu_set_bulk_copies(self._h, enable, C.c_longlong(polls)), "tsu_set_bulk_copies")
 
     def autotune(self, reps: int = 3):

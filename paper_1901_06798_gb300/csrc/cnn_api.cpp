@@ -21,7 +21,8 @@ namespace {
 // the process: cudaMalloc and cudaFree take tens of microseconds each and wait for
 // the device, and the calls used up to twelve of both.  The pool (one per device,
 // stream-ordered, safe from several threads) keeps at most kPoolKeep bytes between
-// calls; what is above that goes back to the device at the next synchronisation.
+// calls; what is above that goes back to the device at the next synchronisation, so a
+// call that needs more maps the rest anew each time.
 constexpr unsigned long long kPoolKeep = 64ull << 20;
 constexpr int kMaxDevices = 64;
 

@@ -17,13 +17,14 @@
 // so four CTAs of four warps fit on an SM with tiles of up to 48 rows (12 warps of
 // 168 registers: 143.1 against 141.3 us on 3000^2 developed cells).
 //
-// What bounds it is the issue of instructions: 62% of the issue slots on a developed
-// sea (346 warp instructions for 32 cells, one in six a register move that pairs
-// values of two lanes), DRAM under a third of its rate.  Two kernels with Q* in DRAM
-// between them, one-warp strips in x and row pairs in y, took 309 us for a 4096^2
-// step mostly at rest and 294 us for 2050 x 1537 developed cells in the caller's
-// memory; with this kernel the steps take 221 and 93 us.  The y march over pairs of
-// rows instead of pairs of columns: 237 against 149 us for 3000^2 cells.
+// What bounds it is the issue of instructions: 61% of the issue slots on a developed
+// sea (334 warp instructions for 32 cells), DRAM under a third of its rate.  Two
+// kernels with Q* in DRAM between them, one-warp strips in x and row pairs in y, took
+// 309 us for a step of the 4096^2 shelf some hundred steps after its uplift and 294 us
+// for 2050 x 1537 developed cells in the caller's memory; with this kernel the steps
+// take 222 and 94 us (the shelf's first 20 steps, most of the sea at rest: 174 us each).
+// The y march over pairs of rows instead of pairs of columns: 237 against 149 us for
+// 3000^2 cells.
 //
 // A row of a warp takes the cheapest of four forms, by warp votes; all give the
 // bits of the general one:

@@ -98,8 +98,9 @@ inline int tile_rows_f32p(const HeightStrips *s, int m, int threads)
 // three or more, which is what fits.
 // Both sides (us, developed sea): 771 x 602 543 with the rule's height, 941 with 16 rows,
 // 687 with 12; 512^2 325 and 380 with 12; 2048^2 3972 and 4124 with 24.  256 threads in place
-// of 128: 350 at 512^2, 595 at 771 x 602, but 115 against 127 at 200^2 and 241 against 333 where
-// most of 512^2 is at rest; 64 threads: 398, 568, 191, 467.
+// of 128: 350 at 512^2, 595 at 771 x 602, but 115 against 127 at 200^2 (before narrow strips
+// took two rows of a warp) and 241 against 333 where most of 512^2 is at rest; 64 threads:
+// 398, 568, 191, 467.
 inline int tile_rows_f64(const HeightStrips *s, int m)
 {
     int best = 32;

@@ -1192,7 +1192,7 @@ struct tsu_ctx {
         StepArgs a = step_args(l);
         TailArgs &t_ = a.tail;
         t_.cv = ctrl();
-        // (a finer level saves one launch by it, level 1 two)
+        // (finer levels up to a quarter: see kTailMaxCtas)
         const bool counted = (int)L.items.size() <= (l == 0 ? kTailMaxCtas : kTailMaxCtas / 4);
         t_.count = counted ? tail_count.p : nullptr;
         t_.any_retake = retake_on ? any_retake.p : nullptr;
