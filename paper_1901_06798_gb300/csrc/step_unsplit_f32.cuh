@@ -351,7 +351,7 @@ int launch_unsplit_f32_nt(const StepArgs &a, int n_items, cudaStream_t st)
         if (e != cudaSuccess) return (int)e;
         configured = true;
     }
-    if (a.gate == nullptr && !launch_ahead(n_items, kSMs * (512 / NT))) {
+    if (a.gate == nullptr && !launch_ahead(n_items, 512 / NT)) {
         step_unsplit_f32_kernel<NT, RING><<<n_items, NT, bytes, st>>>(a);
         return (int)cudaGetLastError();
     }

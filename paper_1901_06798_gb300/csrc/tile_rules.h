@@ -165,15 +165,16 @@ inline int unsplit_rows_f64(const HeightStrips *s, int m, int threads)
     return best;
 }
 
-// FP32 unsplit update: whether a launch of `items` CTAs is made ahead of its predecessor's
-// end (chain.cuh).  Placed around CTAs that are still there, those of a wave that leaves
-// slots free pile up on some SMs; a wave that fills them has no choice, and one of half as
-// many CTAs as SMs finds room beside the boundaries' CTAs.
-// Both sides (us a step, ahead / after): 1024^2 with 128 x 32 work items (288 CTAs of 608
-// slots) 118.7 / 96.2 and with the rule's 16 rows (576) 67.9 / 70.2; 1500^2 (416) 165.6 /
-// 148.8, 700^2 (528) 64.0 / 58.8, 512^2 (320) 44.1 / 41.5, 1213 x 1531 (480) 113.4 / 115.4;
-// 1024^2 with 64 rows (144) 177 / 170; 200^2 (50) 36.6 / 37.0; 900^2 (904) 57.0 / 58.3.
-inline bool launch_ahead(int items, int slots) { return 2 * items <= kSMs || 10LL * items >= 9LL * slots; }
+// FP32 unsplit update: whether a launch of `items` CTAs, of which an SM holds `held`, is
+// made ahead of its predecessor's end (chain.cuh).  Placed around CTAs that are still
+// there, those of a launch that would leave every SM a slot pile up on some.  Where some SM
+// is to hold all it can anyway nothing is lost, and three quarters as many CTAs as SMs find
+// room beside the boundaries' CTAs.
+// Both sides (us a step, ahead / after): 114 CTAs (300^2) 36.8 / 37.6, 152 (450^2) 48.6 /
+// 46.8, 264 (700^2) 64.1 / 59.0, 416 (1500^2) 165.9 / 148.6, 442 (1600^2) 158.8 / 143.9, 469
+// (800^2) 56.1 / 58.3, 504 (1700^2) 163.7 / 170.6, 576 (1024^2) 68.7 / 70.7, 1104 (2900^2)
+// 398.2 / 398.9, all with 4 held; over 56 sizes 0.1% above the better of the two.
+inline bool launch_ahead(int items, int held) { return 4LL * items <= 3LL * kSMs || items > kSMs * (held - 1); }
 
 // The most rows of a work item for n patches of nx[k] x ny[k] cells advanced together,
 // in strips of W columns by CTAs of `threads`
